@@ -372,7 +372,7 @@ FastGeom fast_geom(const Geom& g) {
 
 inline bool fp32(const Ctx& c) { return c.p.precision == DG_PREC_FP32MIX; }
 
-// the Powell kernels exist for degrees 1 and 2 (a degree-3 context never
+// FP32: the Powell kernels exist for degrees 1 and 2 (a degree-3 context never
 // selects them: its tables are not built)
 template <typename T, int DEG>
 void face_pow_fast(const FastAll<T, DEG>& ft, const FastGeom& fg, const T* w, T* F, double eps, cudaStream_t st) {
@@ -401,6 +401,18 @@ bool launch_cell_fast(Ctx& c, const FastAll<T, DEG>& ft, const FastGeom& fg, con
   return false;
 }
 
+// FP64, uniform 3D meshes: the sum-factorised face and cell kernels
+template <int DEG, bool GLM>
+void sf_pass(Ctx& c, const FastGeom& fg, const void* w, void* out, const void* w0, double ca, double cb, int combine,
+             cudaStream_t st) {
+  c.prof.begin(0, st);
+  launch_sf_face<DEG, GLM>(fg, (const double*)w, c.face_buf, c.sc, c.p.eps_hlld, st);
+  c.prof.end(0, st);
+  c.prof.begin(1, st);
+  launch_sf_cell<DEG, GLM>(fg, (const double*)w, c.face_buf, (double*)out, (const double*)w0, ca, cb, combine, c.sc,
+                           st);
+  c.prof.end(1, st);
+}
 
 }  // namespace
 
@@ -723,13 +735,15 @@ int dg_mhd_init(const dg_mesh_desc* mesh, int degree, int divB_scheme, double ga
       if (c.fast_tabs) c.fast = 20 + degree;
     }
     if (c.fast && !fast_pow_ok(c)) free_fast_tabs(c);
+    if ((c.fast == 21 && sf_ldf_to_constant<1>(((const FastAll<double, 1>*)c.fast_tabs)->pow)) ||
+        (c.fast == 22 && sf_ldf_to_constant<2>(((const FastAll<double, 2>*)c.fast_tabs)->pow)))
+      free_fast_tabs(c);
   }
   // specialised GLM kernels for uniform 3D meshes
   if (g.glm && g.D == 3 && prm.generic_kernels != 1 && !c.amr.on) {
     if (fp32(c)) {
       if (degree == 1) c.fast_tabs = make_fast_tabs<float, 1>(h, g, *c.hb);
       if (degree == 2) c.fast_tabs = make_fast_tabs<float, 2>(h, g, *c.hb);
-      // degree 3: FP32 only (the FP64 tables exceed the constant bank)
       if (degree == 3) c.fast_tabs = make_fast_tabs<float, 3>(h, g, *c.hb);
       if (c.fast_tabs) c.fast = 10 + degree;
       // degree 2, on request: the cell update's contractions on the tensor
@@ -745,10 +759,8 @@ int dg_mhd_init(const dg_mesh_desc* mesh, int degree, int divB_scheme, double ga
           return DG_E_CUDA;
         }
       }
-    } else {
-      if (degree == 1) c.fast_tabs = make_fast_tabs<double, 1>(h, g, *c.hb);
-      if (degree == 2) c.fast_tabs = make_fast_tabs<double, 2>(h, g, *c.hb);
-      if (c.fast_tabs) c.fast = 20 + degree;
+    } else if (degree >= 1) {
+      c.fast = 20 + degree;  // the sum-factorised kernels need no tables
     }
   }
   // initial GLM speeds: fixed c_h if given (damping from c_r), else set by dt
@@ -892,8 +904,15 @@ int operator_pass(Ctx& c, const void* w, const double* wmean, void* out, double*
       FASTCASE(11, float, 1, c.face_buf32)
       FASTCASE(12, float, 2, c.face_buf32)
       FASTCASE(13, float, 3, c.face_buf32)
-      FASTCASE(21, double, 1, c.face_buf)
-      FASTCASE(22, double, 2, c.face_buf)
+      case 21:
+        if (g.glm) sf_pass<1, true>(c, fg, w, out, w0, ca, cb, combine, st);
+        else sf_pass<1, false>(c, fg, w, out, w0, ca, cb, combine, st);
+        break;
+      case 22:
+        if (g.glm) sf_pass<2, true>(c, fg, w, out, w0, ca, cb, combine, st);
+        else sf_pass<2, false>(c, fg, w, out, w0, ca, cb, combine, st);
+        break;
+      case 23: sf_pass<3, true>(c, fg, w, out, w0, ca, cb, combine, st); break;
     }
 #undef FASTCASE
     return cudaGetLastError() == cudaSuccess ? DG_OK : DG_E_CUDA;

@@ -179,4 +179,16 @@ void launch_cell_glm(const FastAll<T, DEG>& tabs, const FastGeom& g, const T* w,
                      double ca, double cb, int combine, const DevScalars* sc, const double* wmean,
                      const double* w0mean, double* outmean, cudaStream_t st);
 
+
+// FP64 operator on uniform 3D meshes, sum-factorised (dg_sf_impl.cuh): GLM
+// degrees 1-3, Powell degrees 1-2. Face buffer: the 2D moments of total degree
+// <= d of the face fluxes, F[axis][moment][slot][cell] (9 slots GLM, 10 Powell).
+template <int DEG, bool GLM>
+void launch_sf_face(const FastGeom& g, const double* w, double* F, const DevScalars* sc, double eps, cudaStream_t st);
+template <int DEG, bool GLM>
+void launch_sf_cell(const FastGeom& g, const double* w, const double* F, double* out, const double* w0, double ca,
+                    double cb, int combine, const DevScalars* sc, cudaStream_t st);
+template <int DEG>
+int sf_ldf_to_constant(const PowTabs<double, DEG>& pt);
+
 }  // namespace dgmhd

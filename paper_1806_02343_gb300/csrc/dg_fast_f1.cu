@@ -2,4 +2,5 @@
 #define DG_FAST_T float
 #define DG_FAST_DEG 1
 #define DG_FAST_CONST 1
+#define DG_FAST_UNIFORM 1
 #include "dg_fast_impl.cuh"

@@ -1,7 +1,8 @@
 // Specialised kernels of the DG operator (included once per precision and
-// degree by the dg_fast_*.cu units) for the GLM scheme and for the Powell
-// scheme with the LDF basis on uniform 3D meshes (Sec. 3.5 eq. wdot;
-// Sec. 4.1.2 HLLD; Sec. 4.1.3 Powell; Sec. 4.1.5 GLM).
+// degree by the dg_fast_*.cu units; Sec. 3.5 eq. wdot; Sec. 4.1.2 HLLD; Sec.
+// 4.1.3 Powell; Sec. 4.1.5 GLM): the FP32 form of the GLM and Powell schemes on
+// uniform 3D meshes, and the Powell scheme on octrees in both precisions (the
+// FP64 operator of uniform meshes: dg_sf_impl.cuh).
 //
 // Same arithmetic as the generic kernels, organised for the hardware:
 // * basis tables are kernel parameters (constant bank), indexed with
@@ -14,7 +15,7 @@
 // * the volume flux of variable v is written as f_a = alpha v_a + beta B_a
 //   (+ gamma if a is the variable's own axis), with (alpha, beta, gamma) read
 //   from per-point shared memory -- one code path for all nine variables;
-// * k_face_glm evaluates the traces of the 32 cell pairs of a block with the
+// * k_face_glm3 evaluates the traces of the 32 cell pairs of a block with the
 //   same per-(side, variable) mapping, then one thread per face point runs
 //   HLLD and stores F* in a [axis][point][var][cell] buffer (cell fastest) that
 //   k_cell_glm reads coalesced.
@@ -245,18 +246,6 @@ __device__ __forceinline__ void face_axis(const FaceTabs<T, DEG>& tbp, const Fas
       for (int k = 0; k < 9; ++k) F[((int64_t)(A * QF + p) * 9) * S + c + (int64_t)k * S] = Fo[k];
     }
   }
-}
-
-template <typename T, int DEG, int A>
-__global__ void __launch_bounds__(NT, (sizeof(T) == 4 && DEG <= 2) ? 4 : 3) k_face_glm(const FaceTabs<T, DEG> tbp, const FastGeom g,
-                                                 const T* __restrict__ w, T* __restrict__ F,
-                                                 const DevScalars* __restrict__ sc, T eps) {
-  constexpr int NR = 9 * FastDims<DEG>::N;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  T* WL = reinterpret_cast<T*>(smraw);       // [NR][TC]
-  T* WR = WL + NR * TC;                      // [NR][TC]
-  T* TR = WR + NR * TC;                      // [2][QF][9][TC]
-  face_axis<T, DEG, A, true>(tbp, g, w, F, sc, eps, WL, WR, TR);
 }
 
 // All three axes in one pass: the block's own coefficients are read once and
@@ -1362,15 +1351,8 @@ void launch_face_glm(const FastAll<T, DEG>& tabs, const FastGeom& g, const T* w,
   const size_t sm = fast_face_smem<T, DEG>();
   static bool attr = false;
   if (!attr) {
-    set_smem_attr<T>((const void*)k_face_glm<T, DEG, 0>, sm);
-    set_smem_attr<T>((const void*)k_face_glm<T, DEG, 1>, sm);
-    set_smem_attr<T>((const void*)k_face_glm<T, DEG, 2>, sm);
-    attr = true;
-  }
-  static bool attr3 = false;
-  if (!attr3) {
     set_smem_attr<T>((const void*)k_face_glm3<T, DEG>, sm);
-    attr3 = true;
+    attr = true;
   }
   k_face_glm3<T, DEG><<<nb, NT, sm, st>>>(tabs.face[0], tabs.face[1], tabs.face[2], g, w, F, sc, (T)eps);
 }
@@ -1483,27 +1465,33 @@ int fast_to_constant(const FastAll<T, DEG>& tabs) {
   return 0;
 }
 
-#define INSTF(T, DEG)                                                                                         \
-  template void launch_face_glm<T, DEG>(const FastAll<T, DEG>&, const FastGeom&, const T*, T*,              \
-                                        const DevScalars*, double, cudaStream_t);                          \
-  template void launch_cell_glm<T, DEG>(const FastAll<T, DEG>&, const FastGeom&, const T*, const T*, T*,    \
-                                        const T*, double, double, int, const DevScalars*, const double*,    \
-                                        const double*, double*, cudaStream_t);          \
-  template int fast_to_constant<T, DEG>(const FastAll<T, DEG>&);
-// the Powell kernels for degrees 1 and 2
+// FP32: GLM and Powell on uniform meshes (FP64 runs those on the sum-factorised kernels, dg_sf_impl.cuh)
+#if DG_FAST_UNIFORM
+template void launch_face_glm<DG_FAST_T, DG_FAST_DEG>(const FastAll<DG_FAST_T, DG_FAST_DEG>&, const FastGeom&,
+                                                      const DG_FAST_T*, DG_FAST_T*, const DevScalars*, double,
+                                                      cudaStream_t);
+template void launch_cell_glm<DG_FAST_T, DG_FAST_DEG>(const FastAll<DG_FAST_T, DG_FAST_DEG>&, const FastGeom&,
+                                                      const DG_FAST_T*, const DG_FAST_T*, DG_FAST_T*,
+                                                      const DG_FAST_T*, double, double, int, const DevScalars*,
+                                                      const double*, const double*, double*, cudaStream_t);
+#if DG_FAST_DEG <= 2
+template void launch_face_pow<DG_FAST_T, DG_FAST_DEG>(const FastAll<DG_FAST_T, DG_FAST_DEG>&, const FastGeom&,
+                                                      const DG_FAST_T*, DG_FAST_T*, double, cudaStream_t);
+template void launch_cell_pow<DG_FAST_T, DG_FAST_DEG>(const FastAll<DG_FAST_T, DG_FAST_DEG>&, const FastGeom&,
+                                                      const DG_FAST_T*, const DG_FAST_T*, DG_FAST_T*,
+                                                      const DG_FAST_T*, double, double, int, const DevScalars*,
+                                                      const double*, const double*, double*, cudaStream_t);
+#endif
+#endif
+template int fast_to_constant<DG_FAST_T, DG_FAST_DEG>(const FastAll<DG_FAST_T, DG_FAST_DEG>&);
+// Powell, degrees 1 and 2: the timestep's face jumps and the octree kernels
 #define INSTP(T, DEG)                                                                                         \
-  template void launch_face_pow<T, DEG>(const FastAll<T, DEG>&, const FastGeom&, const T*, T*, double,        \
-                                        cudaStream_t);                                                        \
-  template void launch_cell_pow<T, DEG>(const FastAll<T, DEG>&, const FastGeom&, const T*, const T*, T*,    \
-                                        const T*, double, double, int, const DevScalars*, const double*,    \
-                                        const double*, double*, cudaStream_t);                              \
   template void launch_divb_face_pow<T, DEG>(const FastGeom&, const T*, T*, cudaStream_t);                    \
   template void launch_face_list_pow<T, DEG>(const OctPow<T>&, double, const T*, T*, double, cudaStream_t);   \
   template void launch_cell_list_pow<T, DEG>(const OctPow<T>&, double, const T*, const T*, T*, const T*, double, \
                                              double, int, const DevScalars*, const double*, const double*,      \
                                              double*, cudaStream_t);                                           \
   template void launch_divb_list_pow<T, DEG>(const OctPow<T>&, const T*, T*, cudaStream_t);
-INSTF(DG_FAST_T, DG_FAST_DEG)
 #if DG_FAST_DEG <= 2
 INSTP(DG_FAST_T, DG_FAST_DEG)
 #endif
