@@ -18,6 +18,7 @@
 #include "dg_cell_tc.cuh"
 #include "dg_fast.cuh"
 #include "dg_kernels.cuh"
+#include "dg_ldf.cuh"
 #include "dg_limit.cuh"
 #include "dg_mlp.cuh"
 
@@ -198,8 +199,8 @@ inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 // the LDF functions' components by quadrature (exact: every component is a
 // polynomial of total degree <= d), checked against the functions themselves;
 // ok = 0 when the basis lacks the structure the kernels rely on (three
-// constant functions, each along one axis, and no other function with a
-// non-zero mean). The same for every context of this degree.
+// constant functions, each along one axis, no other function with a non-zero
+// mean, no entry outside dg_ldf.cuh's pattern). The same for every context of this degree.
 // A[(j * 3 + c) * n + l]: the Legendre coefficients of component c of the 3D
 // LDF function j of degree <= deg, by quadrature with deg + 1 Gauss points
 // per axis (exact: the products are polynomials of degree <= 2 deg per
@@ -243,7 +244,7 @@ bool ldf_legendre_3d(int deg, std::vector<double>& A, int& ndiv, int& n) {
 template <typename T, int DEG>
 void build_pow_tabs(PowTabs<T, DEG>& pt) {
   using Dm = FastDims<DEG>;
-  constexpr int N = Dm::N, NDIV = PowDims<DEG>::NDIV, NP = PowDims<DEG>::NP;
+  constexpr int N = Dm::N, NDIV = PowDims<DEG>::NDIV;
   pt = PowTabs<T, DEG>();
   std::vector<double> A;
   int nd = 0, nm = 0;
@@ -260,6 +261,7 @@ void build_pow_tabs(PowTabs<T, DEG>& pt) {
       for (int l = 0; l < N; ++l) {
         if (j < 3 && l > 0 && a(j, cc, l) != 0.0) return;
         if (j >= 3 && l == 0 && a(j, cc, l) != 0.0) return;
+        if (a(j, cc, l) != 0.0 && !ldf_has<DEG>(j, cc, l)) return;
       }
   for (int j = 0; j < 3; ++j) {
     int nz = 0, at = -1;
@@ -272,12 +274,6 @@ void build_pow_tabs(PowTabs<T, DEG>& pt) {
   for (int cc = 0; cc < 3; ++cc)
     for (int j = 0; j < NDIV; ++j)
       for (int l = 0; l < N; ++l) pt.Af[cc][j][l] = (T)a(j, cc, l);
-  for (int k = 0; k < NP; ++k)
-    for (int e = 0; e < 2; ++e) {
-      const int j = 3 + 2 * k + e;
-      for (int cc = 0; cc < 3; ++cc)
-        for (int l = 0; l < N; ++l) pt.Ab[k][cc][l][e] = j < NDIV ? (T)a(j, cc, l) : T(0);
-    }
   for (int j = 0; j < NDIV; ++j) pt.minvL[j] = (T)(1.0 / L.ldf_mass[j]);
   for (int a2 = 0; a2 < 3; ++a2)
     for (int sd = 0; sd < 2; ++sd)

@@ -138,6 +138,7 @@ struct LimTabs {
   int deg1[3];
   int mdeg[64];
   int ldf_deg[64];
+  int ldf_lin[64];  // the LDF function has a linear part (a non-zero slope entry)
   double ldf_mean0[64 * 3];
   double ldf_slope[64 * 9];
   double ldf_pc[64 * 3];

@@ -85,12 +85,10 @@ struct CellTabs {
 template <int DEG>
 struct PowDims {
   static constexpr int NDIV = DEG == 1 ? 11 : DEG == 2 ? 26 : 50;  // Table A1, D = 3
-  static constexpr int NP = (NDIV - 3 + 1) / 2;                   // pairs of non-mean LDF rows
 };
 template <typename T, int DEG>
 struct PowTabs {
-  alignas(16) T Af[3][PowDims<DEG>::NDIV][FastDims<DEG>::N];      // forward: [cc][j][l]
-  alignas(16) T Ab[PowDims<DEG>::NP][3][FastDims<DEG>::N][2];     // back: rows 3+2k, 4+2k
+  alignas(16) T Af[3][PowDims<DEG>::NDIV][FastDims<DEG>::N];      // [cc][j][l]; only dg_ldf.cuh's pattern is non-zero
   alignas(16) T minvL[PowDims<DEG>::NDIV + 1];                    // 1 / LDF mass
   // normal component (axis a) of LDF function j at point p of face 2a + s
   alignas(16) T Ln[3][2][PowDims<DEG>::NDIV][FaceTabs<T, DEG>::QFP];

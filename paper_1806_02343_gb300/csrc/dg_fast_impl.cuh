@@ -25,6 +25,7 @@
 #include <utility>
 
 #include "dg_fast.cuh"
+#include "dg_ldf.cuh"
 
 #if !defined(DG_FAST_T) || !defined(DG_FAST_DEG) || !defined(DG_FAST_CONST)
 #error "include from a dg_fast_<precision><degree>.cu unit that defines DG_FAST_T, DG_FAST_DEG, DG_FAST_CONST"
@@ -519,19 +520,28 @@ __device__ __forceinline__ const PowTabs<T, DEG>& pow_tabs() {
 }
 
 // b[l] = sum_j Af[CC][j][l] X[j * TC]: Legendre coefficients of component CC
-// of B from the LDF coefficients staged at X (two modes per packed FMA)
+// of B from the LDF coefficients staged at X. Only the non-zero entries of the
+// map (dg_ldf.cuh: 10 to 14 of 260 per component at degree 2), in the order of
+// j: the sums are bitwise those of the dense map. The dense form kept the three
+// B warps of a block busy while the others waited at the barrier (128^3 Powell
+// blast, per stage: face pass 1.98 -> 1.41 ms, with the sparse back map cell pass
+// 3.20 -> 2.96 ms).
 template <typename T, int DEG, int CC>
 __device__ __forceinline__ void ldf_to_legendre(const T* X, T (&b)[FastDims<DEG>::N]) {
   constexpr int N = FastDims<DEG>::N, NDIV = PowDims<DEG>::NDIV;
   const PowTabs<T, DEG>& pt = pow_tabs<T, DEG>();
 #pragma unroll
   for (int l = 0; l < N; ++l) b[l] = T(0);
-#pragma unroll
-  for (int j = 0; j < NDIV; ++j) {
-    const T x = X[j * TC];
-#pragma unroll
-    for (int l = 0; l < N; l += 2) fma2(b[l], b[l + 1], x, x, pt.Af[CC][j][l], pt.Af[CC][j][l + 1]);
-  }
+  static_for<NDIV>([&](auto J) {
+    constexpr int j = decltype(J)::value;
+    if constexpr (ldf_has<DEG>(j, CC)) {
+      const T x = X[j * TC];
+      static_for<N>([&](auto L) {
+        constexpr int l = decltype(L)::value;
+        if constexpr (ldf_has<DEG>(j, CC, l)) b[l] = fma_rn(x, pt.Af[CC][j][l], b[l]);
+      });
+    }
+  });
 }
 
 template <typename T, int DEG>
@@ -814,7 +824,7 @@ __device__ __forceinline__ void pow_store(const T (&wl)[FastDims<DEG>::N], const
                                           const T* LS, T tm, double km, T* out, const T* w0, double ca, double cb,
                                           float ca32, float cb32, int cmode, const DevScalars* __restrict__ sc,
                                           const double* __restrict__ wmean, const double* w0mean, double* outmean) {
-  constexpr int N = FastDims<DEG>::N, NDIV = PowDims<DEG>::NDIV, NP = PowDims<DEG>::NP;
+  constexpr int N = FastDims<DEG>::N, NDIV = PowDims<DEG>::NDIV;
   const CellTabs<T, DEG>& tb = FastConst<T, DEG>::get().cell;
   const PowTabs<T, DEG>& pt = pow_tabs<T, DEG>();
   T* RL = PR;  // [3][N][TC]
@@ -868,29 +878,24 @@ __device__ __forceinline__ void pow_store(const T (&wl)[FastDims<DEG>::N], const
       }
     }
   } else {
-    // non-mean LDF rows j = 3 + 2k, 4 + 2k, pair k on component thread k mod 3
+    // non-mean LDF rows j >= 3, pairs (3 + 2k, 4 + 2k) on component thread k mod
+    // 3, from the non-zero entries of the map
     const int cc = v - 5;
-    static_for<NP>([&](auto K) {
-      constexpr int k = decltype(K)::value;
-      constexpr int j0 = 3 + 2 * k, j1 = j0 + 1;
-      if (k % 3 == cc) {
-        T R0 = T(0), R1 = T(0);
+    static_for<NDIV - 3>([&](auto J) {
+      constexpr int j = 3 + decltype(J)::value;
+      if ((j - 3) / 2 % 3 == cc) {
+        T R = T(0);
         static_for<3>([&](auto CCI) {
           constexpr int c2 = decltype(CCI)::value;
-#pragma unroll
-          for (int l = 1; l < N; ++l) {
-            const T x = RL[(c2 * N + l) * TC + f];
-            fma2(R0, R1, x, x, pt.Ab[k][c2][l][0], pt.Ab[k][c2][l][1]);
-          }
+          static_for<N>([&](auto L) {
+            constexpr int l = decltype(L)::value;
+            if constexpr (ldf_has<DEG>(j, c2, l)) R = fma_rn(RL[(c2 * N + l) * TC + f], pt.Af[c2][j][l], R);
+          });
         });
-        auto put = [&](int j, T R) {
-          const int64_t i = (int64_t)(5 * N + j) * S + c;
-          const T rhs = tm * pt.minvL[j] * R;
-          if (cmode == 0) out[i] = rhs;
-          else out[i] = tca * w0[i] + tcb * (LS[j * TC + f] + tdt * rhs);
-        };
-        put(j0, R0);
-        if constexpr (j1 < NDIV) put(j1, R1);
+        const int64_t i = (int64_t)(5 * N + j) * S + c;
+        const T rhs = tm * pt.minvL[j] * R;
+        if (cmode == 0) out[i] = rhs;
+        else out[i] = tca * w0[i] + tcb * (LS[j * TC + f] + tdt * rhs);
       }
     });
   }
@@ -1153,32 +1158,6 @@ __global__ void __launch_bounds__(NTP, 3) k_cell_list_pow(const OctPow<T> o, T g
                     ca32, cb32, cmode, sc, wmean, w0mean, outmean);
 }
 
-// Stages the density and LDF rows (N + NDIV) of cell cb into XB (with BOTH)
-// and of cell ca into XA, thread (v, f) rows v + 9 i; every load is issued
-// before the first shared-memory store. Absent faces stage rho = 1, zeros.
-template <typename T, int DEG, bool BOTH>
-__device__ __forceinline__ void stage_rd(const T* __restrict__ w, int64_t S, int64_t cb, int64_t ca, bool live,
-                                         int v, int f, T* XB, T* XA) {
-  constexpr int N = FastDims<DEG>::N, NRD = N + PowDims<DEG>::NDIV, PER = (NRD + 8) / 9;
-  T a[PER], b[PER];
-#pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    const int r = v + 9 * i;
-    const int64_t row = r < N ? r : 5 * N + (r - N);
-    const bool ok = live && r < NRD;
-    if (BOTH) b[i] = ok ? w[row * S + cb] : (r == 0 ? T(1) : T(0));
-    a[i] = ok ? w[row * S + ca] : (r == 0 ? T(1) : T(0));
-  }
-#pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    const int r = v + 9 * i;
-    if (r < NRD) {
-      if (BOTH) XB[r * TC + f] = b[i];
-      XA[r * TC + f] = a[i];
-    }
-  }
-}
-
 // Face jumps of the normal field for the Powell timestep (eq. powell_dt):
 // per face normal to each axis (right cell = this block's cell), B^n_F from
 // the two traces (eq. bxface-average) at every point and the weighted
@@ -1209,14 +1188,16 @@ __device__ __forceinline__ void divb_traces(const T* __restrict__ w, int64_t S, 
 #pragma unroll
       for (int p = 0; p < QF; ++p) acc[p] = fma_rn(x[l], role == 0 ? tb.PL[l][p] : tb.PR[l][p], acc[p]);
   } else {
-    // normal field from the LDF rows
+    // normal field from the LDF rows that have a component along A
     const T* pw = w + (int64_t)(5 * N) * S + cx;
+    static_for<NDIV>([&](auto J) {
+      constexpr int j = decltype(J)::value;
+      if constexpr (ldf_has<DEG>(j, A)) {
+        const T x = live ? pw[j * S] : T(0);
 #pragma unroll
-    for (int j = 0; j < NDIV; ++j, pw += S) {
-      const T x = live ? *pw : T(0);
-#pragma unroll
-      for (int p = 0; p < QF; ++p) acc[p] = fma_rn(x, role == 2 ? pt.Ln[A][1][j][p] : pt.Ln[A][0][j][p], acc[p]);
-    }
+        for (int p = 0; p < QF; ++p) acc[p] = fma_rn(x, role == 2 ? pt.Ln[A][1][j][p] : pt.Ln[A][0][j][p], acc[p]);
+      }
+    });
   }
 #pragma unroll
   for (int p = 0; p < QF; ++p) TD[(role * QF + p) * TC + f] = acc[p];
@@ -1270,51 +1251,89 @@ __global__ void __launch_bounds__(NTD) k_divb_face_pow(const FastGeom g, const T
 }
 
 // Face jumps of the normal field on an octree (the Powell timestep, eq.
-// powell_dt), per face block of one type: the density traces through the
-// type's trace tables, the normal field through the LDF functions' normal
-// components on the type's (sub-)faces (ntab); each face's two sums over its
-// points at jbuf[face * 2 + side].
-template <typename T, int DEG>
-__global__ void __launch_bounds__(NT) k_divb_list_pow(const OctPow<T> o, const T* __restrict__ w,
-                                                      T* __restrict__ jbuf) {
-  constexpr int N = FastDims<DEG>::N, QF = FastDims<DEG>::QF, NDIV = PowDims<DEG>::NDIV, NRD = N + NDIV;
+// powell_dt), per face block of one type, by the roles of k_divb_face_pow: warp
+// 0 / 1 the density traces of the left / right cells through the type's trace
+// tables, warp 2 / 3 their normal-field traces through the LDF functions'
+// normal components on the type's (sub-)faces (ntab), each thread every point
+// of its face: a state row is read once per face and side, and only the rows
+// with a component along the face's axis (10 to 14 of 26 at degree 2); the
+// tables are warp-uniform loads. Each face's two sums over its points at
+// jbuf[face * 2 + side]. (One point per warp with rows and tables staged in
+// shared memory read every row once per point: 0.83 ms on 1,387,520 leaves, now
+// 0.38 ms.)
+template <typename T, int DEG, int A>
+__device__ __forceinline__ void divb_list_traces(const OctPow<T>& o, const T* __restrict__ w, int type, int64_t cx,
+                                                 bool live, int role, int f, T* TD) {
+  constexpr int N = FastDims<DEG>::N, QF = FastDims<DEG>::QF, NDIV = PowDims<DEG>::NDIV;
   constexpr int QFP = FaceTabs<T, DEG>::QFP;
+  using T2 = std::conditional_t<sizeof(T) == 4, float2, double2>;
+  const int64_t S = o.stride;
+  T acc[QFP];
+#pragma unroll
+  for (int p = 0; p < QFP; ++p) acc[p] = T(0);
+  auto row = [&](T x, const T* tab) {
+    const T2* t2 = reinterpret_cast<const T2*>(tab);
+#pragma unroll
+    for (int p = 0; p < QFP / 2; ++p) {
+      const T2 q = __ldg(t2 + p);
+      acc[2 * p] = fma_rn(x, q.x, acc[2 * p]);
+      acc[2 * p + 1] = fma_rn(x, q.y, acc[2 * p + 1]);
+    }
+  };
+  if (role < 2) {
+    const T* tab = o.ftab + (size_t)(type * 2 + role) * N * QFP;
+    T x[N];
+    const T* pw = w + cx;
+#pragma unroll
+    for (int l = 0; l < N; ++l, pw += S) x[l] = live ? *pw : (l == 0 ? T(1) : T(0));
+#pragma unroll
+    for (int l = 0; l < N; ++l) row(x[l], tab + l * QFP);
+  } else {
+    const T* tab = o.ntab + (size_t)(type * 2 + role - 2) * NDIV * QFP;
+    const T* pw = w + (int64_t)(5 * N) * S + cx;
+    T x[NDIV];
+    static_for<NDIV>([&](auto J) {
+      constexpr int j = decltype(J)::value;
+      if constexpr (ldf_has<DEG>(j, A)) x[j] = live ? pw[j * S] : T(0);
+    });
+    static_for<NDIV>([&](auto J) {
+      constexpr int j = decltype(J)::value;
+      if constexpr (ldf_has<DEG>(j, A)) row(x[j], tab + j * QFP);
+    });
+  }
+#pragma unroll
+  for (int p = 0; p < QF; ++p) TD[(role * QF + p) * TC + f] = acc[p];
+}
+
+template <typename T, int DEG>
+__global__ void __launch_bounds__(NTD) k_divb_list_pow(const OctPow<T> o, const T* __restrict__ w,
+                                                       T* __restrict__ jbuf) {
+  constexpr int QF = FastDims<DEG>::QF;
   extern __shared__ __align__(16) unsigned char smraw[];
-  T* TT = reinterpret_cast<T*>(smraw);  // [2][N][QFP] density trace tables
-  T* TN = TT + 2 * N * QFP;             // [2][NDIV][QFP] normal LDF components
-  T* XL = TN + 2 * NDIV * QFP;          // [NRD][TC]
-  T* XR = XL + NRD * TC;                // [NRD][TC]
-  T* JS = XR + NRD * TC;                // [2][QF][TC] weighted jumps per point
+  T* TD = reinterpret_cast<T*>(smraw);  // [4][QF][TC] traces: rho L, rho R, B_n L, B_n R
+  T* JS = TD + 4 * QF * TC;             // [2][QF][TC] weighted jumps per point
   const PowTabs<T, DEG>& pt = pow_tabs<T, DEG>();
   const int t = threadIdx.x;
   const int f = t & (TC - 1);
-  const int v = t >> 5;
+  const int role = t >> 5;  // warp-uniform
   const int bt = o.btype[blockIdx.x];
   const int type = bt & 255, cnt = bt >> 8;
+  const int A = type / 9;
   const bool live = f < cnt;
   const int64_t fid = live ? o.bface[o.bstart[blockIdx.x] + f] : 0;
-  const int64_t cL = live ? o.fL[fid] : 0, cR = live ? o.fR[fid] : 0;
-  const int64_t S = o.stride;
-  for (int i = t; i < 2 * N * QFP; i += NT) TT[i] = o.ftab[(size_t)type * 2 * N * QFP + i];
-  for (int i = t; i < 2 * NDIV * QFP; i += NT) TN[i] = o.ntab[(size_t)type * 2 * NDIV * QFP + i];
-  stage_rd<T, DEG, true>(w, S, cR, cL, live, v, f, XR, XL);
+  const int64_t cx = live ? ((role & 1) ? o.fR[fid] : o.fL[fid]) : 0;
+  if (A == 0) divb_list_traces<T, DEG, 0>(o, w, type, cx, live, role, f, TD);
+  else if (A == 1) divb_list_traces<T, DEG, 1>(o, w, type, cx, live, role, f, TD);
+  else divb_list_traces<T, DEG, 2>(o, w, type, cx, live, role, f, TD);
   __syncthreads();
-  for (int p = v; p < QF; p += 9) {
-    T rL = T(0), rR = T(0), bL = T(0), bR = T(0);
-#pragma unroll
-    for (int l = 0; l < N; ++l) {
-      rL = fma_rn(XL[l * TC + f], TT[l * QFP + p], rL);
-      rR = fma_rn(XR[l * TC + f], TT[(N + l) * QFP + p], rR);
-    }
-#pragma unroll
-    for (int j = 0; j < NDIV; ++j) {
-      bL = fma_rn(XL[(N + j) * TC + f], TN[j * QFP + p], bL);
-      bR = fma_rn(XR[(N + j) * TC + f], TN[(NDIV + j) * QFP + p], bR);
-    }
+  for (int i = t; i < QF * TC; i += NTD) {
+    const int p = i / TC, ff = i % TC;
+    const T rL = TD[(0 * QF + p) * TC + ff], rR = TD[(1 * QF + p) * TC + ff];
+    const T bL = TD[(2 * QF + p) * TC + ff], bR = TD[(3 * QF + p) * TC + ff];
     const T bF = bn_face(rL, rR, bL, bR);
     const T wp = pt.wf[p];
-    JS[(0 * QF + p) * TC + f] = wp * (bF > bL ? bF - bL : bL - bF);
-    JS[(1 * QF + p) * TC + f] = wp * (bF > bR ? bF - bR : bR - bF);
+    JS[(0 * QF + p) * TC + ff] = wp * (bF > bL ? bF - bL : bL - bF);
+    JS[(1 * QF + p) * TC + ff] = wp * (bF > bR ? bF - bR : bR - bF);
   }
   __syncthreads();
   if (t < 2 * TC) {
@@ -1453,10 +1472,8 @@ void launch_cell_list_pow(const OctPow<T>& o, double gamma, const T* w, const T*
 
 template <typename T, int DEG>
 void launch_divb_list_pow(const OctPow<T>& o, const T* w, T* jbuf, cudaStream_t st) {
-  constexpr int N = FastDims<DEG>::N, NDIV = PowDims<DEG>::NDIV, QFP = FaceTabs<T, DEG>::QFP;
-  const size_t sm = (size_t)(2 * N * QFP + 2 * NDIV * QFP + 2 * (N + NDIV) * TC + 2 * FastDims<DEG>::QF * TC) *
-                    sizeof(T);
-  if (o.nblk > 0) k_divb_list_pow<T, DEG><<<(unsigned)o.nblk, NT, sm, st>>>(o, w, jbuf);
+  const size_t sm = (size_t)6 * FastDims<DEG>::QF * TC * sizeof(T);
+  if (o.nblk > 0) k_divb_list_pow<T, DEG><<<(unsigned)o.nblk, NTD, sm, st>>>(o, w, jbuf);
 }
 
 template <typename T, int DEG>

@@ -260,7 +260,7 @@ __device__ bool tvb_cell(const Geom& g, const LimTabs& lt, T* w, const double* w
   }
   if (!g.glm) {
     for (int j = 0; j < g.ndiv; ++j) {
-      if (lt.ldf_deg[j] == 0) continue;
+      if (!lt.ldf_lin[j]) continue;  // no linear part (at degree 2: all but 8 of the 26 functions)
       const R wj = (R)w[(int64_t)(g.ldf0 + j) * S + c];
       for (int cc = 0; cc < g.D; ++cc)
         for (int a = 0; a < g.D; ++a) sl[a][5 + cc] += wj * ltab<R>(lt.ldf_slope, lt.ldf_slope_f, (j * 3 + cc) * 3 + a);
@@ -986,6 +986,8 @@ int upload_limiter_tables(Ctx& c) {
         lt.ldf_slope[(j * 3 + cc) * 3 + a] = ia / xi2;
         lt.ldf_pl[(j * 3 + cc) * 3 + a] = ia / Mj;
       }
+      for (int a = 0; a < g.D; ++a)
+        if (std::fabs(lt.ldf_slope[(j * 3 + cc) * 3 + a]) > 1e-13) lt.ldf_lin[j] = 1;
       double mx = 0.0;
       for (double v : B.ldf[j][cc]) mx += std::fabs(v);
       lt.ldf_maxabs[j * 3 + cc] = mx;

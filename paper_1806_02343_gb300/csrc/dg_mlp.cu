@@ -18,9 +18,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <random>
 #include <vector>
 
+#include "dg_ldf.cuh"
 #include "dg_mlp.cuh"
 #include "dg_pos.cuh"
 #include "dg_tc.cuh"
@@ -54,6 +54,7 @@ __device__ __forceinline__ int mrow(const Geom& g, int m) {
 // Geom at run time; CtDims<GLM, DEG> fixes them at compile time (3D), so the
 // loops over variables and modes unroll and every row index is a constant.
 struct RtDims {
+  static constexpr bool SPARSE = false;
   const Geom& g;
   const MlpTabs& mt;
   __device__ int n() const { return g.n; }
@@ -71,6 +72,12 @@ struct CtDims {
   static constexpr int N = (DEG + 1) * (DEG + 2) * (DEG + 3) / 6;
   // LDF basis size in 3D (Table A1): 3, 11, 26, 50 for degrees 0..3
   static constexpr int NDIV = DEG == 0 ? 3 : DEG == 1 ? 11 : DEG == 2 ? 26 : 50;
+  // the LDF -> Legendre map's pattern is known for degrees 1 and 2
+  static constexpr bool SPARSE = !GLM && (DEG == 1 || DEG == 2);
+  __device__ static constexpr bool has(int j, int c, int l) {
+    if constexpr (SPARSE) return ldf_has<DEG>(j, c, l);
+    else return true;
+  }
   __device__ static constexpr int n() { return N; }
   __device__ static constexpr bool glm() { return GLM; }
   __device__ static constexpr int D() { return 3; }
@@ -217,7 +224,14 @@ __device__ __forceinline__ void features_of(const Dm& dm, const MlpTabs& mt, con
 #pragma unroll
       for (int l = 0; l < n; ++l) {
         float acc = 0.f;
-        for (int j = 0; j < dm.ndiv(); ++j) acc += src.row(dm.ldf0() + j) * mt.l2l[(j * 3 + cc) * MLP_MAXN + l];
+        if constexpr (Dm::SPARSE) {
+          // only the map's non-zero entries (38 of 780 at degree 2), in the order of j
+#pragma unroll
+          for (int j = 0; j < Dm::ndiv(); ++j)
+            if (Dm::has(j, cc, l)) acc += src.row(dm.ldf0() + j) * mt.l2l[(j * 3 + cc) * MLP_MAXN + l];
+        } else {
+          for (int j = 0; j < dm.ndiv(); ++j) acc += src.row(dm.ldf0() + j) * mt.l2l[(j * 3 + cc) * MLP_MAXN + l];
+        }
         put((5 + cc) * n + l, acc * inv[5 + cc]);
 #pragma unroll
         for (int a = 0; a < 3; ++a)

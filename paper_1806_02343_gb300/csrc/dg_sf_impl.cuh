@@ -524,16 +524,13 @@ DG_SF_INST(true)
 #if DG_SF_DEG <= 2
 DG_SF_INST(false)
 
-// copies the map to the constant bank (synchronous; 0, -3, or -7 where the basis has another pattern)
+// copies the map to the constant bank (synchronous; 0 or -3)
 template <int DEG>
 int sf_ldf_to_constant(const PowTabs<double, DEG>& pt) {
   LdfTab<DEG> t;
   for (int j = 0; j < LdfPattern<DEG>::NDIV; ++j) {
     for (int cc = 0; cc < 3; ++cc)
-      for (int l = 0; l < LdfPattern<DEG>::N; ++l) {
-        t.A[j][cc][l] = pt.Af[cc][j][l];
-        if (t.A[j][cc][l] != 0.0 && !ldf_has<DEG>(j, cc, l)) return -7;
-      }
+      for (int l = 0; l < LdfPattern<DEG>::N; ++l) t.A[j][cc][l] = pt.Af[cc][j][l];
     t.minv[j] = pt.minvL[j];
   }
   return cudaMemcpyToSymbol(c_ldf, &t, sizeof(t)) == cudaSuccess ? 0 : -3;
