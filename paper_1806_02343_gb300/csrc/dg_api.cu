@@ -1179,10 +1179,10 @@ int dg_mhd_mlp_loss_grad(const float* X, int ldx, const uint8_t* y, int64_t n, i
                          float pos_weight, float* grad, double* loss, void* stream) {
   if (!X || !y || !theta || !grad || n < 1 || nin < 1 || ldx < nin || n > (int64_t)1 << 30) return DG_E_ARG;
   void* scratch = nullptr;
-  if (cudaMalloc(&scratch, mlp_scratch_bytes((int)n)) != cudaSuccess) return DG_E_CUDA;
+  if (cudaMalloc(&scratch, mlp_scratch_bytes((int)n, nin)) != cudaSuccess) return DG_E_CUDA;
   cudaStream_t st = S(stream);
   if (loss) cudaMemsetAsync(loss, 0, sizeof(double), st);
-  int e = mlp_loss_grad_dev(X, ldx, y, nullptr, 0, (int)n, nin, theta, grad, loss, pos_weight, (float)n, scratch, st);
+  int e = mlp_loss_grad_dev(X, ldx, y, (int)n, nin, theta, grad, loss, pos_weight, scratch, st);
   cudaStreamSynchronize(st);
   cudaFree(scratch);
   return e;

@@ -1,5 +1,5 @@
-// Learned troubled-cell indicator: features, BF16 tensor-core inference fused
-// with the feature pass, and FP32 training kernels (forward, backward, Adam).
+// Learned troubled-cell indicator: features and BF16 tensor-core inference fused
+// with the feature pass (the training kernels: dg_train.cu).
 //
 // Detection is its own step of the limiter (Sec. 4.2: first detect troubled
 // cells, then limit them); this network replaces the TVB detection and only the
@@ -425,111 +425,6 @@ __global__ void __launch_bounds__(128) k_mlp_infer(Geom g, MlpTabs mt, const T* 
   }
 }
 
-// ---------------------------------------------------------------- training (FP32)
-// Z[b][o] = sum_k A[idx(b)][k] W[o][k] + bias[o] (A rows gathered through perm if given)
-__global__ void k_dense(const float* __restrict__ A, int lda, const int64_t* __restrict__ perm, int64_t off,
-                        const float* __restrict__ W, const float* __restrict__ bias, float* __restrict__ Z, int nb,
-                        int nin, int nout, int relu_in) {
-  const int o = threadIdx.x % nout;
-  const int b = blockIdx.x * (blockDim.x / nout) + threadIdx.x / nout;
-  if (b >= nb || threadIdx.x >= (blockDim.x / nout) * nout) return;
-  const int64_t row = perm ? perm[off + b] : off + b;
-  const float* a = A + row * lda;
-  float s = bias[o];
-  for (int k = 0; k < nin; ++k) {
-    float x = a[k];
-    if (relu_in) x = fmaxf(x, 0.f);
-    s += x * W[o * nin + k];
-  }
-  Z[(int64_t)b * nout + o] = s;
-}
-
-// output layer, loss and delta3 = (p - y) * weight / n
-__global__ void k_out(const float* __restrict__ Z2, const float* __restrict__ w3, float b3,
-                      const uint8_t* __restrict__ y, const int64_t* __restrict__ perm, int64_t off, int nb,
-                      float pos_weight, float inv_n, float* __restrict__ d3, double* __restrict__ loss) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nb) return;
-  float z = b3;
-  for (int k = 0; k < HID; ++k) z += fmaxf(Z2[(int64_t)b * HID + k], 0.f) * w3[k];
-  const float p = 1.f / (1.f + expf(-z));
-  const int64_t row = perm ? perm[off + b] : off + b;
-  const float yy = y[row] ? 1.f : 0.f;
-  // weighted BCE: -(pw y log p + (1-y) log(1-p)); dL/dz = pw y (p - 1) + (1 - y) p
-  d3[b] = (pos_weight * yy * (p - 1.f) + (1.f - yy) * p) * inv_n;
-  if (loss) {
-    const double l = -(pos_weight * yy * log((double)p + 1e-12) + (1.0 - yy) * log(1.0 - (double)p + 1e-12));
-    atomicAdd(loss, l * (double)inv_n);
-  }
-}
-
-// delta2[b][k] = d3[b] * w3[k] * (Z2 > 0)
-__global__ void k_back2(const float* __restrict__ d3, const float* __restrict__ w3, const float* __restrict__ Z2,
-                        float* __restrict__ d2, int nb) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)nb * HID) return;
-  const int k = (int)(i % HID);
-  const int64_t b = i / HID;
-  d2[i] = Z2[i] > 0.f ? d3[b] * w3[k] : 0.f;
-}
-
-// delta1[b][k] = sum_o d2[b][o] W2[o][k] * (Z1 > 0)
-__global__ void k_back1(const float* __restrict__ d2, const float* __restrict__ W2, const float* __restrict__ Z1,
-                        float* __restrict__ d1, int nb) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)nb * HID) return;
-  const int k = (int)(i % HID);
-  const int64_t b = i / HID;
-  float s = 0.f;
-  for (int o = 0; o < HID; ++o) s += d2[b * HID + o] * W2[o * HID + k];
-  d1[i] = Z1[i] > 0.f ? s : 0.f;
-}
-
-// gW[o][k] = sum_b delta[b][o] act(A[row(b)][k]); gb[o] = sum_b delta[b][o] (fixed order)
-__global__ void k_wgrad(const float* __restrict__ delta, int nout, const float* __restrict__ A, int lda,
-                        const int64_t* __restrict__ perm, int64_t off, int nin, int relu_in, int nb,
-                        float* __restrict__ gW, float* __restrict__ gb) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nout * (nin + 1)) return;
-  const int o = i / (nin + 1), k = i % (nin + 1);
-  float s = 0.f;
-  for (int b = 0; b < nb; ++b) {
-    const float d = delta[(int64_t)b * nout + o];
-    if (k == nin) {
-      s += d;
-    } else {
-      const int64_t row = perm ? perm[off + b] : off + b;
-      float x = A[row * lda + k];
-      if (relu_in) x = fmaxf(x, 0.f);
-      s += d * x;
-    }
-  }
-  if (k == nin) gb[o] = s;
-  else gW[o * nin + k] = s;
-}
-
-__global__ void k_gout(const float* __restrict__ d3, const float* __restrict__ Z2, int nb, float* __restrict__ gw3,
-                       float* __restrict__ gb3) {
-  const int k = threadIdx.x;
-  if (k > HID) return;
-  float s = 0.f;
-  for (int b = 0; b < nb; ++b) s += k == HID ? d3[b] : d3[b] * fmaxf(Z2[(int64_t)b * HID + k], 0.f);
-  if (k == HID) *gb3 = s;
-  else gw3[k] = s;
-}
-
-__global__ void k_adam(float* __restrict__ th, const float* __restrict__ gr, float* __restrict__ m,
-                       float* __restrict__ v, int n, float lr, float b1, float b2, float eps, float c1, float c2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float g = gr[i];
-  const float mi = b1 * m[i] + (1.f - b1) * g;
-  const float vi = b2 * v[i] + (1.f - b2) * g * g;
-  m[i] = mi;
-  v[i] = vi;
-  th[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
-
 __global__ void k_to_bf16(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, int rows, int cols,
                           int ldd) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -537,10 +432,6 @@ __global__ void k_to_bf16(const float* __restrict__ src, __nv_bfloat16* __restri
   const int r = i / ldd, k = i % ldd;
   dst[i] = __float2bfloat16_rn(k < cols ? src[r * cols + k] : 0.f);
 }
-
-struct Scratch {
-  float *Z1 = nullptr, *Z2 = nullptr, *d1 = nullptr, *d2 = nullptr, *d3 = nullptr;
-};
 
 // ---------------------------------------------------------------- staged inference
 // FP32 form on uniform 3D meshes whose x-rows hold whole 128-cell tiles: the
@@ -846,93 +737,6 @@ __global__ void __launch_bounds__(NTH) k_mlp_staged(Geom g, MlpTabs mt, const fl
 }
 
 }  // namespace
-
-// full-batch (or mini-batch) loss and gradient; grad layout = theta layout
-int mlp_loss_grad_dev(const float* X, int ldx, const uint8_t* y, const int64_t* perm, int64_t off, int nb, int nin,
-                      const float* theta, float* grad, double* loss, float pos_weight, float norm_n, void* scratch,
-                      cudaStream_t st) {
-  const float* W1 = theta;
-  const float* b1 = W1 + HID * nin;
-  const float* W2 = b1 + HID;
-  const float* b2 = W2 + HID * HID;
-  const float* w3 = b2 + HID;
-  float* gW1 = grad;
-  float* gb1 = gW1 + HID * nin;
-  float* gW2 = gb1 + HID;
-  float* gb2 = gW2 + HID * HID;
-  float* gw3 = gb2 + HID;
-  float* gb3 = gw3 + HID;
-  float* s = static_cast<float*>(scratch);
-  float* Z1 = s;
-  float* Z2 = Z1 + (size_t)nb * HID;
-  float* d1 = Z2 + (size_t)nb * HID;
-  float* d2 = d1 + (size_t)nb * HID;
-  float* d3 = d2 + (size_t)nb * HID;
-  float b3;
-  if (cudaMemcpyAsync(&b3, w3 + HID, sizeof(float), cudaMemcpyDeviceToHost, st) != cudaSuccess) return -3;
-  if (cudaStreamSynchronize(st) != cudaSuccess) return -3;
-  const int per = 256 / HID;
-  k_dense<<<(nb + per - 1) / per, per * HID, 0, st>>>(X, ldx, perm, off, W1, b1, Z1, nb, nin, HID, 0);
-  k_dense<<<(nb + per - 1) / per, per * HID, 0, st>>>(Z1, HID, nullptr, 0, W2, b2, Z2, nb, HID, HID, 1);
-  k_out<<<(nb + 255) / 256, 256, 0, st>>>(Z2, w3, b3, y, perm, off, nb, pos_weight, 1.f / norm_n, d3, loss);
-  const int64_t nh = (int64_t)nb * HID;
-  k_back2<<<(unsigned)((nh + 255) / 256), 256, 0, st>>>(d3, w3, Z2, d2, nb);
-  k_back1<<<(unsigned)((nh + 255) / 256), 256, 0, st>>>(d2, W2, Z1, d1, nb);
-  k_gout<<<1, 128, 0, st>>>(d3, Z2, nb, gw3, gb3);
-  k_wgrad<<<(HID * (HID + 1) + 127) / 128, 128, 0, st>>>(d2, HID, Z1, HID, nullptr, 0, HID, 1, nb, gW2, gb2);
-  k_wgrad<<<(HID * (nin + 1) + 127) / 128, 128, 0, st>>>(d1, HID, X, ldx, perm, off, nin, 0, nb, gW1, gb1);
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
-}
-
-size_t mlp_scratch_bytes(int nb) { return ((size_t)nb * HID * 4 + nb) * sizeof(float); }
-
-int mlp_train_dev(const float* X, int ldx, const uint8_t* y, int64_t n, int nin, float* theta, int epochs,
-                  int batch, float lr, float pos_weight, uint64_t seed, double* last_loss, cudaStream_t st) {
-  const int np = mlp_n_params(nin);
-  float *grad = nullptr, *m = nullptr, *v = nullptr;
-  void* scratch = nullptr;
-  int64_t* perm = nullptr;
-  double* dloss = nullptr;
-  int e = 0;
-  if (cudaMalloc(&grad, np * sizeof(float)) || cudaMalloc(&m, np * sizeof(float)) ||
-      cudaMalloc(&v, np * sizeof(float)) || cudaMalloc(&scratch, mlp_scratch_bytes(batch)) ||
-      cudaMalloc(&perm, n * sizeof(int64_t)) || cudaMalloc(&dloss, sizeof(double)))
-    e = -3;
-  if (!e) {
-    cudaMemsetAsync(m, 0, np * sizeof(float), st);
-    cudaMemsetAsync(v, 0, np * sizeof(float), st);
-    std::vector<int64_t> hp(n);
-    for (int64_t i = 0; i < n; ++i) hp[i] = i;
-    std::mt19937_64 rng(seed);
-    int t = 0;
-    for (int ep = 0; ep < epochs && !e; ++ep) {
-      std::shuffle(hp.begin(), hp.end(), rng);
-      if (cudaMemcpyAsync(perm, hp.data(), n * sizeof(int64_t), cudaMemcpyHostToDevice, st)) e = -3;
-      cudaMemsetAsync(dloss, 0, sizeof(double), st);
-      for (int64_t off = 0; off + batch <= n && !e; off += batch) {
-        ++t;
-        e = mlp_loss_grad_dev(X, ldx, y, perm, off, batch, nin, theta, grad, ep == epochs - 1 ? dloss : nullptr,
-                              pos_weight, (float)batch, scratch, st);
-        const float c1 = 1.f - powf(0.9f, (float)t), c2 = 1.f - powf(0.999f, (float)t);
-        k_adam<<<(np + 255) / 256, 256, 0, st>>>(theta, grad, m, v, np, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
-      }
-      if (cudaStreamSynchronize(st) != cudaSuccess) e = -3;
-    }
-    if (!e && last_loss) {
-      double l = 0.0;
-      cudaMemcpy(&l, dloss, sizeof(double), cudaMemcpyDeviceToHost);
-      const int64_t nbat = n / batch;
-      *last_loss = nbat ? l / (double)nbat : 0.0;
-    }
-  }
-  cudaFree(grad);
-  cudaFree(m);
-  cudaFree(v);
-  cudaFree(scratch);
-  cudaFree(perm);
-  cudaFree(dloss);
-  return e;
-}
 
 static AmrFeat amr_feat(const Ctx& c) {
   return AmrFeat{c.amr.side_nb, c.amr.side_info, c.amr.dxc, c.g.dx, c.amr.on ? 1 : 0};

@@ -17,10 +17,10 @@ int mlp_set_weights(Ctx& c, const float* theta_dev, int nin, float thresh);
 // flagged cells after limiting them); *screened tells whether it did.
 int mlp_infer_launch(Ctx& c, const void* w, const double* wmean, uint8_t* flag, float* prob, cudaStream_t st,
                      int32_t* list = nullptr, int32_t* pos_list = nullptr, bool* screened = nullptr);
-size_t mlp_scratch_bytes(int nb);
-int mlp_loss_grad_dev(const float* X, int ldx, const uint8_t* y, const int64_t* perm, int64_t off, int nb, int nin,
-                      const float* theta, float* grad, double* loss, float pos_weight, float norm_n, void* scratch,
-                      cudaStream_t st);
+// training (dg_train.cu): loss and gradient of the mean over nb samples
+size_t mlp_scratch_bytes(int nb, int nin);
+int mlp_loss_grad_dev(const float* X, int ldx, const uint8_t* y, int nb, int nin, const float* theta, float* grad,
+                      double* loss, float pos_weight, void* scratch, cudaStream_t st);
 int mlp_train_dev(const float* X, int ldx, const uint8_t* y, int64_t n, int nin, float* theta, int epochs, int batch,
                   float lr, float pos_weight, uint64_t seed, double* last_loss, cudaStream_t st);
 
