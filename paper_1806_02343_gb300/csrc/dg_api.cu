@@ -290,6 +290,18 @@ void build_pow_tabs(PowTabs<T, DEG>& pt) {
   pt.ok = 1;
 }
 
+// the LDF map of the sum-factorised projection (3D Powell), built on first use;
+// false: another basis than dg_ldf.cuh's (the dense projection runs)
+bool project_ldf(Ctx& c) {
+  if (c.proj_ldf) return true;
+  std::vector<double> A;
+  int nd = 0, nm = 0;
+  if (!ldf_legendre_3d(c.g.d, A, nd, nm) || nd != c.g.ndiv || nm != c.g.n || !ldf_pattern_ok(c.g.d, A.data()))
+    return false;
+  for (int j = 0; j < nd; ++j) A.push_back(1.0 / c.hb->ldf_mass[j]);
+  return upload(&c.proj_ldf, A) == DG_OK;
+}
+
 template <typename T, int DEG>
 void* make_fast_tabs(const HostTables& h, const Geom& g, const Basis& B) {
   using Dm = FastDims<DEG>;
@@ -581,7 +593,7 @@ void dg_mhd_destroy(dg_mhd_ctx* ctx) {
   free_tables(c.t64);
   free_tables(c.t32);
   void* ptrs[] = {c.sc, c.face_buf, c.face_buf32, c.stage_buf[0], c.stage_buf[1], c.stage_buf[2],
-                  c.stage_mean[0], c.stage_mean[1], c.stage_mean[2], c.cellscratch, c.proj_tab, c.proj_w,
+                  c.stage_mean[0], c.stage_mean[1], c.stage_mean[2], c.cellscratch, c.proj_tab, c.proj_w, c.proj_ldf,
                   c.troubled, c.flag_list, c.pos_list, c.mlp_w1, c.mlp_w2, c.mlp_bias, c.rg_tabs, c.qdag_buf,
                   c.tc_tabs, c.owned};
   for (void* p : ptrs)
@@ -788,6 +800,12 @@ int dg_mhd_project(dg_mhd_ctx* ctx, const double* nodal, int npts, void* w, doub
   Ctx& c = ctx->c;
   const Geom& g = c.g;
   if (fp32(c) && !wmean) return DG_E_ARG;
+  if (project_sf_ok(g, npts) && (g.glm || project_ldf(c))) {
+    c.prof.launches[4] += 1;
+    if (fp32(c)) launch_project_sf<float>(g, npts, nodal, c.proj_ldf, (float*)w, wmean, S(stream));
+    else launch_project_sf<double>(g, npts, nodal, c.proj_ldf, (double*)w, nullptr, S(stream));
+    return cudaGetLastError() == cudaSuccess ? DG_OK : DG_E_CUDA;
+  }
   if (npts != c.proj_npts) {
     // table[(r*Qp + q)*3 + k] = k-th active component of row r at point q
     std::vector<double> x1, w1;

@@ -252,6 +252,7 @@ struct Ctx {
   int proj_npts = 0;
   double* proj_tab = nullptr;      // projection table [r][q][comp]
   double* proj_w = nullptr;
+  double* proj_ldf = nullptr;      // LDF map of the sum-factorised projection (dg_project.cu)
   uint8_t* troubled = nullptr;     // per-cell limiter flags (scratch)
   int32_t* flag_list = nullptr;    // cells flagged by the indicator in the current pass
   int32_t* pos_list = nullptr;     // cells the positivity screen could not clear in the current pass

@@ -29,20 +29,26 @@ using V = double;
 // normalised sums below start with a plain addition.
 template <int DEG>
 struct Rule {
+  static_assert(DEG >= 1 && DEG <= 5, "2 to 6 points");
   static constexpr int NQ = DEG + 1, NP = NQ / 2;
   static constexpr bool MID = NQ & 1;
   static constexpr __host__ __device__ double x(int i) {
     return DEG == 1 ? 0.57735026918962576451
          : DEG == 2 ? 0.77459666924148337704
-                    : (i == 0 ? 0.86113631159405257522 : 0.33998104358485626480);
+         : DEG == 3 ? (i == 0 ? 0.86113631159405257522 : 0.33998104358485626480)
+         : DEG == 4 ? (i == 0 ? 0.90617984593866399280 : 0.53846931010568309104)
+                    : (i == 0 ? 0.93246951420315202781 : i == 1 ? 0.66120938646626451366 : 0.23861918608319690863);
   }
-  static constexpr __host__ __device__ double w0() {  // weight of x(0)
-    return DEG == 1 ? 1.0 : DEG == 2 ? 5.0 / 9.0 : 0.34785484513745385737;
+  static constexpr __host__ __device__ double w(int i) {  // weight of x(i)
+    return DEG == 1 ? 1.0
+         : DEG == 2 ? 5.0 / 9.0
+         : DEG == 3 ? (i == 0 ? 0.34785484513745385737 : 0.65214515486254614263)
+         : DEG == 4 ? (i == 0 ? 0.23692688505618908751 : 0.47862867049936646804)
+                    : (i == 0 ? 0.17132449237917034504 : i == 1 ? 0.36076157304813860757 : 0.46791393457269104739);
   }
-  static constexpr __host__ __device__ double wr(int i) {  // w(x(i)) / w0
-    return i == 0 ? 1.0 : 0.65214515486254614263 / 0.34785484513745385737;
-  }
-  static constexpr __host__ __device__ double wm() { return DEG == 0 ? 2.0 : 8.0 / 5.0; }  // w(0) / w0
+  static constexpr __host__ __device__ double w0() { return w(0); }
+  static constexpr __host__ __device__ double wr(int i) { return w(i) / w(0); }
+  static constexpr __host__ __device__ double wm() { return (DEG == 2 ? 8.0 / 9.0 : 0.56888888888888888889) / w(0); }  // of the point 0
   // node of point index q: -x(0) first ... +x(0) last
   static constexpr __host__ __device__ double node(int q) {
     return (MID && q == NP) ? 0.0 : (q < NP ? -x(q) : x(NQ - 1 - q));
@@ -75,6 +81,9 @@ constexpr __host__ __device__ int mode2_idx(int j, int k) {
   int n = 0;
   for (int a = 0; a < j; ++a) n += DEG + 1 - a;
   return n + k;
+}
+constexpr __host__ __device__ double mode_minv(int i, int j, int k) {  // 1 / mass of the Legendre mode
+  return (2 * i + 1) * (2 * j + 1) * (2 * k + 1) / 8.0;
 }
 constexpr __host__ __device__ int n_modes2(int deg) { return (deg + 1) * (deg + 2) / 2; }
 constexpr __host__ __device__ bool is_one(double x) { return x > 1.0 - 1e-13 && x < 1.0 + 1e-13; }

@@ -248,9 +248,6 @@ constexpr __host__ __device__ double mode_scale(int i, int j, int k) {
        : k > 0 ? (2 * k - 1) * sig<DEG>(i) * sig<DEG>(j) * sig<DEG>(k - 1)
                : 1.0;
 }
-constexpr __host__ __device__ double mode_minv(int i, int j, int k) {
-  return (2 * i + 1) * (2 * j + 1) * (2 * k + 1) / 8.0;
-}
 
 // f(i, j, k, l) for the modes (l: their index) of total degree <= DEG
 template <int DEG, typename F>
@@ -456,7 +453,7 @@ __global__ void __launch_bounds__(NTS, 2) k_sf_cell(const FastGeom g, const V* _
     each_mode<DEG>([&](int i, int j, int k, int l) {
       if (l > 0)
         put(v * N + l, wl[l],
-            __fma_rn(-kap, wl[l], tm * (mode_minv(i, j, k) * mode_scale<DEG>(i, j, k)) * racc[l]));
+            __fma_rn(-kap, wl[l], tm * (sf::mode_minv(i, j, k) * mode_scale<DEG>(i, j, k)) * racc[l]));
     });
   }
 #if DG_SF_DEG <= 2
