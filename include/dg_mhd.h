@@ -251,9 +251,9 @@ int dg_mhd_status(dg_mhd_ctx* ctx, int sync);
 int dg_mhd_counters(dg_mhd_ctx* ctx, int64_t* pos_cells, double* inj_mass, double* inj_energy, int reset);
 
 /* Workload of the positivity limiter in the FP32 form (measurement support,
- * no counterpart in the paper): cells whose FP32 screen could not clear them
- * and that therefore went through the full procedure, summed over limiter
- * passes since the last reset (FP64 contexts run the procedure on every cell
+ * no counterpart in the paper): cells whose FP32 bound could not clear them and
+ * that therefore went to the listed-cell kernel (point-wise screen, then the
+ * full procedure of the cells still open), summed over limiter passes since the last reset (FP64 contexts run the procedure on every cell
  * and count 0). Synchronises the device; reset = 1 clears the count. */
 int dg_mhd_positivity_listed(dg_mhd_ctx* ctx, int64_t* listed, int reset);
 

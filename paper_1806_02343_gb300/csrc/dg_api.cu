@@ -195,22 +195,17 @@ void free_tables(Tables<T>& t) {
 
 inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
-// Powell kernels' tables (dg_fast.cuh PowTabs): the Legendre coefficients of
-// the LDF functions' components by quadrature (exact: every component is a
-// polynomial of total degree <= d), checked against the functions themselves;
-// ok = 0 when the basis lacks the structure the kernels rely on (three
-// constant functions, each along one axis, no other function with a non-zero
-// mean, no entry outside dg_ldf.cuh's pattern). The same for every context of this degree.
+}  // namespace
+
+namespace dgmhd {
+
 // A[(j * 3 + c) * n + l]: the Legendre coefficients of component c of the 3D
 // LDF function j of degree <= deg, by quadrature with deg + 1 Gauss points
 // per axis (exact: the products are polynomials of degree <= 2 deg per
 // axis), entries below 1e-13 set to zero, and the expansion checked against
 // the functions at the points (false if it misses by more than 1e-11).
-bool ldf_legendre_3d(int deg, std::vector<double>& A, int& ndiv, int& n) {
-  Basis L;
-  if (!L.build(3, deg, true)) return false;
-  ndiv = L.ndiv;
-  n = L.n;
+bool ldf_legendre_3d(const Basis& L, int deg, std::vector<double>& A) {
+  const int ndiv = L.ndiv, n = L.n;
   std::vector<double> x1, w1;
   gauss_legendre(deg + 1, x1, w1);
   int Qv = 1;
@@ -221,36 +216,47 @@ bool ldf_legendre_3d(int deg, std::vector<double>& A, int& ndiv, int& n) {
     vol_point(3, x1, q, xi);
     double wq = 1.0;
     for (int k = 0, qq = q; k < 3; ++k, qq /= deg + 1) wq *= w1[qq % (deg + 1)];
-    for (int l = 0; l < n; ++l) {
-      const double Pl = L.eval(L.leg[l], xi) * wq / L.leg_mass[l];
-      for (int j = 0; j < ndiv; ++j)
-        for (int cc = 0; cc < 3; ++cc) A[((size_t)j * 3 + cc) * n + l] += L.eval(L.ldf[j][cc], xi) * Pl;
-    }
+    std::vector<double> Pl(n);
+    for (int l = 0; l < n; ++l) Pl[l] = L.eval(L.leg[l], xi) * wq / L.leg_mass[l];
+    for (int j = 0; j < ndiv; ++j)
+      for (int cc = 0; cc < 3; ++cc) {
+        const double e = L.eval(L.ldf[j][cc], xi);
+        for (int l = 0; l < n; ++l) A[((size_t)j * 3 + cc) * n + l] += e * Pl[l];
+      }
   }
   for (double& x : A)
     if (std::fabs(x) < 1e-13) x = 0.0;
   for (int q = 0; q < Qv; ++q) {
     vol_point(3, x1, q, xi);
+    std::vector<double> P(n);
+    for (int l = 0; l < n; ++l) P[l] = L.eval(L.leg[l], xi);
     for (int j = 0; j < ndiv; ++j)
       for (int cc = 0; cc < 3; ++cc) {
         double s = 0.0;
-        for (int l = 0; l < n; ++l) s += A[((size_t)j * 3 + cc) * n + l] * L.eval(L.leg[l], xi);
+        for (int l = 0; l < n; ++l) s += A[((size_t)j * 3 + cc) * n + l] * P[l];
         if (std::fabs(s - L.eval(L.ldf[j][cc], xi)) > 1e-11) return false;
       }
   }
   return true;
 }
 
+}  // namespace dgmhd
+
+namespace {
+
+// Powell kernels' tables (dg_fast.cuh PowTabs): the Legendre coefficients of
+// the LDF functions' components by quadrature (exact: every component is a
+// polynomial of total degree <= d), checked against the functions themselves;
+// ok = 0 when the basis lacks the structure the kernels rely on (three
+// constant functions, each along one axis, no other function with a non-zero
+// mean, no entry outside dg_ldf.cuh's pattern). The same for every context of this degree.
 template <typename T, int DEG>
-void build_pow_tabs(PowTabs<T, DEG>& pt) {
+void build_pow_tabs(const Basis& L, PowTabs<T, DEG>& pt) {
   using Dm = FastDims<DEG>;
   constexpr int N = Dm::N, NDIV = PowDims<DEG>::NDIV;
   pt = PowTabs<T, DEG>();
   std::vector<double> A;
-  int nd = 0, nm = 0;
-  if (!ldf_legendre_3d(DEG, A, nd, nm) || nd != NDIV || nm != N) return;
-  Basis L;
-  L.build(3, DEG, true);
+  if (L.ndiv != NDIV || L.n != N || !ldf_legendre_3d(L, DEG, A)) return;
   std::vector<double> x1, w1;
   gauss_legendre(DEG + 1, x1, w1);
   double xi[3];
@@ -295,10 +301,8 @@ void build_pow_tabs(PowTabs<T, DEG>& pt) {
 bool project_ldf(Ctx& c) {
   if (c.proj_ldf) return true;
   std::vector<double> A;
-  int nd = 0, nm = 0;
-  if (!ldf_legendre_3d(c.g.d, A, nd, nm) || nd != c.g.ndiv || nm != c.g.n || !ldf_pattern_ok(c.g.d, A.data()))
-    return false;
-  for (int j = 0; j < nd; ++j) A.push_back(1.0 / c.hb->ldf_mass[j]);
+  if (!ldf_legendre_3d(*c.hb, c.g.d, A) || !ldf_pattern_ok(c.g.d, A.data())) return false;
+  for (int j = 0; j < c.g.ndiv; ++j) A.push_back(1.0 / c.hb->ldf_mass[j]);
   return upload(&c.proj_ldf, A) == DG_OK;
 }
 
@@ -333,7 +337,9 @@ void* make_fast_tabs(const HostTables& h, const Geom& g, const Basis& B) {
       for (int q = 0; q < Qv; ++q) ft->cell.dP2[a][i / 2][q][i % 2] = (T)(h.dPv[((size_t)a * n + l) * Qv + q] * h.wv[q]);
     }
   static_assert(Dm::N > 0, "");
-  if constexpr (DEG <= 2) build_pow_tabs<T, DEG>(ft->pow);
+  if constexpr (DEG <= 2) {
+    if (!g.glm) build_pow_tabs<T, DEG>(B, ft->pow);
+  }
   if (fast_to_constant<T, DEG>(*ft)) {
     delete ft;
     return nullptr;
@@ -1231,11 +1237,11 @@ int dg_mhd_counters(dg_mhd_ctx* ctx, int64_t* pos_cells, double* inj_mass, doubl
 
 int dg_mhd_ldf_legendre(int degree, int64_t cap, double* A, int* n_div, int* n_modes) {
   if (degree < 0 || degree > MAXD) return DG_E_ARG;
+  Basis L;
   std::vector<double> M;
-  int nd = 0, nm = 0;
-  if (!ldf_legendre_3d(degree, M, nd, nm)) return DG_E_UNSUPPORTED;
-  if (n_div) *n_div = nd;
-  if (n_modes) *n_modes = nm;
+  if (!L.build(3, degree, true) || !ldf_legendre_3d(L, degree, M)) return DG_E_UNSUPPORTED;
+  if (n_div) *n_div = L.ndiv;
+  if (n_modes) *n_modes = L.n;
   if (A) {
     if (cap < (int64_t)M.size()) return DG_E_ARG;
     std::copy(M.begin(), M.end(), A);

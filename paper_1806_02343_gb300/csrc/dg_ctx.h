@@ -158,6 +158,13 @@ struct PosScreen {
   float eps_rho, eps_p, gm1;
 };
 
+// LDF -> Legendre map of the point-wise positivity screen (kernel parameter):
+// A[(j * 3 + c) * n + l], 3D degrees 1 and 2; ok: the basis has dg_ldf.cuh's pattern
+struct LdfLeg {
+  float A[26 * 3 * 10];
+  int ok;
+};
+
 // Launch accounting: counts every kernel launch; with `on`, records a CUDA
 // event pair on the launch stream around each launch of a given kind.
 struct Prof {
@@ -232,6 +239,7 @@ struct Ctx {
   AmrHost amr;
   Prof prof;
   LimTabs lim;
+  LdfLeg ldf_leg;
   MlpTabs mlp;
   void* mlp_w1 = nullptr;     // bf16 [64][kp]
   void* mlp_w2 = nullptr;     // bf16 [64][64]

@@ -1,5 +1,7 @@
 // Kernels of the CUDA-core DG-MHD path (FP64 plain form and the FP32 form).
 #pragma once
+#include <vector>
+
 #include "dg_ctx.h"
 
 namespace dgmhd {
@@ -18,6 +20,8 @@ void launch_cell(const Geom& g, const Tables<T>& tb, const T* w, const T* fbuf, 
 // 3D, one axis at a time (dg_project.cu); ldf: the LDF map and 1 / mass (Powell)
 bool project_sf_ok(const Geom& g, int npts);
 bool ldf_pattern_ok(int degree, const double* A);
+// the LDF -> Legendre map of a 3D basis (dg_api.cu), A[(j * 3 + c) * n + l]
+bool ldf_legendre_3d(const Basis& L, int deg, std::vector<double>& A);
 template <typename T>
 void launch_project_sf(const Geom& g, int npts, const double* nodal, const double* ldf, T* w, double* wmean,
                        cudaStream_t st);

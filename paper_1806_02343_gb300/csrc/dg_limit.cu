@@ -23,6 +23,7 @@
 #include <cstring>
 #include <vector>
 
+#include "dg_kernels.cuh"
 #include "dg_limit.cuh"
 #include "dg_pos.cuh"
 #include "dg_mlp.cuh"
@@ -740,15 +741,24 @@ __global__ void k_pos(Geom g, Tables<T> tb, LimTabs lt, T* w, double* wmean, dg_
 }
 
 // FP32 form, 3D degrees 1-2: the positivity procedure of pos_cell on the
-// listed cells. A warp takes 32 list entries: each lane stages its cell's rows
-// (coalesced where the listed cells are neighbours), applies the mean floors
-// and the rigorous screen; the cells that stay open are then done one at a
-// time by the whole warp, lanes over the volume and face points, the limiting
-// factors being warp minima. Every point value is accumulated in the same
-// order as in pos_cell, so the two agree bit for bit.
+// listed cells. A warp takes up to 32 list entries at a time: each lane stages
+// its cell's rows (coalesced where the listed cells are neighbours) and screens
+// its points in FP32 (pos_points_clear); the few cells that leaves get the mean
+// floors and the rigorous screen, and those still open are done one at a time by
+// the whole warp, lanes over the volume and face points, the limiting factors
+// being warp minima. Every point value is accumulated in the same order as in
+// pos_cell, so the two agree bit for bit. A short list is spread over the
+// launch's warps, one cell per warp, instead of 32.
+// What bounded it: every open cell cost its warp about 45 FP64 instructions
+// (conversions and warp minima, 16 cycles of the SM each) although hardly any
+// needs its FP64 pressures -- 86% of the cells of a Mach-1.5 flow are listed and
+// none limited -- and the lists of a blast filled only 131 warps. Measured per
+// pass: flow, 436,000 of 504,000 cells listed, 1.69 ms; 256^3 turbulence,
+// 415,000 listed, 1.60 ms; 128^3 Powell blast, 4,000 listed, 0.69 ms.
 template <int DEG, int GLMF>
-__global__ void __launch_bounds__(128) k_pos_list(Geom gin, Tables<float> tb, LimTabs lt, float* w, double* wmean,
-                                                  dg_mhd_params p, DevScalars* sc, const int32_t* __restrict__ list) {
+__global__ void __launch_bounds__(128) k_pos_list(Geom gin, Tables<float> tb, LimTabs lt, LdfLeg ll, float* w,
+                                                  double* wmean, dg_mhd_params p, DevScalars* sc,
+                                                  const int32_t* __restrict__ list) {
   const Geom g = pin_geom<DEG, GLMF>(gin);
   constexpr int N = (DEG + 1) * (DEG + 2) * (DEG + 3) / 6;
   constexpr int NR = GLMF ? 9 * N : 5 * N + (DEG == 1 ? 11 : 26);
@@ -772,9 +782,12 @@ __global__ void __launch_bounds__(128) k_pos_list(Geom gin, Tables<float> tb, Li
   };
   const int64_t total = (int64_t)sc->npos;
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&sc->cnt_poslisted, (unsigned long long)total);
-  for (int64_t i0 = ((int64_t)blockIdx.x * 4 + warp) * 32; i0 < total; i0 += (int64_t)gridDim.x * 4 * 32) {
-    const bool valid = i0 + lane < total;
-    const int64_t c = valid ? (int64_t)list[i0 + lane] : 0;
+  // entries per warp and turn
+  const int64_t nwarp = (int64_t)gridDim.x * 4;
+  const int grp = (int)(total >= 32 * nwarp ? 32 : (total + nwarp - 1) / nwarp);
+  for (int64_t i0 = ((int64_t)blockIdx.x * 4 + warp) * grp; i0 < total; i0 += nwarp * grp) {
+    const bool listed = lane < grp && i0 + lane < total;
+    const int64_t c = listed ? (int64_t)list[i0 + lane] : 0;
     __syncwarp();  // the previous group's reads of R are done
     double mr[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, m[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     double pmean = 0.0;
@@ -782,9 +795,41 @@ __global__ void __launch_bounds__(128) k_pos_list(Geom gin, Tables<float> tb, Li
     // per variable, sum of |coefficients| beyond the mean (x |basis| bound): with
     // |mean|, the scale of every point value, which bounds its FP32 rounding
     float devt[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (valid) {
+    bool valid = listed;
+    if (listed) {
 #pragma unroll
       for (int r = 0; r < NR; ++r) R[r][lane] = w[(int64_t)r * S + c];
+      const int nlg = g.glm ? 8 : 5;
+#pragma unroll
+      for (int v = 0; v < 8; ++v) {
+        if (v >= nlg) continue;
+        for (int l = 1; l < g.n; ++l) devt[v] += fabsf(R[v * g.n + l][lane]);
+      }
+      if (!g.glm)
+        for (int j = g.D; j < g.ndiv; ++j) {
+          const float aj = fabsf(R[g.ldf0 + j][lane]);
+#pragma unroll
+          for (int cc = 0; cc < 3; ++cc) devt[5 + cc] += aj * (float)lt.ldf_maxabs[j * 3 + cc];
+        }
+      auto coef = [&](auto VI, int i, int j, int k) -> float {
+        constexpr int v = decltype(VI)::value;
+        const int l = sf::mode_idx(i, j, k);
+        if constexpr (GLMF || v < 5) {
+          return R[v * N + l][lane];
+        } else {
+          float x = 0.f;
+#pragma unroll
+          for (int q = 0; q < LdfPattern<DEG>::NDIV; ++q)
+            if (ldf_has<DEG>(q, v - 5, l)) x = fmaf(R[5 * N + q][lane], ll.A[(q * 3 + v - 5) * N + l], x);
+          return x;
+        }
+      };
+      float mt[8];
+      sf::each<0, 8>([&](auto VI) { mt[decltype(VI)::value] = coef(VI, 0, 0, 0); });
+      valid = !pos_points_clear<DEG>(coef, mt, devt, (float)p.eps_rho, (float)p.eps_p, gm1t);
+    }
+    if (!__any_sync(0xffffffffu, valid)) continue;
+    if (valid) {
       for (int k = 0; k < nm; ++k) mr[k] = wmean[k * S + c];
       // physical mean state and the mean floors
       for (int k = 0; k < 5; ++k) m[k] = mr[k];
@@ -817,18 +862,6 @@ __global__ void __launch_bounds__(128) k_pos_list(Geom gin, Tables<float> tb, Li
       }
       pmean = pres(m);
       // the rigorous screen of pos_cell
-      const int nlg = g.glm ? 8 : 5;
-#pragma unroll
-      for (int v = 0; v < 8; ++v) {
-        if (v >= nlg) continue;
-        for (int l = 1; l < g.n; ++l) devt[v] += fabsf(R[v * g.n + l][lane]);
-      }
-      if (!g.glm)
-        for (int j = g.D; j < g.ndiv; ++j) {
-          const float aj = fabsf(R[g.ldf0 + j][lane]);
-#pragma unroll
-          for (int cc = 0; cc < 3; ++cc) devt[5 + cc] += aj * (float)lt.ldf_maxabs[j * 3 + cc];
-        }
       double dev[8];
       for (int v = 0; v < 8; ++v) dev[v] = (double)devt[v] * (1.0 + 1e-5) + 1e-5 * fabs(m[v]);
       open = true;
@@ -1001,6 +1034,16 @@ int upload_limiter_tables(Ctx& c) {
     lt.ldf_pl_f[i] = (float)lt.ldf_pl[i];
   }
   c.lim = lt;
+  // the LDF map of the point-wise screen (3D degrees 1 and 2)
+  std::memset(&c.ldf_leg, 0, sizeof(c.ldf_leg));
+  c.ldf_leg.ok = 1;
+  if (!g.glm && pinned_sizes_ok(g)) {
+    std::vector<double> A;
+    if (ldf_legendre_3d(B, g.d, A) && ldf_pattern_ok(g.d, A.data()))
+      for (size_t i = 0; i < A.size(); ++i) c.ldf_leg.A[i] = (float)A[i];
+    else
+      c.ldf_leg.ok = 0;
+  }
   PosScreen& ps = c.pscr;
   std::memset(&ps, 0, sizeof(ps));
   for (int i = 0; i < 9; ++i) ps.ldf_mean0[i] = (float)lt.ldf_mean0[i];
@@ -1066,9 +1109,9 @@ int run_limiter(Ctx& c, void* w, double* wmean, uint8_t* troubled, cudaStream_t 
         else g.glm ? scr(k_pos_screen<1, 1>) : scr(k_pos_screen<1, 0>);
       }
       const unsigned nbl = (unsigned)std::min<int64_t>(nb, (int64_t)c.nsm * 16);
-      auto pw = [&](auto k) { k<<<(unsigned)c.nsm * 8, 128, 0, st>>>(g, c.t32, c.lim, (float*)w, wmean, c.p, c.sc,
-                                                                    c.pos_list); };
-      if (!pinned_sizes_ok(g) || !wmean)
+      auto pw = [&](auto k) { k<<<(unsigned)c.nsm * 8, 128, 0, st>>>(g, c.t32, c.lim, c.ldf_leg, (float*)w, wmean, c.p,
+                                                                    c.sc, c.pos_list); };
+      if (!pinned_sizes_ok(g) || !wmean || !c.ldf_leg.ok)
         k_pos<float><<<nbl, 128, 0, st>>>(g, c.t32, c.lim, (float*)w, wmean, c.p, c.sc, c.pos_list);
       else if (g.d == 2) g.glm ? pw(k_pos_list<2, 1>) : pw(k_pos_list<2, 0>);
       else g.glm ? pw(k_pos_list<1, 1>) : pw(k_pos_list<1, 0>);

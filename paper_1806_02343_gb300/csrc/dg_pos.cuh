@@ -3,6 +3,8 @@
 // in shared memory already.
 #pragma once
 #include "dg_ctx.h"
+#include "dg_ldf.cuh"
+#include "dg_sf.cuh"
 
 namespace dgmhd {
 
@@ -67,6 +69,92 @@ __device__ __forceinline__ bool pos_screen_rows(const Geom& g, const PosScreen& 
     if (plo > ps.eps_p * 2.f + mg * fabsf(mt[4])) return true;
   }
   return false;
+}
+
+// Point-wise screen in FP32, 3D degrees 1 and 2: the state at every volume and
+// face point of the cell, one axis at a time (planes of z, rows of y, points of
+// x; on a plane or row through the cell's faces only the points that exist).
+// True: the density clears its floor and the pressure of every point and of the
+// mean clears its floor by more than the rounding, so the positivity procedure
+// leaves the cell as it is. With S_v = |mean_v| + dev_v (dev: sum of
+// |coefficients| x basis bound) every value carries at most about 30 roundings,
+// 2e-6 S_v; a point is cleared with rho >= 0.1 S_rho and
+//   rho (E - B^2/2 - eps_p/(g-1) - t (S_E + S_B^2/2)) >= m^2/2 + t S_m^2/2,
+// t = 1e-4: at least four times what those roundings can move either side.
+// A non-finite value clears nothing. coef(v, l): Legendre coefficient l of
+// variable v (v < 8).
+template <int DEG, typename Coef>
+__device__ __forceinline__ bool pos_points_clear(Coef coef, const float (&mt)[8], const float (&dv)[8], float eps_rho,
+                                                 float eps_p, float gm1) {
+  constexpr int NQ = DEG + 1, NX = NQ + 2, M2 = sf::n_modes2(DEG);
+  constexpr float t = 1e-4f;
+  float S[8];
+#pragma unroll
+  for (int v = 0; v < 8; ++v) S[v] = fabsf(mt[v]) + dv[v];
+  const float c1 = eps_p / gm1 + t * (S[4] + 0.5f * (S[5] * S[5] + S[6] * S[6] + S[7] * S[7]));
+  const float c2 = 0.5f * t * (S[1] * S[1] + S[2] * S[2] + S[3] * S[3]);
+  const float r0 = fmaxf(eps_rho + t * S[0], 0.1f * S[0]);
+  bool ok = true;
+  auto test = [&](const float (&u)[8]) {
+    const float b2 = u[5] * u[5] + u[6] * u[6] + u[7] * u[7], m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
+    const float e = u[4] - 0.5f * b2 - c1;
+    ok = ok && u[0] >= r0 && u[0] * e - 0.5f * m2 >= c2;
+  };
+  test(mt);
+  auto node = [](int i) {  // -1, the Gauss points, +1
+    constexpr float a = (float)sf::Rule<DEG>::x(0);
+    return i == 0 ? -1.f : i == NX - 1 ? 1.f : i == 1 ? -a : i == NX - 2 ? a : 0.f;
+  };
+#pragma unroll 1
+  for (int iz = 0; iz < NX; ++iz) {
+    const float z = node(iz), z2 = 1.5f * z * z - 0.5f;
+    const bool zin = iz > 0 && iz < NX - 1;
+    float g[8][M2];
+    sf::each<0, 8>([&](auto VI) {
+      constexpr int v = decltype(VI)::value;
+#pragma unroll
+      for (int i = 0; i <= DEG; ++i)
+#pragma unroll
+        for (int j = 0; i + j <= DEG; ++j) {
+          float x = coef(VI, i, j, 0);
+          if (i + j + 1 <= DEG) x = fmaf(coef(VI, i, j, 1), z, x);
+          if (i + j + 2 <= DEG) x = fmaf(coef(VI, i, j, 2), z2, x);
+          g[v][sf::mode2_idx<DEG>(i, j)] = x;
+        }
+    });
+#pragma unroll 1
+    for (int iy = zin ? 0 : 1; iy < (zin ? NX : NX - 1); ++iy) {
+      const float yy = node(iy), y2 = 1.5f * yy * yy - 0.5f;
+      const bool in = zin && iy > 0 && iy < NX - 1;
+      float h[8][DEG + 1];
+#pragma unroll
+      for (int v = 0; v < 8; ++v)
+#pragma unroll
+        for (int i = 0; i <= DEG; ++i) {
+          float x = g[v][sf::mode2_idx<DEG>(i, 0)];
+          if (i + 1 <= DEG) x = fmaf(g[v][sf::mode2_idx<DEG>(i, 1)], yy, x);
+          if (i + 2 <= DEG) x = fmaf(g[v][sf::mode2_idx<DEG>(i, 2)], y2, x);
+          h[v][i] = x;
+        }
+      auto point = [&](float x) {
+        const float x2 = 1.5f * x * x - 0.5f;
+        float u[8];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+          u[v] = fmaf(h[v][1], x, h[v][0]);
+          if (DEG >= 2) u[v] = fmaf(h[v][DEG >= 2 ? 2 : 0], x2, u[v]);
+        }
+        test(u);
+      };
+#pragma unroll
+      for (int ix = 1; ix < NX - 1; ++ix) point(node(ix));
+      if (in) {
+        point(-1.f);
+        point(1.f);
+      }
+    }
+  }
+  return ok;
 }
 
 // ballot compaction of a warp's cells into list[0 .. *count)
