@@ -599,6 +599,43 @@ int build_amr(Ctx& c, const dg_mesh_desc* mesh) {
       octree_faces(D, N, mesh->level, mesh->ijk, mi, fL, fR, fmeta, cstart, centry, maxent, mesh->partial != 0);
   if (ef) return ef;
   c.amr.partial = mesh->partial != 0;
+  // specialised Powell kernels: faces renumbered by type (axis; same level, or
+  // the left or right side coarse with sub-face s) in blocks of 32 faces of one
+  // type, the last block of a type padded with faces that no cell lists. Face
+  // f is lane f % 32 of block f / 32 of the face pass, so that pass writes its
+  // fluxes coalesced and consecutive leaves of the cell pass, whose faces of one
+  // type are mostly consecutive, read them coalesced. (The order of a leaf's
+  // entries is unchanged.)
+  const bool fast = !g.glm && D == 3 && (g.d == 1 || g.d == 2) && c.p.generic_kernels != 1 && c.p.powell_q != 1;
+  std::vector<int32_t> btype;
+  if (fast) {
+    auto type_of = [](int m) {
+      const int a = m & 3, kind = (m >> 2) & 3, sb = m >> 4;
+      return a * 9 + (kind == 0 ? 0 : kind == 1 ? 1 + sb : 5 + sb);
+    };
+    const size_t nf0 = fL.size();
+    int64_t cnt[27] = {0}, at[27];
+    for (size_t f = 0; f < nf0; ++f) ++cnt[type_of(fmeta[f])];
+    for (int ty = 0; ty < 27; ++ty) {
+      at[ty] = (int64_t)btype.size() * 32;
+      for (int64_t k = 0; k < cnt[ty]; k += 32)
+        btype.push_back(ty | (int32_t)(std::min<int64_t>(32, cnt[ty] - k) << 8));
+    }
+    if (btype.size() * 32 > (size_t)INT32_MAX / 2) return DG_E_MESH;  // entries are face << 1 | side
+    std::vector<int32_t> pos(nf0);
+    std::vector<int32_t> L(btype.size() * 32, 0), R(btype.size() * 32, 0), M(btype.size() * 32, 0);
+    for (size_t f = 0; f < nf0; ++f) {
+      const int64_t q = at[type_of(fmeta[f])]++;
+      pos[f] = (int32_t)q;
+      L[q] = fL[f];
+      R[q] = fR[f];
+      M[q] = fmeta[f];
+    }
+    for (int32_t& e : centry) e = (pos[e >> 1] << 1) | (e & 1);
+    fL.swap(L);
+    fR.swap(R);
+    fmeta.swap(M);
+  }
   const int64_t nf = (int64_t)fL.size();
   std::vector<double> dxc(N);
   for (int64_t cidx = 0; cidx < N; ++cidx) dxc[cidx] = mesh->box_len / (double)(1ll << mesh->level[cidx]);
@@ -683,26 +720,10 @@ int build_amr(Ctx& c, const dg_mesh_desc* mesh) {
     int e3;
     if ((e3 = upload_vec(&h.side_nb, snb)) || (e3 = upload_vec(&h.side_info, sinf))) return e3;
   }
-  // specialised Powell kernels: faces grouped by type in blocks of <= 32, and
-  // the tables of each type (the std tables: the full face; coarse sides: the
-  // sub-face tables Ps above)
-  if (!g.glm && D == 3 && (g.d == 1 || g.d == 2) && c.p.generic_kernels != 1 && c.p.powell_q != 1) {
+  // the specialised Powell kernels' tables of each type (the std tables: the
+  // full face; coarse sides: the sub-face tables Ps above)
+  if (fast) {
     const int n = g.n, Qf = g.Qf, QFP = Qf + (Qf & 1);
-    std::vector<std::vector<int32_t>> by_type(27);
-    for (int64_t f = 0; f < nf; ++f) {
-      const int m = fmeta[f], a = m & 3, kind = (m >> 2) & 3, sb = m >> 4;
-      by_type[a * 9 + (kind == 0 ? 0 : kind == 1 ? 1 + sb : 5 + sb)].push_back((int32_t)f);
-    }
-    std::vector<int32_t> bface, bstart, btype;
-    bface.reserve(nf);
-    for (int ty = 0; ty < 27; ++ty) {
-      const auto& L = by_type[ty];
-      for (size_t k = 0; k < L.size(); k += 32) {
-        bstart.push_back((int32_t)(bface.size() + k));
-        btype.push_back(ty | (int32_t)(std::min<size_t>(32, L.size() - k) << 8));
-      }
-      bface.insert(bface.end(), L.begin(), L.end());
-    }
     // Legendre values on the full face f (its tangential axes in increasing
     // order, the last fastest), and face_val: full face (sb < 0) or sub-face sb
     std::vector<double> Pfull((size_t)2 * D * n * Qf);
@@ -769,8 +790,7 @@ int build_amr(Ctx& c, const dg_mesh_desc* mesh) {
         for (int l = 0; l < n; ++l)
           ctab[((size_t)t * Qf + p) * n + l] = face_val(f, sb, l, p) * wf[p] * (sb < 0 ? 1.0 : 1.0 / nsub);
     }
-    if ((e = upload_vec(&h.bface, bface)) || (e = upload_vec(&h.bstart, bstart)) || (e = upload_vec(&h.btype, btype)))
-      return e;
+    if ((e = upload_vec(&h.btype, btype))) return e;
     if (c.p.precision == DG_PREC_FP32MIX) {
       std::vector<float> a(ftab.begin(), ftab.end()), b(ctab.begin(), ctab.end()), nt(ntab.begin(), ntab.end());
       if ((e = upload_vec((float**)&h.ftab, a)) || (e = upload_vec((float**)&h.ctab, b)) ||
@@ -789,14 +809,12 @@ int build_amr(Ctx& c, const dg_mesh_desc* mesh) {
 
 OctPow<float> oct_pow32(const Ctx& c) {
   const AmrHost& h = c.amr;
-  return OctPow<float>{h.fL, h.fR, h.fmeta, h.cstart, h.centry, h.dxc, h.bface, h.bstart, h.btype,
-                       (const float*)h.ftab, (const float*)h.ctab, (const float*)h.ntab, c.g.ncell, c.g.stride,
+  return OctPow<float>{h.fL, h.fR, h.cstart, h.centry, h.dxc, h.btype, (const float*)h.ftab, (const float*)h.ctab, (const float*)h.ntab, c.g.ncell, c.g.stride,
                        h.nblk};
 }
 OctPow<double> oct_pow64(const Ctx& c) {
   const AmrHost& h = c.amr;
-  return OctPow<double>{h.fL, h.fR, h.fmeta, h.cstart, h.centry, h.dxc, h.bface, h.bstart, h.btype,
-                        (const double*)h.ftab, (const double*)h.ctab, (const double*)h.ntab, c.g.ncell,
+  return OctPow<double>{h.fL, h.fR, h.cstart, h.centry, h.dxc, h.btype, (const double*)h.ftab, (const double*)h.ctab, (const double*)h.ntab, c.g.ncell,
                         c.g.stride, h.nblk};
 }
 
@@ -804,7 +822,7 @@ void free_amr(Ctx& c) {
   AmrHost& h = c.amr;
   void* ptrs[] = {h.fL,     h.fR,     h.fmeta,    h.cstart,   h.centry,   h.dxc,    h.Psub64, h.Lsub64,
                   h.Psub32, h.Lsub32, h.Psub64p, h.Lsub64p, h.Psub32p, h.Lsub32p, h.groups, h.lev_dev,
-                  h.bface,  h.bstart, h.btype,    h.ftab,     h.ctab,     h.ntab,     h.side_nb, h.side_info};
+                  h.btype,  h.ftab,     h.ctab,     h.ntab,     h.side_nb, h.side_info};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   h = AmrHost();

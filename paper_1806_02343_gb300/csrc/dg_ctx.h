@@ -216,10 +216,11 @@ struct AmrHost {
   std::vector<int32_t> hgroups;
   int32_t* groups = nullptr;
   int8_t* lev_dev = nullptr;
-  // specialised Powell kernels (3D, degrees 1 and 2): face blocks by type and
-  // the trace / own-side tables in the context's precision (OctPow)
+  // specialised Powell kernels (3D, degrees 1 and 2): the faces are numbered in
+  // blocks of 32 of one type (btype), and the trace / own-side tables are in the
+  // context's precision (OctPow)
   bool fast = false;
-  int32_t *bface = nullptr, *bstart = nullptr, *btype = nullptr;
+  int32_t* btype = nullptr;
   int64_t nblk = 0;
   void* ftab = nullptr;
   void* ctab = nullptr;

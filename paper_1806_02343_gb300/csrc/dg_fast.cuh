@@ -133,25 +133,21 @@ template <typename T, int DEG>
 void launch_cell_pow(const FastAll<T, DEG>& tabs, const FastGeom& g, const T* w, const T* F, T* out, const T* w0,
                      double ca, double cb, int combine, const DevScalars* sc, const double* wmean,
                      const double* w0mean, double* outmean, cudaStream_t st);
-// Octree meshes (Powell / LDF): the face list of the generic octree kernels
-// plus the face blocks of the specialised pass -- bface lists the faces
-// grouped by type (axis a, same level / left coarse / right coarse, sub-face),
-// block b takes bface[bstart[b] ..] with btype[b] = type | count << 8 (count
-// <= 32, type = 9 a + (0 | 1 + sub | 5 + sub)); ftab[type][side][N][QFP] the
-// trace tables of the two sides (side 0: the left cell) and
-// ctab[30][QF][N] the own-side weighted face tables of the cell pass (0..5:
-// the faces, 6 + 4 f + sub: sub-face sub of face f of a coarse cell, weights
-// w_p / 4).
+// Octree meshes (Powell / LDF): faces in blocks of 32 of one type: face f is
+// lane f % 32 of block f / 32, btype[block] = type | count << 8 (count <= 32
+// faces; the rest of a block is padding), type = 9 a + (0: same level | 1 + sub:
+// left side coarse | 5 + sub: right side coarse). Face buffer
+// F[block][point][slot][32]. ftab[type][side][N][QFP]: the trace tables of the
+// two sides (side 0: the left cell); ctab[30][QF][N]: the own-side weighted face
+// tables of the cell pass (0..5: the faces, 6 + 4 f + sub: sub-face sub of face
+// f of a coarse cell, weights w_p / 4).
 template <typename T>
 struct OctPow {
   const int32_t* fL;
   const int32_t* fR;
-  const int32_t* fmeta;
   const int32_t* cstart;
-  const int32_t* centry;
+  const int32_t* centry;  // face << 1 | side
   const double* dxc;
-  const int32_t* bface;
-  const int32_t* bstart;
   const int32_t* btype;
   const T* ftab;
   const T* ctab;
