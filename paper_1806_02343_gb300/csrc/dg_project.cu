@@ -98,7 +98,8 @@ __global__ void __launch_bounds__(NTJ) k_project_sf(Geom g, const double* __rest
           constexpr int cc = decltype(I)::value / N, l = decltype(I)::value % N;
           if constexpr (ldf_has<DEG>(j, cc, l)) s = __fma_rn(RL[cc * N + l][lane], __ldg(ldf + (j * 3 + cc) * N + l), s);
         });
-        put(5 * N + j, j < 3 ? 5 + j : -1, s * __ldg(ldf + NDIV * 3 * N + j));
+        // 1 / mass in the working precision, as in the operator's tables (and the dense projection)
+        put(5 * N + j, j < 3 ? 5 + j : -1, s * (double)(T)__ldg(ldf + NDIV * 3 * N + j));
       }
     });
   }
