@@ -806,10 +806,10 @@ int dg_mhd_project(dg_mhd_ctx* ctx, const double* nodal, int npts, void* w, doub
   Ctx& c = ctx->c;
   const Geom& g = c.g;
   if (fp32(c) && !wmean) return DG_E_ARG;
-  if (project_sf_ok(g, npts) && (g.glm || project_ldf(c))) {
+  const bool rows = project_rows_ok(g) && c.p.generic_kernels != 1 && (g.glm || project_ldf(c));
+  if (rows && fp32(c) && project_sf_ok(g, npts)) {
     c.prof.launches[4] += 1;
-    if (fp32(c)) launch_project_sf<float>(g, npts, nodal, c.proj_ldf, (float*)w, wmean, S(stream));
-    else launch_project_sf<double>(g, npts, nodal, c.proj_ldf, (double*)w, nullptr, S(stream));
+    launch_project_sf(g, npts, nodal, c.proj_ldf, (float*)w, wmean, S(stream));
     return cudaGetLastError() == cudaSuccess ? DG_OK : DG_E_CUDA;
   }
   if (npts != c.proj_npts) {
@@ -845,7 +845,11 @@ int dg_mhd_project(dg_mhd_ctx* ctx, const double* nodal, int npts, void* w, doub
     c.proj_npts = npts;
   }
   c.prof.launches[4] += 1;
-  if (fp32(c))
+  if (rows && fp32(c))
+    launch_project_rows<float>(g, npts, c.proj_tab, c.proj_w, nodal, c.t32.minv, (float*)w, wmean, S(stream));
+  else if (rows)
+    launch_project_rows<double>(g, npts, c.proj_tab, c.proj_w, nodal, c.t64.minv, (double*)w, nullptr, S(stream));
+  else if (fp32(c))
     launch_project<float>(g, npts, c.proj_tab, c.proj_w, nodal, c.t32.minv, (float*)w, wmean, S(stream));
   else
     launch_project<double>(g, npts, c.proj_tab, c.proj_w, nodal, c.t64.minv, (double*)w, nullptr, S(stream));

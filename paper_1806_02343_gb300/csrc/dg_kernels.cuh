@@ -17,14 +17,18 @@ template <typename T>
 void launch_cell(const Geom& g, const Tables<T>& tb, const T* w, const T* fbuf, T* out, const T* w0,
                  double ca, double cb, int combine, const DevScalars* sc, const double* wmean,
                  const double* w0mean, double* outmean, cudaStream_t st, const T* qbuf = nullptr);
-// 3D, one axis at a time (dg_project.cu); ldf: the LDF map and 1 / mass (Powell)
+// 3D (dg_project.cu): one axis at a time (FP32 form; ldf: the LDF map and
+// 1 / mass, Powell), and dense with the rows of a variable per warp
 bool project_sf_ok(const Geom& g, int npts);
+bool project_rows_ok(const Geom& g);
 bool ldf_pattern_ok(int degree, const double* A);
 // the LDF -> Legendre map of a 3D basis (dg_api.cu), A[(j * 3 + c) * n + l]
 bool ldf_legendre_3d(const Basis& L, int deg, std::vector<double>& A);
-template <typename T>
-void launch_project_sf(const Geom& g, int npts, const double* nodal, const double* ldf, T* w, double* wmean,
+void launch_project_sf(const Geom& g, int npts, const double* nodal, const double* ldf, float* w, double* wmean,
                        cudaStream_t st);
+template <typename T>
+void launch_project_rows(const Geom& g, int npts, const double* tab, const double* wq, const double* nodal,
+                         const T* minv, T* w, double* wmean, cudaStream_t st);
 template <typename T>
 void launch_project(const Geom& g, int npts, const double* tab, const double* wq, const double* nodal,
                     const T* minv, T* w, double* wmean, cudaStream_t st);
