@@ -999,7 +999,8 @@ __device__ __forceinline__ void face_trace_smem(const T (&wl)[FastDims<DEG>::N],
 }
 
 template <typename T, int DEG, int A>
-__device__ __forceinline__ void list_hlld(const T* TRC, int v, int f, bool live, T gamma, T eps, T* __restrict__ F) {
+__device__ __forceinline__ void list_hlld(const T* TRC, int v, int f, bool live, int64_t fid, T gamma, T eps,
+                                          T* __restrict__ F) {
   constexpr int QF = FastDims<DEG>::QF;
   for (int p = v; p < QF; p += 9) {
     T uL[9], uR[9], Fo[9];
@@ -1011,7 +1012,7 @@ __device__ __forceinline__ void list_hlld(const T* TRC, int v, int f, bool live,
     uL[8] = uR[8] = T(0);
     const T bnF = face_flux(uL, uR, A, gamma, false, T(0), eps, Fo);
     if (live) {
-      T* q = F + ((int64_t)blockIdx.x * QF + p) * NFS * TC + f;
+      T* q = F + ((fid >> 5) * QF + p) * NFS * TC + (fid & 31);
 #pragma unroll
       for (int k = 0; k < 8; ++k) q[k * TC] = Fo[k];
       q[8 * TC] = bnF - uL[5 + A];
@@ -1039,7 +1040,12 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && DEG <= 2) ? 4 : 2) k_fa
   const int type = bt & 255, cnt = bt >> 8;
   const int A = type / 9;
   const bool live = f < cnt;
-  const int64_t fid = (int64_t)blockIdx.x * TC + f;
+  // face number, opaque to the compiler: known to be linear in the block and
+  // lane, it led to other multiply-add contractions in the flux (the FP32 form's
+  // means then moved by up to 9e-10 in one step)
+  int face = (int)blockIdx.x * TC + f;
+  asm volatile("" : "+r"(face));
+  const int64_t fid = face;
   const int64_t cL = live ? o.fL[fid] : 0, cR = live ? o.fR[fid] : 0;
   const int64_t S = o.stride;
   for (int i = t; i < 2 * N * QFP; i += NT) TT[i] = o.ftab[(size_t)type * 2 * N * QFP + i];
@@ -1080,9 +1086,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && DEG <= 2) ? 4 : 2) k_fa
     }
   }
   __syncthreads();
-  if (A == 0) list_hlld<T, DEG, 0>(TRC, v, f, live, gamma, eps, F);
-  else if (A == 1) list_hlld<T, DEG, 1>(TRC, v, f, live, gamma, eps, F);
-  else list_hlld<T, DEG, 2>(TRC, v, f, live, gamma, eps, F);
+  if (A == 0) list_hlld<T, DEG, 0>(TRC, v, f, live, fid, gamma, eps, F);
+  else if (A == 1) list_hlld<T, DEG, 1>(TRC, v, f, live, fid, gamma, eps, F);
+  else list_hlld<T, DEG, 2>(TRC, v, f, live, fid, gamma, eps, F);
 }
 
 template <typename T, int DEG>
