@@ -600,7 +600,7 @@ void dg_mhd_destroy(dg_mhd_ctx* ctx) {
   free_tables(c.t32);
   void* ptrs[] = {c.sc, c.face_buf, c.face_buf32, c.stage_buf[0], c.stage_buf[1], c.stage_buf[2],
                   c.stage_mean[0], c.stage_mean[1], c.stage_mean[2], c.cellscratch, c.proj_tab, c.proj_w, c.proj_ldf,
-                  c.troubled, c.flag_list, c.pos_list, c.mlp_w1, c.mlp_w2, c.mlp_bias, c.rg_tabs, c.qdag_buf,
+                  c.troubled, c.flag_list, c.tvb_list, c.pos_list, c.mlp_w1, c.mlp_w2, c.mlp_bias, c.rg_tabs, c.qdag_buf,
                   c.tc_tabs, c.owned};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -712,6 +712,7 @@ int dg_mhd_init(const dg_mesh_desc* mesh, int degree, int divB_scheme, double ga
             cudaMalloc(&c.stage_buf[1], state_bytes) == cudaSuccess &&
             cudaMalloc(&c.troubled, (size_t)g.stride) == cudaSuccess &&
             cudaMalloc(&c.flag_list, (size_t)g.stride * sizeof(int32_t)) == cudaSuccess &&
+            cudaMalloc(&c.tvb_list, (size_t)g.stride * sizeof(int32_t)) == cudaSuccess &&
             cudaMalloc(&c.pos_list, (size_t)g.stride * sizeof(int32_t)) == cudaSuccess;
   {
     int dev = 0, nsm = 0;

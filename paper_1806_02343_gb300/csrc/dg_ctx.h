@@ -114,6 +114,7 @@ struct DevScalars {
   unsigned long long pos_cells;  // cells the positivity limiter rescaled (tau < 1)
   unsigned int nflag;            // cells the indicator flagged in the current limiter pass
   unsigned int npos;             // cells the FP32 positivity screen listed in the current pass
+  unsigned int ntvb;             // cells the TVB procedure could change in the current pass
   unsigned long long cnt_flagged;  // cells flagged by the indicator, summed over passes
   unsigned long long cnt_limited;  // cells whose slopes the TVB procedure changed, summed over passes
   float dt32, ch32, kappa32;       // FP32 copies of dt, ch, kappa (written with them)
@@ -264,6 +265,7 @@ struct Ctx {
   double* proj_ldf = nullptr;      // LDF map of the sum-factorised projection (dg_project.cu)
   uint8_t* troubled = nullptr;     // per-cell limiter flags (scratch)
   int32_t* flag_list = nullptr;    // cells flagged by the indicator in the current pass
+  int32_t* tvb_list = nullptr;     // cells the TVB procedure could change in the current pass
   int32_t* pos_list = nullptr;     // cells the positivity screen could not clear in the current pass
   PosScreen pscr;                  // FP32 positivity screen tables
   double* rg_tabs = nullptr;       // regridding tables (dg_regrid.cu), built on first use

@@ -26,6 +26,7 @@
 #include "dg_kernels.cuh"
 #include "dg_limit.cuh"
 #include "dg_pos.cuh"
+#include "dg_tvb_detect.cuh"
 #include "dg_mlp.cuh"
 
 namespace dgmhd {
@@ -399,13 +400,119 @@ __device__ bool tvb_cell(const Geom& g, const LimTabs& lt, T* w, const double* w
   return true;
 }
 
-// TVB over every cell (list == nullptr: the plain detector) or over the cells
-// the learned indicator listed (list[0 .. sc->nflag)); grid-stride, so any
-// grid covers the work. Counts the cells whose slopes changed.
+// Cells the TVB procedure could change (dg_tvb_detect.cuh), out of every cell
+// (list == nullptr) or of the listed ones (list[0 .. *count)), appended to
+// out[0 .. sc->ntvb). With SCREEN, the other ones take the positivity screen
+// here (their rows stay as they are). Most cells are excluded by their own
+// slopes; the neighbours' means are read for the rest. The procedure on every
+// cell, one thread each with its arrays in local memory, was latency-bound. Per
+// pass, before and now with the procedure on the list: 1,387,520-leaf octree 0.83
+// and 0.06 ms; 48^3 FP64 blast 0.67 and 0.18 ms; 256^3 turbulence, the indicator's
+// list, 0.69 and 0.59 ms.
+template <typename T, bool SCREEN, int DEG, int GLMF>
+__global__ void __launch_bounds__(128) k_tvb_detect(Geom gin, LdfLeg ll, const T* __restrict__ w, float thr0,
+                                                    double mtilde, float beta, DevScalars* sc, AmrNb an,
+                                                    const int32_t* __restrict__ list,
+                                                    const unsigned* __restrict__ count, int32_t* __restrict__ out,
+                                                    int32_t* __restrict__ plist, PosScreen ps) {
+  const Geom g = pin_geom<DEG, GLMF>(gin);
+  constexpr int N = LdfPattern<DEG>::N, NM = GLMF ? 9 : 8;
+  const int64_t total = list ? (int64_t)*count : g.ncell;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  const int64_t S = g.stride;
+  const float gamma = (float)g.gamma;
+  const float ch = GLMF ? sc->ch32 : 0.f;
+  // Legendre coefficient l of B component cc from the LDF rows of cell c
+  auto ldf = [&](int64_t c, auto CC, auto L) {
+    float x = 0.f;
+    sf::each<0, LdfPattern<DEG>::NDIV>([&](auto J) {
+      constexpr int j = decltype(J)::value, cc = decltype(CC)::value, l = decltype(L)::value;
+      if constexpr (ldf_has<DEG>(j, cc, l))
+        x = fmaf((float)w[(int64_t)(5 * N + j) * S + c], ll.A[(j * 3 + cc) * N + l], x);
+    });
+    return x;
+  };
+  auto means = [&](int64_t c, float (&m)[9]) {
+#pragma unroll
+    for (int k = 0; k < NM; ++k)
+      if (GLMF || k < 5) m[k] = (float)w[(int64_t)(k * N) * S + c];
+    if constexpr (!GLMF) {
+      sf::each<0, 3>([&](auto CC) { m[5 + decltype(CC)::value] = ldf(c, CC, std::integral_constant<int, 0>{}); });
+      m[8] = 0.f;
+    }
+  };
+  // warp-uniform trip count (the appends below are warp ballots)
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < total; i0 += step) {
+    const int64_t i = i0 + (threadIdx.x & 31);
+    bool todo = false, fail = false;
+    int64_t c = 0;
+    if (i < total) {
+      c = list ? (int64_t)list[i] : i;
+      const float thr = an.on ? (float)(mtilde * an.dxc[c]) : thr0;
+      float m[9], sls[3][9];  // every load of the cell's own rows is issued before the first use
+      means(c, m);
+      sf::each<0, 3>([&](auto AX) {
+        constexpr int A = decltype(AX)::value;
+#pragma unroll
+        for (int v = 0; v < NM; ++v)
+          if (GLMF || v < 5) sls[A][v] = (float)w[(int64_t)(v * N + 1 + A) * S + c];
+        if constexpr (!GLMF) {
+          sf::each<0, 3>(
+              [&](auto CC) { sls[A][5 + decltype(CC)::value] = ldf(c, CC, std::integral_constant<int, 1 + A>{}); });
+          sls[A][8] = 0.f;
+        }
+      });
+      bool clear = !GLMF || ch > 0.f;  // no c_h yet: the procedure takes B_n and psi as separate fields
+      sf::each<0, 3>([&](auto AX) {
+        constexpr int A = decltype(AX)::value;
+        if (!clear) return;
+        clear = tvb_axis_clear<A, GLMF>(m, sls[A], gamma, ch, thr, beta, [&](float (&dp)[9], float (&dm)[9]) {
+#pragma unroll
+          for (int sd = 0; sd < 2; ++sd) {
+            float mn[9], f = 0.5f;
+            if (!an.on) {
+              means(nb(g, c, A, sd ? 1 : -1), mn);
+            } else {  // the average of the leaves across the side, the centre distance 2, 1.5 or 3
+              const int sidx = 2 * A + sd, inf = an.side_info[c * 6 + sidx];
+              const int cnt = inf & 15, rel = inf >> 4;
+#pragma unroll
+              for (int k = 0; k < 9; ++k) mn[k] = 0.f;
+              for (int q = 0; q < cnt; ++q) {
+                float t[9];
+                means((int64_t)an.side_nb[c * 24 + sidx * 4 + q], t);
+#pragma unroll
+                for (int k = 0; k < NM; ++k) mn[k] += t[k];
+              }
+              const float ic = 1.f / (float)(cnt > 0 ? cnt : 1);
+#pragma unroll
+              for (int k = 0; k < NM; ++k) mn[k] *= ic;
+              if (cnt > 0) f = rel == 0 ? 0.5f : (rel == 1 ? 1.f / 1.5f : 1.f / 3.f);
+            }
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+              const float d = k < NM ? (sd ? mn[k] - m[k] : m[k] - mn[k]) * f : 0.f;
+              (sd ? dp[k] : dm[k]) = d;
+            }
+          }
+        });
+      });
+      todo = !clear;
+      if constexpr (SCREEN)
+        if (clear) fail = !pos_screen_rows(g, ps, [&](int r) { return (float)w[(int64_t)r * S + c]; });
+    }
+    append_cells(todo, c, out, &sc->ntvb);
+    if constexpr (SCREEN) append_cells(fail, c, plist, &sc->npos);
+  }
+}
+
+// TVB over every cell (list == nullptr) or over the listed ones (list[0 ..
+// *count)); grid-stride, so any grid covers the work. Counts the cells whose
+// slopes changed.
 template <typename T, bool SCREEN>
 __global__ void k_tvb(Geom g, LimTabs lt, T* w, double* wmean, uint8_t* troubled, const int32_t* __restrict__ list,
-                      dg_mhd_params p, DevScalars* sc, AmrNb an, int32_t* __restrict__ plist, PosScreen ps) {
-  const int64_t total = list ? (int64_t)sc->nflag : g.ncell;
+                      const unsigned* __restrict__ count, dg_mhd_params p, DevScalars* sc, AmrNb an,
+                      int32_t* __restrict__ plist, PosScreen ps) {
+  const int64_t total = list ? (int64_t)*count : g.ncell;
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
   const int64_t S = g.stride;
@@ -1060,24 +1167,33 @@ int run_limiter(Ctx& c, void* w, double* wmean, uint8_t* troubled, cudaStream_t 
   bool screened = false;  // the positivity screen already ran (indicator: unflagged cells, TVB: flagged ones)
   if (c.p.limiter == DG_LIMIT_TVB || c.p.limiter == DG_LIMIT_MLP) {
     const int32_t* list = nullptr;
+    const unsigned* count = nullptr;
     unsigned nbt = nb;
+    const unsigned nbl = (unsigned)std::min<int64_t>(nb, (int64_t)c.nsm * 16);  // a list's persistent grid
+    const bool f32 = c.p.precision == DG_PREC_FP32MIX;
+    // 3D degrees 1 and 2: the procedure runs on the cells the detector in front
+    // of it cannot exclude. Not for the plain limiter of the FP32 form on uniform
+    // meshes: there the procedure on every cell takes 0.40 ms on 504,000 cells of
+    // a GLM flow, detector and procedure on the list 0.45 ms (a third of the
+    // cells trigger), against 0.83 and 0.10 ms on the 1,387,520-leaf octree.
+    const bool detect = pinned_sizes_ok(g) && c.ldf_leg.ok && (!f32 || c.amr.on || c.p.limiter == DG_LIMIT_MLP);
     ++c.lim_passes;
+    if (troubled && (detect || c.p.limiter == DG_LIMIT_MLP)) cudaMemsetAsync(troubled, 0, (size_t)g.ncell, st);
+    cudaMemsetAsync(&c.sc->nflag, 0, 3 * sizeof(unsigned), st);  // nflag, npos, ntvb
     if (c.p.limiter == DG_LIMIT_MLP) {
       if (!c.mlp_w1) return DG_E_ARG;  // no weights set
       // the indicator appends the cells it flags to flag_list; only those go
       // through the TVB procedure (a persistent grid walks the list)
-      if (troubled) cudaMemsetAsync(troubled, 0, (size_t)g.ncell, st);
-      cudaMemsetAsync(&c.sc->nflag, 0, sizeof(unsigned), st);
       // FP32 form: the indicator's kernel also screens positivity on the rows it stages
-      const bool fuse_pos = c.p.positivity && c.p.precision == DG_PREC_FP32MIX;
-      if (fuse_pos) cudaMemsetAsync(&c.sc->npos, 0, sizeof(unsigned), st);
+      const bool fuse_pos = c.p.positivity && f32;
       c.prof.begin(6, st);
       const int e =
           mlp_infer_launch(c, w, wmean, nullptr, nullptr, st, c.flag_list, fuse_pos ? c.pos_list : nullptr, &screened);
       c.prof.end(6, st);
       if (e) return e;
       list = c.flag_list;
-      nbt = (unsigned)std::min<int64_t>(nb, (int64_t)c.nsm * 16);
+      count = &c.sc->nflag;
+      nbt = nbl;
     } else {
       c.lim_plain_cells += g.ncell;
     }
@@ -1086,13 +1202,32 @@ int run_limiter(Ctx& c, void* w, double* wmean, uint8_t* troubled, cudaStream_t 
     // them avoids FP64 conversions (the limiter never changes the means)
     const AmrNb an{c.amr.fL,  c.amr.fR, c.amr.fmeta, c.amr.cstart, c.amr.centry, c.amr.dxc, c.amr.on ? 1 : 0,
                    c.amr.side_nb, c.amr.side_info};
-    if (c.p.precision == DG_PREC_FP32MIX)
-      screened ? k_tvb<float, true><<<nbt, 128, 0, st>>>(g, c.lim, (float*)w, nullptr, troubled, list, c.p, c.sc,
+    if (detect) {
+      auto run = [&](auto k, auto* x) {
+        k<<<nbt, 128, 0, st>>>(g, c.ldf_leg, x, (float)(c.p.Mtilde * g.dx), c.p.Mtilde, (float)c.p.beta, c.sc, an, list,
+                               count, c.tvb_list, c.pos_list, c.pscr);
+      };
+      auto by_size = [&](auto SCR, auto* x) {
+        using T = std::remove_const_t<std::remove_pointer_t<decltype(x)>>;
+        constexpr bool s = decltype(SCR)::value;
+        if (g.d == 2) g.glm ? run(k_tvb_detect<T, s, 2, 1>, x) : run(k_tvb_detect<T, s, 2, 0>, x);
+        else g.glm ? run(k_tvb_detect<T, s, 1, 1>, x) : run(k_tvb_detect<T, s, 1, 0>, x);
+      };
+      if (!f32) by_size(std::false_type{}, (const double*)w);
+      else if (screened) by_size(std::true_type{}, (const float*)w);
+      else by_size(std::false_type{}, (const float*)w);
+      list = c.tvb_list;
+      count = &c.sc->ntvb;
+      nbt = nbl;
+      c.prof.launches[3] += 1;
+    }
+    if (f32)
+      screened ? k_tvb<float, true><<<nbt, 128, 0, st>>>(g, c.lim, (float*)w, nullptr, troubled, list, count, c.p, c.sc,
                                                           an, c.pos_list, c.pscr)
-               : k_tvb<float, false><<<nbt, 128, 0, st>>>(g, c.lim, (float*)w, nullptr, troubled, list, c.p, c.sc,
+               : k_tvb<float, false><<<nbt, 128, 0, st>>>(g, c.lim, (float*)w, nullptr, troubled, list, count, c.p, c.sc,
                                                            an, nullptr, c.pscr);
     else
-      k_tvb<double, false><<<nbt, 128, 0, st>>>(g, c.lim, (double*)w, nullptr, troubled, list, c.p, c.sc, an,
+      k_tvb<double, false><<<nbt, 128, 0, st>>>(g, c.lim, (double*)w, nullptr, troubled, list, count, c.p, c.sc, an,
                                                 nullptr, c.pscr);
     c.prof.end(3, st);
   }
@@ -1102,7 +1237,7 @@ int run_limiter(Ctx& c, void* w, double* wmean, uint8_t* troubled, cudaStream_t 
       // cheap FP32 screen over every cell; the full procedure only on the few
       // cells it lists (so a warp never waits on one lane's FP64 recovery)
       if (!screened) {
-        cudaMemsetAsync(&c.sc->npos, 0, sizeof(unsigned), st);
+        if (c.p.limiter == DG_LIMIT_OFF) cudaMemsetAsync(&c.sc->npos, 0, sizeof(unsigned), st);
         auto scr = [&](auto k) { k<<<nb, 128, 0, st>>>(g, c.pscr, (const float*)w, c.sc, c.pos_list); };
         if (!pinned_sizes_ok(g)) scr(k_pos_screen<-1, 0>);
         else if (g.d == 2) g.glm ? scr(k_pos_screen<2, 1>) : scr(k_pos_screen<2, 0>);
