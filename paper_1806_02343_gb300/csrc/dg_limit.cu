@@ -836,6 +836,162 @@ __device__ void pos_cell(const Geom& g, const Tables<T>& tb, const LimTabs& lt, 
   }
 }
 
+// FP64, 3D degrees 1 and 2: the cells that neither the rigorous bound nor the
+// point-wise screen clears, both in FP32 on the rounded coefficients (their
+// margins exceed that rounding), appended to list[0 .. sc->npos). The procedure
+// on every cell evaluated the points of each open one in FP64, one thread each:
+// 0.99 ms per pass on the 48^3 Powell blast; this screen 0.03 ms, the list 0.05.
+template <int DEG, int GLMF>
+__global__ void __launch_bounds__(128) k_pos_pre64(Geom gin, PosScreen ps, LdfLeg ll, const double* __restrict__ w,
+                                                   float eps_rho, float eps_p, DevScalars* sc,
+                                                   int32_t* __restrict__ list) {
+  const Geom g = pin_geom<DEG, GLMF>(gin);
+  constexpr int N = LdfPattern<DEG>::N, NDIV = LdfPattern<DEG>::NDIV, NR = GLMF ? 8 * N : 5 * N + NDIV;
+  __shared__ float rows[4][NR][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float(*R)[32] = rows[warp];
+  const int64_t c = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  bool fail = false;
+  if (c < g.ncell) {
+#pragma unroll
+    for (int r = 0; r < NR; ++r) R[r][lane] = (float)w[(int64_t)r * g.stride + c];
+    if (!pos_screen_rows(g, ps, [&](int r) { return R[r][lane]; })) {
+      float dev[8];
+      fail = !pos_points_rows<DEG, GLMF>([&](int r) { return R[r][lane]; }, ll, eps_rho, eps_p, ps, dev);
+    }
+  }
+  append_cells(fail, c, list, &sc->npos);
+}
+
+// The positivity procedure of pos_cell on the cells k_pos_pre64 listed: a warp
+// per cell with its rows in shared memory, lanes over the volume and face points,
+// the limiting factors warp minima; every point value is accumulated in pos_cell's
+// order. One thread per cell was a serial chain of 81 points times 160 dependent
+// multiply-adds at degree 2, 1 ms however short the list.
+template <int DEG, int GLMF>
+__global__ void __launch_bounds__(128) k_pos_list64(Geom gin, Tables<double> tb, double* w, dg_mhd_params p,
+                                                    DevScalars* sc, const int32_t* __restrict__ list) {
+  const Geom g = pin_geom<DEG, GLMF>(gin);
+  constexpr int N = LdfPattern<DEG>::N, NDIV = LdfPattern<DEG>::NDIV, NR = GLMF ? 9 * N : 5 * N + NDIV;
+  constexpr int NL = GLMF ? 8 : 5, NPS = GLMF ? 9 : 5;
+  __shared__ double rows[4][NR];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double* R = rows[warp];
+  const int64_t S = g.stride;
+  const int nm = GLMF ? 9 : 8, npt = g.Qv + 2 * g.D * g.Qf;
+  const double gm1 = g.gamma - 1.0, vol = g.dx * g.dx * g.dx;
+  auto pres = [&](const double* u) {
+    return gm1 * (u[4] - 0.5 * (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) / u[0] -
+                  0.5 * (u[5] * u[5] + u[6] * u[6] + u[7] * u[7]));
+  };
+  auto wmin = [](double v) {
+    for (int o = 16; o; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+  };
+  const int64_t total = (int64_t)sc->npos;
+  for (int64_t i = (int64_t)blockIdx.x * 4 + warp; i < total; i += (int64_t)gridDim.x * 4) {
+    const int64_t c = list[i];
+    __syncwarp();  // the previous cell's reads of R are done
+    for (int r = lane; r < NR; r += 32) R[r] = w[(int64_t)r * S + c];
+    __syncwarp();
+    double mr[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, m[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < NL; ++k) mr[k] = R[k * N];
+    if constexpr (GLMF) mr[8] = R[8 * N];
+    else
+#pragma unroll
+      for (int k = 0; k < 3; ++k) mr[5 + k] = R[5 * N + k];
+    for (int k = 0; k < 5; ++k) m[k] = mr[k];
+    if constexpr (GLMF) {
+      for (int k = 5; k < 9; ++k) m[k] = mr[k];
+    } else {
+      for (int j = 0; j < 3; ++j)
+        for (int cc = 0; cc < 3; ++cc) m[5 + cc] += mr[5 + j] * tb.L0[j * 3 + cc];
+    }
+    // mean floors
+    bool changed_mean = false;
+    if (m[0] < p.eps_rho) {
+      if (lane == 0) atomicAdd(&sc->inj_mass, (p.eps_rho - m[0]) * vol);
+      m[0] = mr[0] = p.eps_rho;
+      changed_mean = true;
+    }
+    const double pm = pres(m);
+    if (pm < p.eps_p) {
+      const double dE = (p.eps_p - pm) / gm1;
+      if (lane == 0) atomicAdd(&sc->inj_energy, dE * vol);
+      m[4] += dE;
+      mr[4] += dE;
+      changed_mean = true;
+    }
+    if (changed_mean && lane == 0) {
+      atomicOr(&sc->floor_used, 1);
+      for (int k = 0; k < nm; ++k) w[(int64_t)lmean_row(g, k) * S + c] = mr[k];
+    }
+    const double pmean = pres(m);
+    double dev[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // unused by the FP64 test of a point
+    // tau_rho over the volume and face points
+    double tau = 1.0;
+    for (int pt = lane; pt < npt; pt += 32) {
+      double acc = 0.0;
+#pragma unroll
+      for (int l = 1; l < N; ++l) acc += R[l] * tb.Pp[l * npt + pt];
+      if (mr[0] + acc < p.eps_rho) {
+        double rd = mr[0];
+        for (int l = 1; l < N; ++l) rd += R[l] * tb.Pp[l * npt + pt];
+        if (rd < p.eps_rho) tau = fmin(tau, (m[0] - p.eps_rho) / (m[0] - rd));
+      }
+    }
+    tau = fmax(wmin(tau), 0.0);
+    // tau_p from the density-limited state m + tau (u - m)
+    double taup = 1.0;
+    for (int pt = lane; pt < npt; pt += 32) {
+      double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll 3
+      for (int l = 1; l < N; ++l) {
+        const double P = tb.Pp[l * npt + pt];
+#pragma unroll
+        for (int v = 0; v < NL; ++v) acc[v] += R[v * N + l] * P;
+      }
+      if constexpr (!GLMF) {
+#pragma unroll 4
+        for (int j = 3; j < NDIV; ++j) {
+          const double wj = R[5 * N + j];
+#pragma unroll
+          for (int cc = 0; cc < 3; ++cc) acc[5 + cc] += wj * tb.Lp[(j * 3 + cc) * npt + pt];
+        }
+      }
+      double uu[8];
+#pragma unroll
+      for (int v = 0; v < 8; ++v) uu[v] = m[v] + tau * acc[v];
+      if (pos_point_open(uu, m, dev, tau, gm1, p.eps_p, 0.0)) {
+        double u[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+        for (int v = 0; v < NPS; ++v) {
+          double sv = mr[v];
+          for (int l = 1; l < N; ++l) sv += R[v * N + l] * tb.Pp[l * npt + pt];
+          u[v] = sv;
+        }
+        if constexpr (!GLMF)
+          for (int j = 0; j < NDIV; ++j) {
+            const double wj = j < 3 ? mr[5 + j] : R[5 * N + j];
+            for (int cc = 0; cc < 3; ++cc) u[5 + cc] += wj * tb.Lp[(j * 3 + cc) * npt + pt];
+          }
+        for (int v = 0; v < 9; ++v) u[v] = m[v] + tau * (u[v] - m[v]);
+        const double pq = pres(u);
+        if (pq < p.eps_p) taup = fmin(taup, (pmean - p.eps_p) / (pmean - pq));
+      }
+    }
+    taup = fmax(wmin(taup), 0.0);
+    const double t = tau * taup;
+    if (t >= 1.0) continue;
+    if (lane == 0) atomicAdd(&sc->pos_cells, 1ull);
+    // scale every non-mean row by tau
+    for (int r = lane; r < NR; r += 32) {
+      const bool mean = r < NPS * N ? r % N == 0 : r - 5 * N < 3;
+      if (!mean) w[(int64_t)r * S + c] = t * R[r];
+    }
+  }
+}
+
 // Every cell (list == nullptr) or the listed cells list[0 .. sc->npos); grid-stride.
 template <typename T>
 __global__ void k_pos(Geom g, Tables<T> tb, LimTabs lt, T* w, double* wmean, dg_mhd_params p, DevScalars* sc,
@@ -863,7 +1019,7 @@ __global__ void k_pos(Geom g, Tables<T> tb, LimTabs lt, T* w, double* wmean, dg_
 // pass: flow, 436,000 of 504,000 cells listed, 1.69 ms; 256^3 turbulence,
 // 415,000 listed, 1.60 ms; 128^3 Powell blast, 4,000 listed, 0.69 ms.
 template <int DEG, int GLMF>
-__global__ void __launch_bounds__(128) k_pos_list(Geom gin, Tables<float> tb, LimTabs lt, LdfLeg ll, float* w,
+__global__ void __launch_bounds__(128) k_pos_list(Geom gin, Tables<float> tb, PosScreen ps, LdfLeg ll, float* w,
                                                   double* wmean, dg_mhd_params p, DevScalars* sc,
                                                   const int32_t* __restrict__ list) {
   const Geom g = pin_geom<DEG, GLMF>(gin);
@@ -906,34 +1062,7 @@ __global__ void __launch_bounds__(128) k_pos_list(Geom gin, Tables<float> tb, Li
     if (listed) {
 #pragma unroll
       for (int r = 0; r < NR; ++r) R[r][lane] = w[(int64_t)r * S + c];
-      const int nlg = g.glm ? 8 : 5;
-#pragma unroll
-      for (int v = 0; v < 8; ++v) {
-        if (v >= nlg) continue;
-        for (int l = 1; l < g.n; ++l) devt[v] += fabsf(R[v * g.n + l][lane]);
-      }
-      if (!g.glm)
-        for (int j = g.D; j < g.ndiv; ++j) {
-          const float aj = fabsf(R[g.ldf0 + j][lane]);
-#pragma unroll
-          for (int cc = 0; cc < 3; ++cc) devt[5 + cc] += aj * (float)lt.ldf_maxabs[j * 3 + cc];
-        }
-      auto coef = [&](auto VI, int i, int j, int k) -> float {
-        constexpr int v = decltype(VI)::value;
-        const int l = sf::mode_idx(i, j, k);
-        if constexpr (GLMF || v < 5) {
-          return R[v * N + l][lane];
-        } else {
-          float x = 0.f;
-#pragma unroll
-          for (int q = 0; q < LdfPattern<DEG>::NDIV; ++q)
-            if (ldf_has<DEG>(q, v - 5, l)) x = fmaf(R[5 * N + q][lane], ll.A[(q * 3 + v - 5) * N + l], x);
-          return x;
-        }
-      };
-      float mt[8];
-      sf::each<0, 8>([&](auto VI) { mt[decltype(VI)::value] = coef(VI, 0, 0, 0); });
-      valid = !pos_points_clear<DEG>(coef, mt, devt, (float)p.eps_rho, (float)p.eps_p, gm1t);
+      valid = !pos_points_rows<DEG, GLMF>([&](int r) { return R[r][lane]; }, ll, (float)p.eps_rho, (float)p.eps_p, ps, devt);
     }
     if (!__any_sync(0xffffffffu, valid)) continue;
     if (valid) {
@@ -1244,7 +1373,7 @@ int run_limiter(Ctx& c, void* w, double* wmean, uint8_t* troubled, cudaStream_t 
         else g.glm ? scr(k_pos_screen<1, 1>) : scr(k_pos_screen<1, 0>);
       }
       const unsigned nbl = (unsigned)std::min<int64_t>(nb, (int64_t)c.nsm * 16);
-      auto pw = [&](auto k) { k<<<(unsigned)c.nsm * 8, 128, 0, st>>>(g, c.t32, c.lim, c.ldf_leg, (float*)w, wmean, c.p,
+      auto pw = [&](auto k) { k<<<(unsigned)c.nsm * 8, 128, 0, st>>>(g, c.t32, c.pscr, c.ldf_leg, (float*)w, wmean, c.p,
                                                                     c.sc, c.pos_list); };
       if (!pinned_sizes_ok(g) || !wmean || !c.ldf_leg.ok)
         k_pos<float><<<nbl, 128, 0, st>>>(g, c.t32, c.lim, (float*)w, wmean, c.p, c.sc, c.pos_list);
@@ -1252,7 +1381,21 @@ int run_limiter(Ctx& c, void* w, double* wmean, uint8_t* troubled, cudaStream_t 
       else g.glm ? pw(k_pos_list<1, 1>) : pw(k_pos_list<1, 0>);
       if (!screened) c.prof.launches[5] += 1;  // the screen and the list kernel
     } else {
-      k_pos<double><<<nb, 128, 0, st>>>(g, c.t64, c.lim, (double*)w, nullptr, c.p, c.sc, nullptr);
+      if (pinned_sizes_ok(g) && c.ldf_leg.ok) {
+        if (c.p.limiter == DG_LIMIT_OFF) cudaMemsetAsync(&c.sc->npos, 0, sizeof(unsigned), st);
+        auto pre = [&](auto k) {
+          k<<<nb, 128, 0, st>>>(g, c.pscr, c.ldf_leg, (const double*)w, (float)c.p.eps_rho, (float)c.p.eps_p, c.sc,
+                                c.pos_list);
+        };
+        if (g.d == 2) g.glm ? pre(k_pos_pre64<2, 1>) : pre(k_pos_pre64<2, 0>);
+        else g.glm ? pre(k_pos_pre64<1, 1>) : pre(k_pos_pre64<1, 0>);
+        auto lst = [&](auto k) { k<<<(unsigned)c.nsm * 8, 128, 0, st>>>(g, c.t64, (double*)w, c.p, c.sc, c.pos_list); };
+        if (g.d == 2) g.glm ? lst(k_pos_list64<2, 1>) : lst(k_pos_list64<2, 0>);
+        else g.glm ? lst(k_pos_list64<1, 1>) : lst(k_pos_list64<1, 0>);
+        c.prof.launches[5] += 1;
+      } else {
+        k_pos<double><<<nb, 128, 0, st>>>(g, c.t64, c.lim, (double*)w, nullptr, c.p, c.sc, nullptr);
+      }
     }
     c.prof.end(5, st);
   }

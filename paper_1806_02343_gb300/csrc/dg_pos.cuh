@@ -157,6 +157,41 @@ __device__ __forceinline__ bool pos_points_clear(Coef coef, const float (&mt)[8]
   return ok;
 }
 
+// pos_points_clear from a cell's rows (LDF B through the sparse map)
+template <int DEG, int GLMF, typename Row>
+__device__ __forceinline__ bool pos_points_rows(Row row, const LdfLeg& ll, float eps_rho, float eps_p,
+                                                const PosScreen& ps, float (&devt)[8]) {
+  constexpr int N = LdfPattern<DEG>::N, NDIV = LdfPattern<DEG>::NDIV;
+#pragma unroll
+  for (int v = 0; v < 8; ++v) {
+    devt[v] = 0.f;
+    if (GLMF || v < 5)
+      for (int l = 1; l < N; ++l) devt[v] += fabsf(row(v * N + l));
+  }
+  if (!GLMF)
+    for (int j = 3; j < NDIV; ++j) {
+      const float aj = fabsf(row(5 * N + j));
+#pragma unroll
+      for (int cc = 0; cc < 3; ++cc) devt[5 + cc] += aj * ps.ldf_maxabs[j * 3 + cc];
+    }
+  auto coef = [&](auto VI, int i, int j, int k) -> float {
+    constexpr int v = decltype(VI)::value;
+    const int l = sf::mode_idx(i, j, k);
+    if constexpr (GLMF || v < 5) {
+      return row(v * N + l);
+    } else {
+      float x = 0.f;
+#pragma unroll
+      for (int q = 0; q < NDIV; ++q)
+        if (ldf_has<DEG>(q, v - 5, l)) x = fmaf(row(5 * N + q), ll.A[(q * 3 + v - 5) * N + l], x);
+      return x;
+    }
+  };
+  float mt[8];
+  sf::each<0, 8>([&](auto VI) { mt[decltype(VI)::value] = coef(VI, 0, 0, 0); });
+  return pos_points_clear<DEG>(coef, mt, devt, eps_rho, eps_p, ps.gm1);
+}
+
 // ballot compaction of a warp's cells into list[0 .. *count)
 __device__ __forceinline__ void append_cells(bool mine, int64_t c, int32_t* __restrict__ list, unsigned* count) {
   const int lane = threadIdx.x & 31;
