@@ -705,7 +705,8 @@ int dg_mhd_init(const dg_mesh_desc* mesh, int degree, int divB_scheme, double ga
                         prm.powell_q != 1;
   size_t face_pts = (size_t)g.D * g.stride * g.Qf;
   if (c.amr.on) face_pts = std::max(face_pts, (size_t)c.amr.nface * g.Qf);
-  const size_t face_elems = face_pts * (pow_fast ? 10 : 9);
+  c.op2d = !fp32(c) && !c.amr.on && prm.generic_kernels != 1 && prm.powell_q != 1 && op2d_ok(g);
+  const size_t face_elems = face_pts * (pow_fast || (c.op2d && !g.glm) ? 10 : 9);
   bool ok = cudaMalloc(&c.sc, sizeof(DevScalars)) == cudaSuccess &&
             cudaMemset(c.sc, 0, sizeof(DevScalars)) == cudaSuccess &&
             cudaMalloc(&c.stage_buf[0], state_bytes) == cudaSuccess &&
@@ -950,6 +951,13 @@ int operator_pass(Ctx& c, const void* w, const double* wmean, void* out, double*
     launch_cell<float>(g, c.t32, (const float*)w, c.face_buf32, (float*)out, (const float*)w0, ca, cb, combine,
                        c.sc, wmean, w0mean, outmean, st, (const float*)c.qdag_buf);
     c.prof.end(1, st);
+  } else if (c.op2d) {
+    c.prof.begin(0, st);
+    launch_face_2d(g, c.t64, (const double*)w, c.face_buf, c.sc, c.p.eps_hlld, st);
+    c.prof.end(0, st);
+    c.prof.begin(1, st);
+    launch_cell_2d(g, c.t64, (const double*)w, c.face_buf, (double*)out, (const double*)w0, ca, cb, combine, c.sc, st);
+    c.prof.end(1, st);
   } else {
     c.prof.begin(0, st);
     launch_face<double>(g, c.t64, (const double*)w, c.face_buf, c.sc, c.p.eps_hlld, st, (double*)c.qdag_buf);
@@ -990,6 +998,12 @@ int dt_pass(Ctx& c, const void* w, const double* wmean, double* dt_out, cudaStre
     return cudaGetLastError() == cudaSuccess ? DG_OK : DG_E_CUDA;
   }
   c.prof.begin(2, st);
+  if (c.op2d) {
+    launch_dt_2d(g, c.t64, (const double*)w, c.face_buf, c.p, c.sc, dt_out, c.nsm, st);
+    c.prof.end(2, st);
+    c.prof.launches[2] += 1;  // the jumps, or the reset (GLM), and k2_dt
+    return cudaGetLastError() == cudaSuccess ? DG_OK : DG_E_CUDA;
+  }
   // the specialised Powell jump kernel stores two sums per face (gj.jq = 1)
   Geom gj = g;
   if (!g.glm && divb_face_fast(c, w, st)) gj.jq = 1;

@@ -122,6 +122,7 @@ struct DevScalars {
   double dt_step;                  // the step's dt; dt itself may be a fraction of it for some stages
   unsigned long long dt64_bits;    // FP32 form: FP64 minimum of the screened cells' FP64 bounds
   unsigned long long cnt_poslisted;  // cells listed for the full positivity procedure, summed over passes
+  unsigned int dt_done;              // blocks of the 2D timestep kernel that are done (0 between launches)
 };
 
 // a device scalar in the working precision T (FP32 kernels read the float copy)
@@ -275,6 +276,7 @@ struct Ctx {
   int nsm = 152;                   // streaming multiprocessors of the device
   int fast = 0;                    // specialised GLM path: 10*prec + degree, 0 = none
   void* fast_tabs = nullptr;       // host FastAll<T, DEG> (kernel parameters)
+  bool op2d = false;               // FP64, uniform 2D: the kernels of dg_2d.cu
   float* tc_tabs = nullptr;        // device operand tables of the tensor-core cell kernel (FP32, degree 2)
   uint8_t* owned = nullptr;        // device copy of the owned-cell mask (dg_mhd_set_owned), or NULL
   bool glm_speeds_set = false;     // GLM: c_h and the damping rate hold a value (from a dt, set_glm or set_dt)

@@ -40,6 +40,14 @@ void launch_dt(const Geom& g, const Tables<T>& tb, const T* w, const double* wme
 void launch_dt_from_value(const Geom& g, const dg_mhd_params& p, const double* dt_in, DevScalars* sc,
                           cudaStream_t st);
 void launch_set_glm(DevScalars* sc, double ch, double kappa, cudaStream_t st);
+// FP64 on uniform 2D meshes, degrees 1-3 (dg_2d.cu)
+bool op2d_ok(const Geom& g);
+void launch_face_2d(const Geom& g, const Tables<double>& tb, const double* w, double* F, const DevScalars* sc,
+                    double eps, cudaStream_t st);
+void launch_cell_2d(const Geom& g, const Tables<double>& tb, const double* w, double* F, double* out, const double* w0,
+                    double ca, double cb, int combine, const DevScalars* sc, cudaStream_t st);
+void launch_dt_2d(const Geom& g, const Tables<double>& tb, const double* w, double* J, const dg_mhd_params& p,
+                  DevScalars* sc, double* dt_out, int nsm, cudaStream_t st);
 void launch_dt_init(DevScalars* sc, cudaStream_t st);
 // div B diagnostics of App. C (uniform meshes): res[4] on the device, per_cell
 // [3][stride] or null; scratch: 3 doubles per face point
