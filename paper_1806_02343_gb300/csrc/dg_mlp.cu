@@ -433,23 +433,25 @@ __global__ void k_to_bf16(const float* __restrict__ src, __nv_bfloat16* __restri
   dst[i] = __float2bfloat16_rn(k < cols ? src[r * cols + k] : 0.f);
 }
 
-// ---------------------------------------------------------------- staged inference
-// FP32 form on uniform 3D meshes whose x-rows hold whole 128-cell tiles: the
-// state rows of a tile (128 consecutive cells, 512 B per row) and the mean
-// rows of its four y/z neighbour tiles are fetched by bulk asynchronous copies
-// (cp.async.bulk, completion counted on an mbarrier) into shared memory; the
-// features are then built from shared memory, so each block keeps ~57 KB of
-// loads in flight instead of each thread walking 80+ dependent global loads.
+// ---------------------------------------------------------------- tiled inference
+// FP32 form on uniform 3D meshes whose x-rows hold whole 128-cell tiles, on the
+// tensor core: two threads per cell build the features of their variables straight
+// from coalesced loads (a row of a warp's 32 cells is one 128-byte line; the x, y, z
+// neighbours' means are lines that other tiles of the same SMs read as rows) and
+// store them, eight at a time, as the layer's BF16 operand. Each part reads only its
+// own variables of the neighbours, and the FP32 positivity screen is summed from the
+// same registers. 57 KB of shared memory at degree 2: four blocks per SM overlap
+// their loads, their two layers and their epilogues. Bound by the loads' latency
+// and the instruction issue. (Staging the 112 rows of a tile in shared memory by
+// bulk copies took 57 KB more: two blocks per SM, each waiting for its copies, and
+// 2-byte feature stores with 4-way bank conflicts: 3.91 ms per pass on 256^3 cells,
+// GLM, degree 2, now 2.00 ms; 128^3, Powell, 0.51 and 0.28 ms.)
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
   return (unsigned)__cvta_generic_to_shared(p);
 }
 __device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, unsigned parity) {
   unsigned ok;
@@ -462,80 +464,172 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, unsigned parity) {
       : "memory");
   return ok != 0;
 }
-// global -> shared bulk copy of `bytes` (multiple of 16, both addresses 16-byte aligned)
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-
-// a cell of the staged tile: own rows st[r][t], y/z neighbour means nbm[q][k][t]
-// (q = 2 (axis - 1) + side), x neighbours inside the tile or, at its two ends,
-// xe[side][k]
-template <typename Dm>
-struct StagedSrc {
-  Dm dm;
-  const float* st;
-  const float* nbm;
-  const float* xe;
-  int t;
-  __device__ float row(int r) const { return st[r * 128 + t]; }
-  __device__ float imdx(const MlpTabs& mt) const { return mt.inv_mdx; }
-  __device__ void nbraw(int a, int s, float* raw) const {
-    if (a == 0) {
-      const int tt = t + (s ? 1 : -1);
-      if (tt < 0 || tt > 127)
-        for (int k = 0; k < 8; ++k) raw[k] = xe[s * 8 + k];
-      else
-        for (int k = 0; k < 8; ++k) raw[k] = st[dm.mrow(k) * 128 + tt];
-    } else {
-      const int q = 2 * (a - 1) + s;
-      for (int k = 0; k < 8; ++k) raw[k] = nbm[(q * 8 + k) * 128 + t];
-    }
-  }
-};
 
 constexpr long long kWaitCycles = 2000000000ll;  // about one second at GB300 clocks
 
-template <int KP, bool GLM, int DEG, int NTH>
-__global__ void __launch_bounds__(NTH) k_mlp_staged(Geom g, MlpTabs mt, const float* __restrict__ w,
-                                                    const __nv_bfloat16* __restrict__ W1,
-                                                    const __nv_bfloat16* __restrict__ W2,
-                                                    const float* __restrict__ bias, float thresh,
-                                                    uint8_t* __restrict__ flag, float* __restrict__ prob,
-                                                    int32_t* __restrict__ list, DevScalars* __restrict__ sc,
-                                                    int nrs, int nbuf, int32_t* __restrict__ plist, PosScreen ps) {
+// feature words (two BF16 each) START .. START + CNT of cell `cell`: 16-byte
+// stores where four words of a core-matrix row are complete
+template <int START, int CNT, int KP>
+__device__ __forceinline__ void put_words(__nv_bfloat16* Xs, int cell, const uint32_t* W) {
+  sf::each<0, CNT>([&](auto K) {
+    constexpr int k = decltype(K)::value, at = START + k, q0 = at / 4 * 4;  // q0: the quad's first word
+    constexpr bool quad = q0 >= START && q0 + 4 <= START + CNT;
+    __nv_bfloat16* d = Xs + tc::kmajor_index(cell, 2 * at, KP);
+    if constexpr (!quad) *reinterpret_cast<uint32_t*>(d) = W[k];
+    else if constexpr (at == q0) *reinterpret_cast<uint4*>(d) = make_uint4(W[k], W[k + 1], W[k + 2], W[k + 3]);
+  });
+}
+
+// Features of `features_of` (same expressions, so the same BF16 values) of the
+// variables of part P (GLM: 0-3, 4-7; Powell: the hydro variables, B), and of the
+// same variables the terms of pos_screen_rows: dv (sum of |coefficients| beyond the
+// mean, times the basis bound) and ms (mean). cn: the cell's neighbours.
+template <bool GLM, int DEG, int KP, int P>
+__device__ __forceinline__ void tile_features(const MlpTabs& mt, const PosScreen& ps, const float* __restrict__ w,
+                                              int64_t S, int64_t c, const int64_t (&cn)[6], int cell,
+                                              __nv_bfloat16* Xs, float* dv, float* ms) {
+  using Dm = CtDims<GLM, DEG>;
+  constexpr int N = Dm::N, SLOPE = 8 * N + 6;
+  static_assert(N % 2 == 0, "pairs of features stay within a variable");
+  if constexpr (GLM || P == 0) {
+    constexpr int V0 = GLM ? 4 * P : 0, NV = GLM ? 4 : 5;
+    const float* base = w + (int64_t)(V0 * N) * S;
+    float m[NV], dmax[NV], nd[6];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      m[v] = base[(int64_t)(v * N) * S + c];
+      dmax[v] = 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const float x = base[(int64_t)(v * N) * S + cn[q]];
+        dmax[v] = fmaxf(dmax[v], fabsf(x - m[v]));
+        if (P == 0 && v == 0) nd[q] = x / m[0] - 1.f;
+      }
+    uint32_t W[NV * N / 2];
+    float sl[3][NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const float inv = 1.f / (fabsf(m[v]) + dmax[v] + 1e-12f);
+      float f[N], d = 0.f;
+#pragma unroll
+      for (int l = 0; l < N; ++l) {
+        const float av = l == 0 ? m[v] : base[(int64_t)(v * N + l) * S + c];
+        f[l] = av * inv;
+        if (l > 0) d += fabsf(av);
+        if (l >= 1 && l <= 3) sl[l - 1][v] = av * mt.inv_mdx;
+      }
+      dv[v] = d;
+      ms[v] = m[v];
+#pragma unroll
+      for (int l = 0; l < N; l += 2) W[(v * N + l) / 2] = pack_bf16(f[l], f[l + 1]);
+    }
+    put_words<V0 * N / 2, NV * N / 2, KP>(Xs, cell, W);
+    uint32_t x[3];
+    if constexpr (P == 0) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) x[a] = pack_bf16(nd[2 * a], nd[2 * a + 1]);
+      put_words<4 * N, 3, KP>(Xs, cell, x);
+    } else {  // padding up to KP
+      x[0] = 0u;
+      put_words<(SLOPE + 24) / 2, 1, KP>(Xs, cell, x);
+    }
+    sf::each<0, 3>([&](auto A) {
+      constexpr int a = decltype(A)::value;
+      x[0] = pack_bf16(sl[a][0], sl[a][1]);
+      x[1] = pack_bf16(sl[a][2], sl[a][3]);
+      put_words<(SLOPE + 8 * a + V0) / 2, 2, KP>(Xs, cell, x);
+      if constexpr (NV == 5) Xs[tc::kmajor_index(cell, SLOPE + 8 * a + 4, KP)] = __float2bfloat16_rn(sl[a][4]);
+    });
+  } else {
+    constexpr int NDIV = Dm::NDIV;
+    const float* base = w + (int64_t)(5 * N) * S;
+    auto phys = [&](const float* raw, float* m) {
+      m[0] = m[1] = m[2] = 0.f;
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+#pragma unroll
+        for (int cc = 0; cc < 3; ++cc) m[cc] += raw[j] * mt.l2l[(j * 3 + cc) * MLP_MAXN + 0];
+    };
+    float R[NDIV], m[3], dmax[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < NDIV; ++j) R[j] = base[(int64_t)j * S + c];
+    phys(R, m);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      float raw[3], mn[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) raw[j] = base[(int64_t)j * S + cn[q]];
+      phys(raw, mn);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) dmax[k] = fmaxf(dmax[k], fabsf(mn[k] - m[k]));
+    }
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc) {
+      dv[cc] = ms[cc] = 0.f;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) ms[cc] += R[j] * ps.ldf_mean0[j * 3 + cc];
+    }
+#pragma unroll
+    for (int j = 3; j < NDIV; ++j)
+#pragma unroll
+      for (int cc = 0; cc < 3; ++cc) dv[cc] += fabsf(R[j]) * ps.ldf_maxabs[j * 3 + cc];
+    uint32_t W[3 * N / 2], x[1];
+    sf::each<0, 3>([&](auto CC) {
+      constexpr int cc = decltype(CC)::value;
+      const float inv = 1.f / (fabsf(m[cc]) + dmax[cc] + 1e-12f);
+      float f[N];
+      sf::each<0, N>([&](auto L) {
+        constexpr int l = decltype(L)::value;
+        float acc = 0.f;
+        sf::each<0, NDIV>([&](auto J) {
+          constexpr int j = decltype(J)::value;
+          if constexpr (Dm::has(j, cc, l)) acc += R[j] * mt.l2l[(j * 3 + cc) * MLP_MAXN + l];
+        });
+        f[l] = acc * inv;
+        if constexpr (l >= 1 && l <= 3) {
+          constexpr int q = SLOPE + 8 * (l - 1) + 5 + cc;
+          Xs[tc::kmajor_index(cell, q, KP)] = __float2bfloat16_rn(acc * mt.inv_mdx);
+        }
+      });
+#pragma unroll
+      for (int l = 0; l < N; l += 2) W[(cc * N + l) / 2] = pack_bf16(f[l], f[l + 1]);
+    });
+    put_words<5 * N / 2, 3 * N / 2, KP>(Xs, cell, W);
+    x[0] = 0u;
+    put_words<(SLOPE + 24) / 2, 1, KP>(Xs, cell, x);
+  }
+}
+
+constexpr int kTileThreads = 256;  // two threads per cell of the 128-cell tile
+
+template <int KP, bool GLM, int DEG>
+__global__ void __launch_bounds__(kTileThreads, DEG <= 2 ? 4 : 2)
+    k_mlp_tile(Geom g, const __grid_constant__ MlpTabs mt, const float* __restrict__ w,
+               const __nv_bfloat16* __restrict__ W1, const __nv_bfloat16* __restrict__ W2,
+               const float* __restrict__ bias, float thresh, uint8_t* __restrict__ flag, float* __restrict__ prob,
+               int32_t* __restrict__ list, DevScalars* __restrict__ sc, int32_t* __restrict__ plist,
+               const __grid_constant__ PosScreen ps) {
+  constexpr int NTH = kTileThreads, CG = NTH / 128, CW = HID / CG, N1 = GLM ? 4 : 3;
   extern __shared__ __align__(128) unsigned char smraw[];
-  // nbuf tile buffers, each [nrs][128] own rows then [4][8][128] neighbour means
-  float* buf = reinterpret_cast<float*>(smraw);
-  const int bufsz = (nrs + 32) * 128;
-  float* xe = buf + nbuf * bufsz;                        // [2][8]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(xe + 16);  // [0], [1]: tile copies; [2]: MMA completion
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 3);
   // tensor-core operands in the K-major core-matrix layout (dg_tc.cuh)
-  __nv_bfloat16* W1s = reinterpret_cast<__nv_bfloat16*>(xe + 32);  // [HID][KP]
-  __nv_bfloat16* W2s = W1s + HID * KP;                              // [HID][HID]
+  __nv_bfloat16* W1s = reinterpret_cast<__nv_bfloat16*>(smraw);  // [HID][KP]
+  __nv_bfloat16* W2s = W1s + HID * KP;                           // [HID][HID]
   __nv_bfloat16* Xs = W2s + HID * HID;  // [128][KP] features; then layer 1's output [128][HID]
-  float* bs = reinterpret_cast<float*>(Xs + 128 * KP);  // b1[64], b2[64], w3[64], b3
-  // NP = NTH / 128 threads per cell split the feature work; the NTH / 32 warps
-  // split the epilogues: warp w reads tensor-memory lanes 32 (w % 4).. and a
-  // group of CW = HID / CG columns, CG = NTH / 128 groups
-  constexpr int NP = NTH / 128, CG = NTH / 128, CW = HID / CG;
-  static_assert(CW == 32 || CW == 16, "column groups of 32 or 16");
-  float* part = bs + 3 * HID + 1;                       // [CG][128] partial sums of the output layer
-  uint8_t* fl = reinterpret_cast<uint8_t*>(part + CG * 128);  // [128] flags of the tile
-  uint8_t* sfail = fl + 128;                              // [128] positivity screen not cleared
+  float* scr = reinterpret_cast<float*>(Xs + 128 * KP);  // [2][N1][128] part 1's dv and ms
+  float* part = scr + 2 * N1 * 128;                      // [CG][128] partial sums of the output layer
+  float* bs = part + CG * 128;                           // b1[64], b2[64], w3[64], b3
+  uint64_t* bar = reinterpret_cast<uint64_t*>(bs + 3 * HID + 2);  // MMA completion
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 1);
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int cell = t & 127, fpart = t >> 7;
+  const int cell = t & 127, fpart = t >> 7;  // warp-uniform part
   for (int i = t; i < HID * KP; i += NTH) W1s[tc::kmajor_index(i / KP, i % KP, KP)] = W1[i];
   for (int i = t; i < HID * HID; i += NTH) W2s[tc::kmajor_index(i / HID, i % HID, HID)] = W2[i];
   for (int i = t; i < 3 * HID + 1; i += NTH) bs[i] = bias[i];
   if (t == 0) {
     mbar_init(bar, 1);
-    mbar_init(bar + 1, 1);
-    mbar_init(bar + 2, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // 128 tensor-memory columns: layer 1's accumulator [128 x 64], then layer 2's
@@ -546,76 +640,41 @@ __global__ void __launch_bounds__(NTH) k_mlp_staged(Geom g, MlpTabs mt, const fl
   const uint32_t tm = *tslot;
   constexpr uint32_t IDESC = tc::idesc_bf16_f32(128, HID);
   const int64_t S = g.stride;
-  const int nin = 8 * g.n + 10 * g.D;
-  const unsigned bytes = (unsigned)(nrs + 32) * 512u;
-  const int64_t ntile = g.ncell / 128;
-  // thread 0: bulk copies of tile `tl` into buffer b, completion counted on bar[b]
-  auto issue = [&](int64_t tl, int b) {
-    float* st = buf + b * bufsz;
-    float* nbm = st + nrs * 128;
-    const int64_t c0 = tl * 128;
-    // the buffer's previous reads (generic proxy) are ordered before these writes
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_arrive_expect_tx(bar + b, bytes);
-    for (int r = 0; r < nrs; ++r) bulk_g2s(st + r * 128, w + (int64_t)r * S + c0, 512u, bar + b);
-    for (int q = 0; q < 4; ++q) {
-      const int64_t cn = nbc(g, c0, 1 + (q >> 1), (q & 1) ? 1 : -1);  // the whole tile shifts
-      for (int k = 0; k < 8; ++k)
-        bulk_g2s(nbm + (q * 8 + k) * 128, w + (int64_t)mrow(g, k) * S + cn, 512u, bar + b);
-    }
-  };
+  const unsigned ntile = (unsigned)(g.ncell / 128), tpr = (unsigned)g.nx / 128u;
   // bounded wait of every thread on an mbarrier phase; false on timeout (all threads agree)
-  auto wait_all = [&](uint64_t* b, unsigned parity) {
+  auto wait_all = [&](unsigned parity) {
     bool ok = false;
     const long long t0 = clock64();
-    while (!(ok = mbar_try_wait(b, parity)))
+    while (!(ok = mbar_try_wait(bar, parity)))
       if (clock64() - t0 > kWaitCycles) break;
     return __syncthreads_and(ok) != 0;
   };
-  // two buffers: the next tile's copies run while this one is computed.
-  // Every thread tracks which buffers have copies issued but not yet observed
-  // complete (the issue decisions are block-uniform): a block that gives up on
-  // a wait drains them before it exits, so no asynchronous write into its
-  // shared memory outlives it.
-  unsigned pend = 0;  // bit b: copies into buffer b issued, completion not yet observed
-  if (nbuf == 2 && blockIdx.x < ntile) {
-    if (t == 0) issue(blockIdx.x, 0);
-    pend |= 1u;
-  }
-  unsigned par = 0;  // bit b: phase parity of bar[b]
-  int it = 0;
   int mma_pending = -1;  // parity of an MMA commit not yet observed (timeout path), else -1
-  for (int64_t tile = blockIdx.x; tile < ntile; tile += gridDim.x, ++it) {
-    const int64_t c0 = tile * 128;
-    const int b = nbuf == 2 ? (it & 1) : 0;
-    const int64_t next = tile + gridDim.x;
-    if (nbuf == 1) {
-      if (t == 0) issue(tile, 0);
-      pend |= 1u;
-    } else if (next < ntile) {
-      if (t == 0) issue(next, b ^ 1);  // released by the previous iteration's barrier
-      pend |= 1u << (b ^ 1);
-    }
-    if (t < 16) {
-      const int sd = t >> 3, k = t & 7;
-      xe[t] = w[(int64_t)mrow(g, k) * S + nbc(g, c0 + (sd ? 127 : 0), 0, sd ? 1 : -1)];
-    }
-    // bounded wait for the tile's bytes (every thread polls: measured faster
-    // than one polling warp and a block barrier)
-    if (!wait_all(bar + b, (par >> b) & 1u)) {
-      if (t == 0) atomicOr(&sc->status, 8);
-      break;
-    }
-    par ^= 1u << b;
-    pend &= ~(1u << b);
-    const float* st = buf + b * bufsz;
+  for (unsigned tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    const int64_t c0 = (int64_t)tile * 128, c = c0 + cell;
+    int64_t cn[6];
     {
-      using Dm = CtDims<GLM, DEG>;
-      if (fpart == NP - 1)
-        for (int q = nin; q < KP; ++q) Xs[tc::kmajor_index(cell, q, KP)] = __float2bfloat16_rn(0.f);
-      features_of(Dm{}, mt, StagedSrc<Dm>{Dm{}, st, st + nrs * 128, xe, cell},
-                  [&](int q, float v) { Xs[tc::kmajor_index(cell, q, KP)] = __float2bfloat16_rn(v); }, fpart,
-                  NP);
+      const unsigned rowi = tile / tpr, xt = tile - rowi * tpr;
+      const int iz = (int)(rowi / (unsigned)g.ny), iy = (int)(rowi - (unsigned)iz * (unsigned)g.ny);
+      const int x = (int)(xt * 128u) + cell;
+      const int64_t pl = (int64_t)g.nx * g.ny;
+      cn[0] = x == 0 ? c + g.nx - 1 : c - 1;
+      cn[1] = x == g.nx - 1 ? c - (g.nx - 1) : c + 1;
+      cn[2] = iy == 0 ? c + pl - g.nx : c - g.nx;
+      cn[3] = iy == g.ny - 1 ? c - (pl - g.nx) : c + g.nx;
+      cn[4] = iz == 0 ? c + pl * (g.nz - 1) : c - pl;
+      cn[5] = iz == g.nz - 1 ? c - pl * (g.nz - 1) : c + pl;
+    }
+    float dv[5], ms[5];
+    if (fpart == 0) {
+      tile_features<GLM, DEG, KP, 0>(mt, ps, w, S, c, cn, cell, Xs, dv, ms);
+    } else {
+      tile_features<GLM, DEG, KP, 1>(mt, ps, w, S, c, cn, cell, Xs, dv, ms);
+#pragma unroll
+      for (int k = 0; k < N1; ++k) {
+        scr[k * 128 + cell] = dv[k];
+        scr[(N1 + k) * 128 + cell] = ms[k];
+      }
     }
     tc::fence_proxy_async();  // the features, written by every thread, become tensor-core operands
     __syncthreads();
@@ -626,19 +685,29 @@ __global__ void __launch_bounds__(NTH) k_mlp_staged(Geom g, MlpTabs mt, const fl
       for (int kk = 0; kk < KP / 16; ++kk)
         tc::mma_bf16(tm, tc::smem_desc(tc::smem_u32(Xs + kk * 128), 128, KP * 16),
                      tc::smem_desc(tc::smem_u32(W1s + kk * 128), 128, KP * 16), IDESC, kk > 0);
-      tc::commit(bar + 2);
+      tc::commit(bar);
     }
     mma_pending = 0;
-    if (plist && t < 128) {
-      // FP32 positivity screen on the staged rows (they hold every row the
-      // screen reads), while the tensor core runs layer 1; only the cells the
-      // indicator does not flag are listed from it (the TVB kernel screens the
+    bool sfail = false;
+    if (plist && fpart == 0) {
+      // FP32 positivity screen, while the tensor core runs layer 1; only the cells
+      // the indicator does not flag are listed from it (the TVB kernel screens the
       // flagged ones after limiting them)
-      Geom gp = g;
-      if constexpr (DEG <= 2) gp = pin_geom<DEG, GLM ? 1 : 0>(g);
-      sfail[t] = pos_screen_rows(gp, ps, [&](int r) { return st[r * 128 + t]; }) ? 0 : 1;
+      constexpr int N0 = GLM ? 4 : 5;
+      float d8[8], m8[8];
+#pragma unroll
+      for (int k = 0; k < N0; ++k) {
+        d8[k] = dv[k];
+        m8[k] = ms[k];
+      }
+#pragma unroll
+      for (int k = N0; k < 8; ++k) {
+        d8[k] = scr[(k - N0) * 128 + cell];
+        m8[k] = scr[(N1 + k - N0) * 128 + cell];
+      }
+      sfail = !pos_screen_bound(ps, m8, d8);
     }
-    if (!wait_all(bar + 2, 0)) {
+    if (!wait_all(0)) {
       if (t == 0) atomicOr(&sc->status, 8);
       break;
     }
@@ -650,8 +719,7 @@ __global__ void __launch_bounds__(NTH) k_mlp_staged(Geom g, MlpTabs mt, const fl
     const uint32_t tlane = (uint32_t)(32 * quarter) << 16;
     {
       float v[CW];
-      if constexpr (CW == 32) tc::ld32(tm + tlane + CW * colh, v);
-      else tc::ld16(tm + tlane + CW * colh, v);
+      tc::ld32(tm + tlane + CW * colh, v);
       // 16-byte stores of eight BF16 values: the 8 rows of a core matrix fill 128 contiguous bytes
 #pragma unroll
       for (int j = 0; j < CW / 8; ++j) {
@@ -675,10 +743,10 @@ __global__ void __launch_bounds__(NTH) k_mlp_staged(Geom g, MlpTabs mt, const fl
       for (int kk = 0; kk < HID / 16; ++kk)
         tc::mma_bf16(tm + HID, tc::smem_desc(tc::smem_u32(Xs + kk * 128), 128, HID * 16),
                      tc::smem_desc(tc::smem_u32(W2s + kk * 128), 128, HID * 16), IDESC, kk > 0);
-      tc::commit(bar + 2);
+      tc::commit(bar);
     }
     mma_pending = 1;
-    if (!wait_all(bar + 2, 1)) {
+    if (!wait_all(1)) {
       if (t == 0) atomicOr(&sc->status, 8);
       break;
     }
@@ -687,8 +755,7 @@ __global__ void __launch_bounds__(NTH) k_mlp_staged(Geom g, MlpTabs mt, const fl
     // epilogue 2: bias, ReLU and this warp's share of the output layer's dot product
     {
       float v[CW];
-      if constexpr (CW == 32) tc::ld32(tm + tlane + HID + CW * colh, v);
-      else tc::ld16(tm + tlane + HID + CW * colh, v);
+      tc::ld32(tm + tlane + HID + CW * colh, v);
       float o = 0.f;
 #pragma unroll
       for (int j = 0; j < CW; ++j) o += fmaxf(v[j] + bs[HID + CW * colh + j], 0.f) * bs[2 * HID + CW * colh + j];
@@ -696,39 +763,24 @@ __global__ void __launch_bounds__(NTH) k_mlp_staged(Geom g, MlpTabs mt, const fl
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (t < 128) {
+    // output and lists, by the first part's four warps; the other part goes on to the
+    // next tile (it writes `part` again only behind that tile's barriers)
+    if (fpart == 0) {
       float z = bs[3 * HID];
 #pragma unroll
       for (int gq = 0; gq < CG; ++gq) z += part[gq * 128 + t];
       const float p = 1.f / (1.f + __expf(-z));
-      fl[t] = p > thresh ? 1 : 0;
-      const int64_t cc = c0 + t;
-      if (cc < g.ncell) {
-        if (flag) flag[cc] = p > thresh ? 1 : 0;
-        if (prob) prob[cc] = p;
-      }
+      const bool hit = p > thresh;
+      if (flag) flag[c] = hit ? 1 : 0;
+      if (prob) prob[c] = p;
+      if (list) compact_warp(hit, c, list, sc);
+      if (plist) append_cells(!hit && sfail, c, plist, &sc->npos);
     }
-    __syncthreads();  // the flags of the tile are written
-    if (list && warp < 8)
-      compact_warp(lane < 16 && fl[warp * 16 + (lane & 15)] != 0, c0 + warp * 16 + lane, list, sc);
-    if (plist && warp < 8) {
-      const int cl = warp * 16 + (lane & 15);
-      append_cells(lane < 16 && fl[cl] == 0 && sfail[cl] != 0, c0 + cl, plist, &sc->npos);
-    }
-    __syncthreads();  // every read of this buffer, of xe and of the flags done before they are refilled
   }
   if (mma_pending >= 0) {
     // a commit not observed in time: wait once more (bounded) before the columns are freed
     const long long t0 = clock64();
-    while (!mbar_try_wait(bar + 2, (unsigned)mma_pending))
-      if (clock64() - t0 > kWaitCycles) break;
-  }
-  // timeout path: no new copies were issued after the failed wait; drain those
-  // still in flight (bounded) before the block's shared memory is released
-  for (int bb = 0; bb < 2; ++bb) {
-    if (!((pend >> bb) & 1u)) continue;
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar + bb, (par >> bb) & 1u))
+    while (!mbar_try_wait(bar, (unsigned)mma_pending))
       if (clock64() - t0 > kWaitCycles) break;
   }
   tc::fence_before_sync();
@@ -817,77 +869,46 @@ int mlp_set_weights(Ctx& c, const float* theta_dev, int nin, float thresh) {
   return cudaDeviceSynchronize() == cudaSuccess ? 0 : -3;
 }
 
-// shared memory of k_mlp_staged for nrs staged rows and nbuf tile buffers
-template <int KP>
-static size_t staged_smem(int nrs, int nbuf) {
-  return (size_t)nbuf * (nrs + 32) * 512 + 128 + (size_t)HID * KP * 2 + (size_t)HID * HID * 2 + (size_t)128 * KP * 2 +
-         (3 * HID + 1) * sizeof(float) + 512 * sizeof(float) + 256;
+template <int KP, bool GLM>
+static constexpr size_t tile_smem() {
+  return (size_t)HID * KP * 2 + (size_t)HID * HID * 2 + (size_t)128 * KP * 2 +
+         (2 * (GLM ? 4 : 3) * 128 + 2 * 128 + 3 * HID + 2) * sizeof(float) + 16;
 }
 
-// threads per block of the staged kernel: two per cell of the 128-cell tile
-// (measured at 256^3: four per cell, 512 threads, 3.97 against 3.92 ms per
-// stage; two tile buffers at one block per SM 6.8 ms)
-constexpr int kStagedThreads = 256;
-
-// the staged kernel applies: FP32 form, uniform 3D mesh, x-rows of whole
-// 128-cell tiles, and the shared memory fits. Two tile buffers only where two
-// blocks still fit on an SM: measured at degree 2, one double-buffered block
-// of 4 warps per SM is twice as slow as two single-buffered ones (the feature
-// code needs the warps to hide its latencies).
-template <int KP>
-static bool staged_ok(const Ctx& c, int* nrs, int* nbuf) {
+// the tiled kernel applies: FP32 form, uniform 3D mesh, x-rows of whole 128-cell
+// tiles (other meshes keep k_mlp_infer: the two sum the layers in another order,
+// and a probability near the threshold must not change sides with the kernel)
+static bool tile_ok(const Ctx& c) {
   const Geom& g = c.g;
-  if (c.p.precision != DG_PREC_FP32MIX || c.amr.on || g.D != 3 || g.nx % 128 != 0) return false;
-  *nrs = g.glm ? 8 * g.n : g.nrows;
-  *nbuf = 2 * (staged_smem<KP>(*nrs, 2) + 1024) <= 228 * 1024 ? 2 : 1;
-  return staged_smem<KP>(*nrs, *nbuf) <= 227 * 1024;
+  return c.p.precision == DG_PREC_FP32MIX && !c.amr.on && g.D == 3 && g.nx % 128 == 0;
 }
 
 template <int KP, bool GLM, int DEG>
-static void staged_launch(Ctx& c, const void* w, uint8_t* flag, float* prob, cudaStream_t st, int32_t* list,
-                          int nrs, int nbuf, int32_t* plist) {
-  const Geom& g = c.g;
-  const size_t sm = staged_smem<KP>(nrs, nbuf);
-  static size_t attr = 0;
-  if (attr < sm) {
-    cudaFuncSetAttribute(k_mlp_staged<KP, GLM, DEG, kStagedThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sm);
-    attr = sm;
-  }
-  // resident blocks per SM from the SM's shared memory (1 KB reserved per
-  // block) and the kernel's registers
-  static int per_sm = 0;
-  static size_t per_sm_smem = 0;
-  if (per_sm_smem != sm) {
-    per_sm_smem = sm;
-    int dev = 0, smem_sm = 0;
-    cudaFuncAttributes fa;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    per_sm = smem_sm / (int)(sm + 1024);
-    if (cudaFuncGetAttributes(&fa, k_mlp_staged<KP, GLM, DEG, kStagedThreads>) == cudaSuccess && fa.numRegs > 0)
-      per_sm = std::min(per_sm, 65536 / (fa.numRegs * kStagedThreads));
-    per_sm = std::max(per_sm, 1);
-  }
-  // at most four blocks per SM: each holds 128 of the SM's 512 tensor-memory columns
-  const unsigned nb = (unsigned)std::min<int64_t>(g.ncell / 128, (int64_t)c.nsm * std::min(per_sm, 4));
-  k_mlp_staged<KP, GLM, DEG, kStagedThreads><<<nb, kStagedThreads, sm, st>>>(
-      g, c.mlp, (const float*)w, (const __nv_bfloat16*)c.mlp_w1, (const __nv_bfloat16*)c.mlp_w2, c.mlp_bias,
-      c.mlp_thresh, flag, prob, list, c.sc, nrs, nbuf, plist, c.pscr);
+static void tile_launch(Ctx& c, const void* w, uint8_t* flag, float* prob, cudaStream_t st, int32_t* list,
+                        int32_t* plist) {
+  constexpr size_t sm = tile_smem<KP, GLM>();
+  const auto k = k_mlp_tile<KP, GLM, DEG>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  // persistent: the weights are staged once per block. At most four blocks per
+  // SM: each holds 128 of the SM's 512 tensor-memory columns
+  const int per_sm = DEG <= 2 ? 4 : 2;
+  const unsigned nb = (unsigned)std::min<int64_t>(c.g.ncell / 128, (int64_t)c.nsm * per_sm);
+  k<<<nb, kTileThreads, sm, st>>>(c.g, c.mlp, (const float*)w, (const __nv_bfloat16*)c.mlp_w1,
+                                  (const __nv_bfloat16*)c.mlp_w2, c.mlp_bias, c.mlp_thresh, flag, prob, list, c.sc,
+                                  plist, c.pscr);
 }
 
 template <typename T, int KP>
 static void infer_launch(Ctx& c, const void* w, const double* wmean, uint8_t* flag, float* prob, cudaStream_t st,
                          int32_t* list, int32_t* plist, bool* screened) {
-  int nrs = 0, nbuf = 1;
   if constexpr (sizeof(T) == 4) {
-    if (staged_ok<KP>(c, &nrs, &nbuf)) {
+    if (tile_ok(c)) {
       // compile-time feature code for the scheme and degree (KP follows the degree)
       constexpr int DEG = KP == 64 ? 1 : KP == 112 ? 2 : KP == 192 ? 3 : 0;
       if constexpr (DEG > 0) {
         if (c.g.d == DEG) {
-          if (c.g.glm) staged_launch<KP, true, DEG>(c, w, flag, prob, st, list, nrs, nbuf, plist);
-          else staged_launch<KP, false, DEG>(c, w, flag, prob, st, list, nrs, nbuf, plist);
+          if (c.g.glm) tile_launch<KP, true, DEG>(c, w, flag, prob, st, list, plist);
+          else tile_launch<KP, false, DEG>(c, w, flag, prob, st, list, plist);
           if (screened) *screened = plist != nullptr;
           return;
         }

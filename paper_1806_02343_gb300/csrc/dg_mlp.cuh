@@ -11,7 +11,7 @@ int mlp_features_launch(Ctx& c, const void* w, const double* wmean, float* X, in
 int mlp_set_weights(Ctx& c, const float* theta_dev, int nin, float thresh);
 // flag / prob / list may be null; with list, the flagged cells are appended to
 // list[0 .. c.sc->nflag) (the caller zeroes nflag first). With pos_list (FP32
-// form), the staged kernel also runs the FP32 positivity screen on the cells
+// form), the tiled kernel also runs the FP32 positivity screen on the cells
 // it does not flag and appends those that do not clear it to
 // pos_list[0 .. c.sc->npos) (the caller zeroes npos first and screens the
 // flagged cells after limiting them); *screened tells whether it did.

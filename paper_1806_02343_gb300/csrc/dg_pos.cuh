@@ -1,6 +1,6 @@
 // FP32 positivity screen (Sec. 4.3), shared by the screen kernel of the
-// limiter and the staged learned indicator, which holds every row of its cells
-// in shared memory already.
+// limiter and the tiled learned indicator, which holds every row of its cells in
+// registers already.
 #pragma once
 #include "dg_ctx.h"
 #include "dg_ldf.cuh"
@@ -14,6 +14,27 @@ __host__ __device__ __forceinline__ int screen_mean_row(const Geom& g, int k) {
   if (g.glm || k < 5) return k * g.n;
   if (g.D == 3) return g.ldf0 + (k - 5);
   return k < 7 ? g.ldf0 + (k - 5) : g.bz2d;
+}
+
+// The end of pos_screen_rows: means mt and deviation bounds dv of the 8 variables
+__device__ __forceinline__ bool pos_screen_bound(const PosScreen& ps, const float* mt, float* dv) {
+  const float mg = 1e-4f;
+#pragma unroll
+  for (int v = 0; v < 8; ++v) dv[v] = dv[v] * (1.f + mg) + mg * fabsf(mt[v]);
+  const float rlo = mt[0] - dv[0];
+  if (rlo > ps.eps_rho * 2.f) {
+    float kin = 0.f, mag = 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const float mu = fabsf(mt[1 + i]) + dv[1 + i];
+      const float bu = fabsf(mt[5 + i]) + dv[5 + i];
+      kin += mu * mu;
+      mag += bu * bu;
+    }
+    const float plo = ps.gm1 * (mt[4] - dv[4] - 0.5f * kin / rlo - 0.5f * mag);
+    if (plo > ps.eps_p * 2.f + mg * fabsf(mt[4])) return true;
+  }
+  return false;
 }
 
 // Rigorous screen in FP32 from the float mirror of the means: |P_l| <= 1 and
@@ -52,23 +73,7 @@ __device__ __forceinline__ bool pos_screen_rows(const Geom& g, const PosScreen& 
     if (g.bz2d >= 0)
       for (int l = 1; l < g.n; ++l) dv[7] += fabsf(row(g.bz2d + l));
   }
-  const float mg = 1e-4f;
-#pragma unroll
-  for (int v = 0; v < 8; ++v) dv[v] = dv[v] * (1.f + mg) + mg * fabsf(mt[v]);
-  const float rlo = mt[0] - dv[0];
-  if (rlo > ps.eps_rho * 2.f) {
-    float kin = 0.f, mag = 0.f;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const float mu = fabsf(mt[1 + i]) + dv[1 + i];
-      const float bu = fabsf(mt[5 + i]) + dv[5 + i];
-      kin += mu * mu;
-      mag += bu * bu;
-    }
-    const float plo = ps.gm1 * (mt[4] - dv[4] - 0.5f * kin / rlo - 0.5f * mag);
-    if (plo > ps.eps_p * 2.f + mg * fabsf(mt[4])) return true;
-  }
-  return false;
+  return pos_screen_bound(ps, mt, dv);
 }
 
 // Point-wise screen in FP32, 3D degrees 1 and 2: the state at every volume and
