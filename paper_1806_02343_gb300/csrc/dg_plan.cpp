@@ -6,7 +6,6 @@
 
 #include <algorithm>
 #include <numeric>
-#include <thread>
 #include <utility>
 
 #include "../../include/dg_mhd.h"
@@ -91,27 +90,43 @@ inline uint64_t leaf_key(int l, const int32_t* k, int D) {
 
 }  // namespace
 
-int morton_index(int D, int64_t N, const int8_t* level, const int32_t* ijk, MortonIndex& mi, bool partial) {
+int morton_index(HostTeam& team, int D, int64_t N, const int8_t* level, const int32_t* ijk, MortonIndex& mi,
+                 bool partial) {
   if ((D != 2 && D != 3) || N < 1 || N > ((int64_t)1 << 30) || !level || !ijk) return DG_E_ARG;
   mi = MortonIndex{};
   mi.D = D;
   mi.N = N;
-  int lmax = 0;
-  for (int64_t i = 0; i < N; ++i) {
-    const int l = level[i];
-    if (l < 0 || l > kMaxLevel) return DG_E_MESH;
-    for (int a = 0; a < D; ++a)
-      if (ijk[i * D + a] < 0 || ijk[i * D + a] >= (1 << l)) return DG_E_MESH;
-    lmax = std::max(lmax, l);
-  }
+  const int np = team.size();
+  std::vector<int> lmaxp((size_t)np, 0);
+  std::vector<char> bad((size_t)np, 0), unsorted((size_t)np, 0);
+  auto any = [](const std::vector<char>& x) { return std::find(x.begin(), x.end(), 1) != x.end(); };
+  team.ranges(N, [&](int t, int64_t i0, int64_t i1) {
+    int lm = 0;
+    for (int64_t i = i0; i < i1; ++i) {
+      const int l = level[i];
+      bool ok = l >= 0 && l <= kMaxLevel;
+      for (int a = 0; a < D && ok; ++a) ok = ijk[i * D + a] >= 0 && ijk[i * D + a] < (1 << l);
+      if (!ok) {
+        bad[t] = 1;
+        return;
+      }
+      lm = std::max(lm, l);
+    }
+    lmaxp[t] = lm;
+  });
+  if (any(bad)) return DG_E_MESH;
+  const int lmax = *std::max_element(lmaxp.begin(), lmaxp.end());
   mi.lmax = lmax;
   mi.R = lmax + 1;
   std::vector<uint64_t> code((size_t)N);
-  bool sorted = true;
-  for (int64_t i = 0; i < N; ++i) {
-    code[i] = morton(D, mi.R, level[i], &ijk[i * D]);
-    if (i > 0 && code[i] <= code[i - 1]) sorted = false;
-  }
+  team.ranges(N, [&](int t, int64_t i0, int64_t i1) {
+    for (int64_t i = i0; i < i1; ++i) {
+      code[i] = morton(D, mi.R, level[i], &ijk[i * D]);
+      if (i > i0 && code[i] <= code[i - 1]) unsorted[t] = 1;
+    }
+  });
+  bool sorted = !any(unsorted);
+  for (int t = 1; t < np; ++t) sorted = sorted && code[N * t / np] > code[N * t / np - 1];
   if (sorted) {
     mi.start.swap(code);
     mi.lev.assign(level, level + N);
@@ -131,12 +146,16 @@ int morton_index(int D, int64_t N, const int8_t* level, const int32_t* ijk, Mort
   // the leaves tile the cube iff, in Morton order, each starts where the one
   // before it ends (a leaf of level l spans 2^(D (R - l)) codes) and the last
   // ends at 2^(D R)
-  uint64_t next = 0;
-  for (int64_t p = 0; p < N; ++p) {
-    if (partial ? mi.start[p] < next : mi.start[p] != next) return DG_E_MESH;  // overlap (or a hole)
-    next = mi.start[p] + (1ull << (D * (mi.R - mi.lev[p])));
-  }
-  if (!partial && next != 1ull << (D * mi.R)) return DG_E_MESH;
+  auto end_of = [&](int64_t p) { return p < 0 ? 0ull : mi.start[p] + (1ull << (D * (mi.R - mi.lev[p]))); };
+  team.ranges(N, [&](int t, int64_t p0, int64_t p1) {
+    uint64_t next = end_of(p0 - 1);
+    for (int64_t p = p0; p < p1; ++p) {
+      if (partial ? mi.start[p] < next : mi.start[p] != next) bad[t] = 1;  // overlap (or a hole)
+      next = end_of(p);
+    }
+  });
+  if (any(bad)) return DG_E_MESH;
+  if (!partial && end_of(N - 1) != 1ull << (D * mi.R)) return DG_E_MESH;
   return DG_OK;
 }
 
@@ -165,11 +184,11 @@ bool mesh_balanced(const MortonIndex& mi, const int32_t* ijk) {
   return true;
 }
 
-int octree_faces(int D, int64_t N, const int8_t* level, const int32_t* ijk, MortonIndex& mi,
+int octree_faces(HostTeam& team, int D, int64_t N, const int8_t* level, const int32_t* ijk, MortonIndex& mi,
                  std::vector<int32_t>& fL, std::vector<int32_t>& fR, std::vector<int32_t>& fmeta,
                  std::vector<int32_t>& cstart, std::vector<int32_t>& centry, int& maxent, bool partial) {
   if (N < 1 || N > ((int64_t)1 << 30)) return DG_E_MESH;
-  if (morton_index(D, N, level, ijk, mi, partial) != DG_OK) return DG_E_MESH;
+  if (morton_index(team, D, N, level, ijk, mi, partial) != DG_OK) return DG_E_MESH;
   // the leaf at Morton position q holds the code (always, on a full mesh)
   auto holds = [&](int64_t q, uint64_t code) {
     return mi.start[q] <= code && code - mi.start[q] < (1ull << (D * (mi.R - mi.lev[q])));
@@ -250,65 +269,62 @@ int octree_faces(int D, int64_t N, const int8_t* level, const int32_t* ijk, Mort
     }
       return DG_OK;
   };
-  // The leaves are split into contiguous chunks searched by parallel host
-  // threads; each chunk lists its faces in leaf order and the chunks are
+  // The leaves are split into contiguous parts searched by parallel host
+  // threads; each part lists its faces in leaf order and the parts are
   // concatenated in order, so the lists do not depend on the thread count.
   struct Part {
     std::vector<int32_t> L, R, M;
     int err = DG_OK;
+    size_t at = 0;
   };
-  const int64_t kChunk = 1 << 16;
-  const int nth = (int)std::max<int64_t>(
-      1, std::min<int64_t>({(int64_t)std::max(1u, std::thread::hardware_concurrency()), 16, (N + kChunk - 1) / kChunk}));
-  std::vector<Part> parts((size_t)nth);
-  auto work = [&](int t) {
+    std::vector<Part> parts((size_t)team.size());
+  team.ranges(N, [&](int t, int64_t c0, int64_t c1) {
     Part& P = parts[(size_t)t];
-    const int64_t c0 = N * t / nth, c1 = N * (t + 1) / nth;
     P.L.reserve((size_t)((c1 - c0) * D + (c1 - c0) / 2));
     P.R.reserve(P.L.capacity());
     P.M.reserve(P.L.capacity());
     for (int64_t cidx = c0; cidx < c1 && P.err == DG_OK; ++cidx) P.err = faces_of_leaf(cidx, P.L, P.R, P.M);
-  };
-  {
-    std::vector<std::thread> pool;
-    for (int t = 1; t < nth; ++t) pool.emplace_back(work, t);
-    work(0);
-    for (auto& th : pool) th.join();
-  }
+  });
   size_t total = 0;
-  for (const Part& P : parts) {
+  for (Part& P : parts) {
     if (P.err != DG_OK) return P.err;
+    P.at = total;
     total += P.L.size();
   }
-  fL.clear();
-  fR.clear();
-  fmeta.clear();
-  fL.reserve(total);
-  fR.reserve(total);
-  fmeta.reserve(total);
-  for (const Part& P : parts) {
-    fL.insert(fL.end(), P.L.begin(), P.L.end());
-    fR.insert(fR.end(), P.R.begin(), P.R.end());
-    fmeta.insert(fmeta.end(), P.M.begin(), P.M.end());
-  }
-  // per-cell entries in face order (counting sort)
-  const int64_t nf = (int64_t)fL.size();
+  fL.resize(total);
+  fR.resize(total);
+  fmeta.resize(total);
+  team.ranges(N, [&](int t, int64_t, int64_t) {
+    const Part& P = parts[(size_t)t];
+    std::copy(P.L.begin(), P.L.end(), fL.begin() + P.at);
+    std::copy(P.R.begin(), P.R.end(), fR.begin() + P.at);
+    std::copy(P.M.begin(), P.M.end(), fmeta.begin() + P.at);
+  });
+  // per-cell entries in face order (counting sort): every part walks all faces and
+  // counts, then places, the entries of its own cells
+  const int64_t nf = (int64_t)total;
   cstart.assign((size_t)N + 1, 0);
-  for (int64_t f = 0; f < nf; ++f) {
-    ++cstart[fL[f] + 1];
-    ++cstart[fR[f] + 1];
-  }
+  team.ranges(N, [&](int, int64_t c0, int64_t c1) {
+    const uint64_t len = (uint64_t)(c1 - c0);
+    for (int64_t f = 0; f < nf; ++f) {
+      if ((uint64_t)(fL[f] - c0) < len) ++cstart[fL[f] + 1];
+      if ((uint64_t)(fR[f] - c0) < len) ++cstart[fR[f] + 1];
+    }
+  });
   maxent = 0;
   for (int64_t c = 0; c < N; ++c) {
     maxent = std::max(maxent, cstart[c + 1]);
     cstart[c + 1] += cstart[c];
   }
-  centry.assign((size_t)cstart[N], 0);
-  std::vector<int32_t> fill(cstart.begin(), cstart.end() - 1);
-  for (int64_t f = 0; f < nf; ++f) {
-    centry[fill[fL[f]]++] = (int32_t)(f << 1);
-    centry[fill[fR[f]]++] = (int32_t)((f << 1) | 1);
-  }
+  centry.resize((size_t)cstart[N]);
+  team.ranges(N, [&](int, int64_t c0, int64_t c1) {
+    const uint64_t len = (uint64_t)(c1 - c0);
+    std::vector<int32_t> fill(cstart.begin() + c0, cstart.begin() + c1);
+    for (int64_t f = 0; f < nf; ++f) {
+      if ((uint64_t)(fL[f] - c0) < len) centry[fill[fL[f] - c0]++] = (int32_t)(f << 1);
+      if ((uint64_t)(fR[f] - c0) < len) centry[fill[fR[f] - c0]++] = (int32_t)((f << 1) | 1);
+    }
+  });
   return DG_OK;
 }
 
@@ -498,7 +514,8 @@ void plan_mesh(const MortonIndex& mi, const int32_t* ijk, const std::vector<int3
 namespace {
 
 int index_checked(int dim, int64_t n, const int8_t* level, const int32_t* ijk, dgmhd::MortonIndex& mi) {
-  const int e = dgmhd::morton_index(dim, n, level, ijk, mi);
+  dgmhd::HostTeam team(n);
+  const int e = dgmhd::morton_index(team, dim, n, level, ijk, mi);
   if (e) return e;
   return dgmhd::mesh_balanced(mi, ijk) ? DG_OK : DG_E_MESH;
 }
@@ -556,7 +573,8 @@ extern "C" int dg_mhd_octree_faces(int dim, int64_t n, const int8_t* level, cons
   dgmhd::MortonIndex mi;
   std::vector<int32_t> fL, fR, fmeta, cstart, centry;
   int maxent = 0;
-  const int e = dgmhd::octree_faces(dim, n, level, ijk, mi, fL, fR, fmeta, cstart, centry, maxent, partial != 0);
+  dgmhd::HostTeam team(n);
+  const int e = dgmhd::octree_faces(team, dim, n, level, ijk, mi, fL, fR, fmeta, cstart, centry, maxent, partial != 0);
   if (e) return e;
   const int64_t nf = (int64_t)fL.size();
   *n_faces = nf;

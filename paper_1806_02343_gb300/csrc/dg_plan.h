@@ -6,9 +6,100 @@
 #pragma once
 #include <stdint.h>
 
+#include <algorithm>
+#include <condition_variable>
+#include <exception>
+#include <functional>
+#include <mutex>
+#include <thread>
+#include <utility>
 #include <vector>
 
 namespace dgmhd {
+
+// Host threads for the passes over a mesh of n leaves: one per 8192 leaves, at
+// most 16 (8192 leaves are 0.2 ms of face search, several times a hand-over). The
+// team lives for one call of the code that builds a mesh: starting 15 threads
+// takes 0.4 ms, as long as a pass over 150,000 leaves, so they are not started
+// for every pass.
+class HostTeam {
+ public:
+  explicit HostTeam(int64_t n) {
+    const int64_t hw = std::max(1u, std::thread::hardware_concurrency());
+    const int want = (int)std::max<int64_t>(1, std::min<int64_t>({hw, 16, n / 8192}));
+    err_.resize((size_t)want);
+    pool_.reserve((size_t)want);
+    for (int t = 1; t < want; ++t) {
+      try {
+        pool_.emplace_back([this, t] { serve(t); });
+      } catch (...) {
+        break;  // no more threads to be had: a smaller team
+      }
+    }
+  }
+  HostTeam(const HostTeam&) = delete;
+  HostTeam& operator=(const HostTeam&) = delete;
+  ~HostTeam() {
+    {
+      std::lock_guard<std::mutex> l(m_);
+      quit_ = true;
+    }
+    go_.notify_all();
+    for (auto& th : pool_) th.join();
+  }
+  int size() const { return (int)pool_.size() + 1; }
+  // f(part, first, end) on contiguous parts of [0, n), one per thread, the first
+  // on the caller; an exception of a part is rethrown here once all are done
+  void ranges(int64_t n, const std::function<void(int, int64_t, int64_t)>& f) {
+    const int np = size();
+    const std::function<void(int)> part = [&](int t) { f(t, n * t / np, n * (t + 1) / np); };
+    {
+      std::lock_guard<std::mutex> l(m_);
+      job_ = &part;
+      left_ = np - 1;
+      ++round_;
+    }
+    if (np > 1) go_.notify_all();
+    call(0);
+    {
+      std::unique_lock<std::mutex> l(m_);
+      done_.wait(l, [&] { return left_ == 0; });
+    }
+    for (auto& e : err_)
+      if (e) std::rethrow_exception(std::exchange(e, nullptr));
+  }
+
+ private:
+  void call(int t) {
+    try {
+      (*job_)(t);
+    } catch (...) {
+      err_[(size_t)t] = std::current_exception();
+    }
+  }
+  void serve(int t) {
+    unsigned seen = 0;
+    for (;;) {
+      {
+        std::unique_lock<std::mutex> l(m_);
+        go_.wait(l, [&] { return quit_ || round_ != seen; });
+        if (quit_) return;
+        seen = round_;
+      }
+      call(t);
+      std::lock_guard<std::mutex> l(m_);
+      if (--left_ == 0) done_.notify_one();
+    }
+  }
+  std::mutex m_;
+  std::condition_variable go_, done_;
+  const std::function<void(int)>* job_ = nullptr;
+  int left_ = 0;
+  unsigned round_ = 0;
+  bool quit_ = false;
+  std::vector<std::exception_ptr> err_;
+  std::vector<std::thread> pool_;
+};
 
 // The leaves in Morton (Z-curve) order of their lower corners, with those
 // corners' Morton codes at resolution level R = (finest level) + 1, one more
@@ -30,7 +121,8 @@ struct MortonIndex {
 // cube without overlap: DG_OK, else DG_E_MESH (DG_E_ARG for a bad dim / count).
 // partial: the leaves need not cover the cube (a partition's owned and ghost
 // leaves); they still must not overlap.
-int morton_index(int D, int64_t N, const int8_t* level, const int32_t* ijk, MortonIndex& mi, bool partial = false);
+int morton_index(HostTeam& team, int D, int64_t N, const int8_t* level, const int32_t* ijk, MortonIndex& mi,
+                 bool partial = false);
 
 // No two face neighbours differ by more than one level (periodic box).
 bool mesh_balanced(const MortonIndex& mi, const int32_t* ijk);
@@ -47,7 +139,7 @@ bool mesh_balanced(const MortonIndex& mi, const int32_t* ijk);
 // partial: a partition's local mesh; a face whose neighbour region holds no
 // leaf is left out (only ghost cells, whose results are discarded, have such
 // faces), and the 2:1 checks apply to the leaves present.
-int octree_faces(int D, int64_t N, const int8_t* level, const int32_t* ijk, MortonIndex& mi,
+int octree_faces(HostTeam& team, int D, int64_t N, const int8_t* level, const int32_t* ijk, MortonIndex& mi,
                  std::vector<int32_t>& fL, std::vector<int32_t>& fR, std::vector<int32_t>& fmeta,
                  std::vector<int32_t>& cstart, std::vector<int32_t>& centry, int& maxent, bool partial = false);
 

@@ -394,7 +394,8 @@ int ensure_groups(Ctx& c) {
   const int D = h.D, no = 1 << D;
   const int64_t N = (int64_t)h.hlevel.size();
   if (h.morton.N != N) {  // built with the face lists at init
-    const int e = morton_index(D, N, h.hlevel.data(), h.hijk.data(), h.morton);
+    HostTeam team(N);
+    const int e = morton_index(team, D, N, h.hlevel.data(), h.hijk.data(), h.morton);
     if (e) return e;
   }
   sibling_groups(h.morton, h.hijk.data(), h.hgroups);
