@@ -979,21 +979,59 @@ __global__ void __launch_bounds__(NTP, 3) k_cell_pow(const FastGeom g, const T* 
 // and store instruction touched 32 sectors: per stage on 1,387,520 leaves, face
 // pass 2.45 -> 1.33 ms, cell pass 3.13 -> 2.96 ms, the timestep's jumps 0.38 ->
 // 0.31 ms.)
+template <typename T, int NC>
+__device__ __forceinline__ void load_row(const T* p, T (&r)[NC]) {
+  if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int k = 0; k < NC; k += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(p + k);
+      r[k] = x.x;
+      r[k + 1] = x.y;
+      r[k + 2] = x.z;
+      r[k + 3] = x.w;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < NC; ++k) r[k] = p[k];
+  }
+}
+
+// stride of a mode's points in the staged trace tables: whole 16-byte words in
+// FP32 (per mode 2 loads of four points and one of the ninth instead of 5 pairs:
+// face pass 1.32 -> 1.12 ms on 1,387,520 leaves)
+template <typename T, int DEG>
+constexpr int list_pts() {
+  return sizeof(T) == 4 ? (FastDims<DEG>::QF + 3) / 4 * 4 : FaceTabs<T, DEG>::QFP;
+}
 template <typename T, int DEG>
 __device__ __forceinline__ void face_trace_smem(const T (&wl)[FastDims<DEG>::N], const T* Pt, T* out) {
-  constexpr int N = FastDims<DEG>::N, QF = FastDims<DEG>::QF, QFP = FaceTabs<T, DEG>::QFP;
+  constexpr int N = FastDims<DEG>::N, QF = FastDims<DEG>::QF, QS = list_pts<T, DEG>();
+  constexpr int G = sizeof(T) == 4 ? 4 : 2;  // points per load
 #pragma unroll
-  for (int p = 0; p + 1 < QF; p += 2) {
-    T a0 = T(0), a1 = T(0);
+  for (int p = 0; p + G <= QF; p += G) {
+    T a[G];
 #pragma unroll
-    for (int l = 0; l < N; ++l) fma2(a0, a1, wl[l], wl[l], Pt[l * QFP + p], Pt[l * QFP + p + 1]);
-    out[p * 8 * TC] = a0;
-    out[(p + 1) * 8 * TC] = a1;
+    for (int k = 0; k < G; ++k) a[k] = T(0);
+#pragma unroll
+    for (int l = 0; l < N; ++l) {
+      T x[G];
+      if constexpr (G == 4) {
+        load_row<T, 4>(Pt + l * QS + p, x);
+      } else {
+        x[0] = Pt[l * QS + p];
+        x[1] = Pt[l * QS + p + 1];
+      }
+#pragma unroll
+      for (int k = 0; k < G; k += 2) fma2(a[k], a[k + 1], wl[l], wl[l], x[k], x[k + 1]);
+    }
+#pragma unroll
+    for (int k = 0; k < G; ++k) out[(p + k) * 8 * TC] = a[k];
   }
-  if (QF & 1) {
+  static_assert(QF % G <= 1, "at most one point left");
+  if (QF % G) {
     T acc = T(0);
 #pragma unroll
-    for (int l = 0; l < N; ++l) acc = fma_rn(wl[l], Pt[l * QFP + QF - 1], acc);
+    for (int l = 0; l < N; ++l) acc = fma_rn(wl[l], Pt[l * QS + QF - 1], acc);
     out[(QF - 1) * 8 * TC] = acc;
   }
 }
@@ -1029,8 +1067,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && DEG <= 2) ? 4 : 2) k_fa
   constexpr int N = FastDims<DEG>::N, QF = FastDims<DEG>::QF, NDIV = PowDims<DEG>::NDIV, NRP = 5 * N + NDIV;
   constexpr int QFP = FaceTabs<T, DEG>::QFP;
   extern __shared__ __align__(16) unsigned char smraw[];
-  T* TT = reinterpret_cast<T*>(smraw);  // [2][N][QFP] the type's left / right trace tables
-  T* WL = TT + 2 * N * QFP;             // [NRP][TC]
+  constexpr int QS = list_pts<T, DEG>();
+  T* TT = reinterpret_cast<T*>(smraw);  // [2][N][QS] the type's left / right trace tables
+  T* WL = TT + 2 * N * QS;              // [NRP][TC]
   T* WR = WL + NRP * TC;                // [NRP][TC]
   T* TRC = WR + NRP * TC;               // [2][QF][8][TC]
   const int t = threadIdx.x;
@@ -1048,7 +1087,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && DEG <= 2) ? 4 : 2) k_fa
   const int64_t fid = face;
   const int64_t cL = live ? o.fL[fid] : 0, cR = live ? o.fR[fid] : 0;
   const int64_t S = o.stride;
-  for (int i = t; i < 2 * N * QFP; i += NT) TT[i] = o.ftab[(size_t)type * 2 * N * QFP + i];
+  for (int i = t; i < 2 * N * QFP; i += NT) TT[i / QFP * QS + i % QFP] = o.ftab[(size_t)type * 2 * N * QFP + i];
   {
     constexpr int PER = (NRP + 8) / 9;
     T a[PER], b[PER];
@@ -1082,7 +1121,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && DEG <= 2) ? 4 : 2) k_fa
       } else {
         ldf_to_legendre<T, DEG>(v - 5, W + 5 * N * TC + f, wl);
       }
-      face_trace_smem<T, DEG>(wl, TT + s * N * QFP, TRC + (s * QF * 8 + v) * TC + f);
+      face_trace_smem<T, DEG>(wl, TT + s * N * QS, TRC + (s * QF * 8 + v) * TC + f);
     }
   }
   __syncthreads();
@@ -1091,6 +1130,13 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && DEG <= 2) ? 4 : 2) k_fa
   else list_hlld<T, DEG, 2>(TRC, v, f, live, fid, gamma, eps, F);
 }
 
+// stride of a table row of the list kernels' own-side tables: whole 16-byte words
+// in FP32 (half the shared-memory load instructions of pair loads; with the next
+// entry's loads in flight the cell pass went from 3.00 to 2.95 ms on 1,387,520 leaves)
+template <typename T, int DEG>
+constexpr int list_row() {
+  return sizeof(T) == 4 ? (FastDims<DEG>::N + 3) / 4 * 4 : FastDims<DEG>::N;
+}
 template <typename T, int DEG>
 __global__ void __launch_bounds__(NTP, 3) k_cell_list_pow(const OctPow<T> o, T gamma, const T* __restrict__ w,
                                                           const T* __restrict__ F, T* out, const T* w0, double ca,
@@ -1107,14 +1153,15 @@ __global__ void __launch_bounds__(NTP, 3) k_cell_list_pow(const OctPow<T> o, T g
   T* PR = reinterpret_cast<T*>(smraw);
   T* LS = PR + QC * NSL * TC;
   T* QM = LS + NDIV * TC;
-  T* CT = QM + 8 * TC;  // [NCT][QF][N] weighted own-side tables
+  constexpr int NC = list_row<T, DEG>();
+  T* CT = QM + 8 * TC;  // [NCT][QF][NC] weighted own-side tables
   const int t = threadIdx.x;
   const int f = t & (TC - 1);
   const int v = t >> 5;
   const int64_t c = (int64_t)blockIdx.x * TC + f;
   const bool live = c < o.ncell;
   const int64_t S = o.stride;
-  for (int i = t; i < NCT * QF * N; i += NTP) CT[i] = o.ctab[i];
+  for (int i = t; i < NCT * QF * N; i += NTP) CT[i / N * NC + i % N] = o.ctab[i];
   T wl[N], racc[N];
   pow_load<T, DEG>(w, S, c, live, v, f, LS, QM, wl);  // (its barrier covers CT)
   pow_volume<T, DEG>(wl, PR, gamma, v, f, racc);
@@ -1125,28 +1172,44 @@ __global__ void __launch_bounds__(NTP, 3) k_cell_list_pow(const OctPow<T> o, T g
   T hi = T(0), lo = T(0);
   if (live) {
     const int e1 = o.cstart[c + 1];
-    for (int e = o.cstart[c]; e < e1; ++e) {
-      const int ent = o.centry[e];
+    // an entry's face, type and values are three dependent loads: FP32 issues those
+    // of the next entry while this one is contracted (FP64 has no registers for it,
+    // and is bound by its multiply-add rate)
+    constexpr bool PRE = sizeof(T) == 4;
+    T Fn[QF], Bn[QF];
+    int ent = 0, type = 0;
+    auto fetch = [&](int e) {
+      ent = o.centry[e];
       const int64_t blk = ent >> 6;
+      type = o.btype[blk] & 255;
+      const T* q = F + blk * QF * NFS * TC + ((ent >> 1) & 31);
+#pragma unroll
+      for (int p = 0; p < QF; ++p) Fn[p] = q[(p * NFS + v) * TC];
+      if (v > 0) {
+#pragma unroll
+        for (int p = 0; p < QF; ++p) Bn[p] = q[(p * NFS + 8 + (ent & 1)) * TC];
+      }
+    };
+    int e = o.cstart[c];
+    if (PRE && e < e1) fetch(e);
+    while (e < e1) {
+      if (!PRE) fetch(e);
       const int side = ent & 1;  // 0: this cell is the face's left cell (its +a face)
-      const int type = o.btype[blk] & 255;
       const int a = type / 9, k = type % 9;  // k: 0 same level, 1 + sub left coarse, 5 + sub right coarse
       const int fo = side == 0 ? 2 * a + 1 : 2 * a;
       const bool coarse = side == 0 ? (k >= 1 && k <= 4) : k >= 5;
-      const T* Pt = CT + (coarse ? 6 + fo * 4 + ((k - 1) & 3) : fo) * QF * N;
-      const T* q = F + blk * QF * NFS * TC + ((ent >> 1) & 31);
+      const T* Pt = CT + (coarse ? 6 + fo * 4 + ((k - 1) & 3) : fo) * QF * NC;
       T Fp[QF];
 #pragma unroll
-      for (int p = 0; p < QF; ++p) Fp[p] = q[(p * NFS + v) * TC];
-      if (v > 0) {
-#pragma unroll
-        for (int p = 0; p < QF; ++p) Fp[p] = fma_rn(qv, q[(p * NFS + 8 + side) * TC], Fp[p]);
-      }
+      for (int p = 0; p < QF; ++p) Fp[p] = v > 0 ? fma_rn(qv, Bn[p], Fn[p]) : Fn[p];
+      ++e;
+      if (PRE && e < e1) fetch(e);
       T fs = T(0);
 #pragma unroll
       for (int p = 0; p < QF; ++p) {
         const T Fv = side == 0 ? -Fp[p] : Fp[p];
-        const T* Pw = Pt + p * N;
+        T Pw[NC];
+        load_row<T, NC>(Pt + p * NC, Pw);
         fma2(fs, racc[1], Fv, Fv, Pw[0], Pw[1]);
 #pragma unroll
         for (int l = 2; l + 1 < N; l += 2) fma2(racc[l], racc[l + 1], Fv, Fv, Pw[l], Pw[l + 1]);
@@ -1451,8 +1514,8 @@ void launch_divb_face_pow(const FastGeom& g, const T* w, T* jbuf, cudaStream_t s
 template <typename T, int DEG>
 void launch_face_list_pow(const OctPow<T>& o, double gamma, const T* w, T* F, double eps, cudaStream_t st) {
   constexpr int N = FastDims<DEG>::N, QF = FastDims<DEG>::QF;
-  constexpr int NDIV = PowDims<DEG>::NDIV, NRP = 5 * N + NDIV, QFP = FaceTabs<T, DEG>::QFP;
-  const size_t smf = (size_t)(2 * N * QFP + 2 * NRP * TC + 2 * QF * 8 * TC) * sizeof(T);
+  constexpr int NDIV = PowDims<DEG>::NDIV, NRP = 5 * N + NDIV;
+  const size_t smf = (size_t)(2 * N * list_pts<T, DEG>() + 2 * NRP * TC + 2 * QF * 8 * TC) * sizeof(T);
   static bool attr = false;
   if (!attr) {
     set_smem_attr<T>((const void*)k_face_list_pow<T, DEG>, smf);
@@ -1467,7 +1530,7 @@ void launch_cell_list_pow(const OctPow<T>& o, double gamma, const T* w, const T*
                           double* outmean, cudaStream_t st) {
   constexpr int N = FastDims<DEG>::N, QF = FastDims<DEG>::QF, QC = FastDims<DEG>::QC;
   constexpr int NDIV = PowDims<DEG>::NDIV;
-  const size_t smc = (size_t)(QC * NSL * TC + NDIV * TC + 8 * TC + 30 * QF * N) * sizeof(T);
+  const size_t smc = (size_t)(QC * NSL * TC + NDIV * TC + 8 * TC + 30 * QF * list_row<T, DEG>()) * sizeof(T);
   static bool attr = false;
   if (!attr) {
     set_smem_attr<T>((const void*)k_cell_list_pow<T, DEG>, smc);
