@@ -170,7 +170,8 @@ namespace {
 constexpr int RG_MAXD = 50;  // LDF rows, degree <= 3
 
 // A non-zero entry of a smoothness form (a: row, b: column; sorted by row) or of
-// a restriction (a: the child's row, b: the parent's; sorted by the child's row)
+// the restriction (a: octant * rows + the child's row, b: the parent's row; sorted
+// by the parent's row)
 struct alignas(16) RgEntry {
   double v;
   int32_t a, b;
@@ -181,11 +182,11 @@ struct RgDev {
   int n, nd, D, no;
   size_t QL, QB, PL, PB, RL, RB;
   // entries of form f: ent[ptr[f] .. ptr[f + 1]); forms: Legendre by direction, LDF by
-  // (component, direction), then the restrictions of the octants, Legendre and LDF
+  // (component, direction), then the restriction, Legendre and LDF
   const RgEntry* ent;
   const int32_t* ptr;
   __host__ __device__ int form(int cc, int a) const { return cc < 0 ? a : D + cc * D + a; }
-  __host__ __device__ int restriction(bool ldf, int o) const { return D + D * D + (ldf ? no : 0) + o; }
+  __host__ __device__ int restriction(bool ldf) const { return D + D * D + (ldf ? 1 : 0); }
 };
 
 // FP64 mean index of row r (mean rows: Legendre mode 0, the D degree-0 LDF
@@ -279,17 +280,22 @@ __global__ void k_rg_marks_leaf(int64_t ncell, const int8_t* __restrict__ level,
 }
 
 // coarsening marks of the sibling groups: the restriction of the group must
-// have S_a < S~/2 for every monitored field and direction. The LDF rows are
-// restricted once for the three components of B, from the non-zero entries of the
-// map (147,456 leaves: once per component and dense 0.71 ms, now 0.56 ms, bound by
-// the latency of the sums in local memory, 4 warps per SM).
+// have S_a < S~/2 for every monitored field and direction. One warp per block, a
+// lane per group, the children's rows in shared memory ([octant][row][lane]): a
+// parent row is one sum in a register over the map's non-zero entries, octants and
+// child rows in order. The LDF rows are restricted once for the components of B.
+// (147,456 leaves: dense and once per component 0.71 ms; entry by entry into sums in
+// local memory 0.56 ms; now 0.45 ms. Eight entries in flight: 0.54 ms.)
 template <typename T>
-__global__ void k_rg_marks_group(Geom g, RgDev L, const T* __restrict__ w, const double* __restrict__ wmean,
-                                 int mask, const int32_t* __restrict__ groups, int64_t ngroups,
-                                 const int8_t* __restrict__ level, double s_tilde, int min_level,
-                                 int8_t* __restrict__ marks) {
-  const int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gi >= ngroups) return;
+__global__ void __launch_bounds__(32) k_rg_marks_group(Geom g, RgDev L, const T* __restrict__ w,
+                                                       const double* __restrict__ wmean, int mask,
+                                                       const int32_t* __restrict__ groups, int64_t ngroups,
+                                                       const int8_t* __restrict__ level, double s_tilde,
+                                                       int min_level, int8_t* __restrict__ marks) {
+  extern __shared__ __align__(16) double X[];
+  const int lane = threadIdx.x;
+  const int64_t gi = (int64_t)blockIdx.x * 32 + lane;
+  if (gi >= ngroups) return;  // (a lane reads only its own column of X)
   const int32_t* mem = groups + gi * L.no;
   if (level[mem[0]] - 1 < min_level) return;
   for (int o = 0; o < L.no; ++o)
@@ -302,20 +308,25 @@ __global__ void k_rg_marks_group(Geom g, RgDev L, const T* __restrict__ w, const
     const bool ldf = rg_field(g, v, &base);
     const int cnt = ldf ? L.nd : L.n;
     if (!(ldf && have)) {
-      for (int l = 0; l < cnt; ++l) coef[l] = 0.0;
       for (int o = 0; o < L.no; ++o) {
-        const int f = L.restriction(ldf, o), e1 = __ldg(L.ptr + f + 1);
-        int m = -1;
-        double x = 0.0;
-        for (int e = __ldg(L.ptr + f); e < e1; ++e) {
-          const RgEntry q = L.ent[e];
-          if (q.a != m) {
-            m = q.a;
-            x = rg_val(g, w, wmean, base + m, (int64_t)mem[o]);
-          }
-          coef[q.b] += q.v * x;
-        }
+        const int64_t c = mem[o];
+#pragma unroll 4
+        for (int m = 0; m < cnt; ++m) X[(o * cnt + m) * 32 + lane] = rg_val(g, w, wmean, base + m, c);
       }
+      for (int l = 0; l < cnt; ++l) coef[l] = 0.0;
+      const int f = L.restriction(ldf), e1 = __ldg(L.ptr + f + 1);
+      int row = 0;
+      double acc = 0.0;
+      for (int e = __ldg(L.ptr + f); e < e1; ++e) {
+        const RgEntry q = L.ent[e];
+        if (q.b != row) {
+          coef[row] = acc;
+          row = q.b;
+          acc = 0.0;
+        }
+        acc += q.v * X[q.a * 32 + lane];
+      }
+      coef[row] = acc;
     }
     have = ldf;
     if (rg_smax(g, L, v, ldf, coef) >= 0.5 * s_tilde) return;
@@ -408,19 +419,28 @@ int ensure_tables(Ctx& c, RgDev& L) {
     std::vector<RgEntry> ent;
     std::vector<int32_t> ptr(1, 0);
     // the dense loops' order; the forms' first rows and columns (no derivative) left out
-    auto add = [&](size_t off, int cnt, int first, bool by_column) {
+    auto form = [&](size_t off, int cnt, int first) {
       for (int i = first; i < cnt; ++i)
         for (int k = first; k < cnt; ++k) {
-          const double x = by_column ? tab[off + (size_t)k * cnt + i] : tab[off + (size_t)i * cnt + k];
+          const double x = tab[off + (size_t)i * cnt + k];
           if (x != 0.0) ent.push_back(RgEntry{x, i, k});
         }
       ptr.push_back((int32_t)ent.size());
     };
+    auto restriction = [&](size_t off, int cnt, int no) {
+      for (int l = 0; l < cnt; ++l)
+        for (int o = 0; o < no; ++o)
+          for (int m = 0; m < cnt; ++m) {
+            const double x = tab[off + ((size_t)o * cnt + l) * cnt + m];
+            if (x != 0.0) ent.push_back(RgEntry{x, o * cnt + m, l});
+          }
+      ptr.push_back((int32_t)ent.size());
+    };
     const int n = lay.n, nd = lay.nd, D = lay.D, no = lay.no;
-    for (int a = 0; a < D; ++a) add(lay.QL + (size_t)a * n * n, n, 1, false);
-    for (int k = 0; k < D * D; ++k) add(lay.QB + (size_t)k * nd * nd, nd, D, false);
-    for (int o = 0; o < no; ++o) add(lay.RL + (size_t)o * n * n, n, 0, true);
-    for (int o = 0; o < no; ++o) add(lay.RB + (size_t)o * nd * nd, nd, 0, true);
+    for (int a = 0; a < D; ++a) form(lay.QL + (size_t)a * n * n, n, 1);
+    for (int k = 0; k < D * D; ++k) form(lay.QB + (size_t)k * nd * nd, nd, D);
+    restriction(lay.RL, n, no);
+    restriction(lay.RB, nd, no);
     tab.resize(pad, 0.0);
     std::vector<char> all(pad * sizeof(double) + ent.size() * sizeof(RgEntry) + ptr.size() * sizeof(int32_t));
     std::memcpy(all.data(), tab.data(), pad * sizeof(double));
@@ -500,13 +520,16 @@ extern "C" int dg_mhd_amr_marks(dg_mhd_ctx* ctx, const void* w, const double* wm
   k_rg_marks_leaf<<<(unsigned)((c.g.ncell + 127) / 128), 128, 0, st>>>(c.g.ncell, c.amr.lev_dev, s_max, s_tilde,
                                                                        max_level, marks);
   if (c.amr.ngroups > 0) {
-    const unsigned nbg = (unsigned)((c.amr.ngroups + 127) / 128);
-    if (c.p.precision == DG_PREC_FP32MIX)
-      k_rg_marks_group<float><<<nbg, 128, 0, st>>>(c.g, L, (const float*)w, wmean, field_mask, c.amr.groups,
-                                                   c.amr.ngroups, c.amr.lev_dev, s_tilde, min_level, marks);
-    else
-      k_rg_marks_group<double><<<nbg, 128, 0, st>>>(c.g, L, (const double*)w, wmean, field_mask, c.amr.groups,
-                                                    c.amr.ngroups, c.amr.lev_dev, s_tilde, min_level, marks);
+    const unsigned nbg = (unsigned)((c.amr.ngroups + 31) / 32);
+    const size_t sm = (size_t)L.no * std::max(L.n, L.nd) * 32 * sizeof(double);  // 53 KB at degree 2, 102 KB at 3
+    auto run = [&](auto k, auto* x) {
+      // (one value for every context: the largest, 8 octants of 50 rows)
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * RG_MAXD * 32 * (int)sizeof(double));
+      k<<<nbg, 32, sm, st>>>(c.g, L, x, wmean, field_mask, c.amr.groups, c.amr.ngroups, c.amr.lev_dev, s_tilde,
+                             min_level, marks);
+    };
+    if (c.p.precision == DG_PREC_FP32MIX) run(k_rg_marks_group<float>, (const float*)w);
+    else run(k_rg_marks_group<double>, (const double*)w);
   }
   return cudaGetLastError() == cudaSuccess ? DG_OK : DG_E_CUDA;
 }
