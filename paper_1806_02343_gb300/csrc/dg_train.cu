@@ -2,13 +2,16 @@
 // network nin -> 64 -> 64 -> 1 (ReLU, sigmoid, weighted cross-entropy; layout of
 // the flat weights in dg_mlp.cu) and Adam steps on shuffled mini-batches.
 //
-// A gradient is two launches. k_train_tile does the forward and backward passes
-// of 32 samples per block entirely in shared memory and leaves the block's
-// share of the gradient in its own row of a scratch matrix; k_train_reduce sums
-// the rows in a fixed order and applies the Adam update. (As eight kernels with
-// one thread per weight walking the batch serially, a 4096-sample step took
-// 1.15 ms, 0.90 of it in the weight gradients; now 0.032 ms: 25 us in the tiles,
-// latency-bound with one 8-warp block per SM, and 7 us in the sum over 128 rows.)
+// A gradient is two launches. k_train_pass does the forward and backward passes of
+// 32 samples per block in shared memory and writes the activations and deltas as
+// [unit][sample]; k_train_grad sums each weight's gradient over the samples, one
+// thread per weight in the order of the samples, and applies the Adam update. Every
+// sum is one chain in a fixed order -- inputs, units and samples ascending -- because
+// Adam divides a gradient by its own size: where a weight's gradient cancels, the
+// rounding of its sum decides the step, and a training of 32 steps from tile-wise
+// sums ended 4e-5 away. (As eight kernels whose weight gradients read both factors
+// from memory for every sample, a 4096-sample step took 1.15 ms; now 0.050 ms: 23 us
+// in the passes, latency-bound with one 8-warp block per SM, 27 us in the chains.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -28,7 +31,8 @@ constexpr int NTT = 256;      // threads per block
 constexpr int SS = TB + 4;    // row stride of the [feature][sample] arrays (16-byte rows, no bank conflicts)
 constexpr int KC = 128;       // inputs per pass over W1 and X
 constexpr int WS = HID + 2;   // row stride of the transposed weights
-constexpr int MAXBLK = 304;   // blocks (and scratch rows) at most: two per SM
+constexpr int MAXBLK = 304;   // blocks of the passes at most: two per SM
+constexpr int GO = 4, GK = 16, GS = 256;  // a gradient block: GO x GK weights, chunks of GS samples
 
 struct TrainSmem {
   float w1t[KC][WS];    // W1 transposed, the current inputs
@@ -40,7 +44,6 @@ struct TrainSmem {
   float d1[HID][SS];    // delta1
   float w3[HID], b1[HID], b2[HID];
   float d3[TB];
-  float part[8][TB];    // partial sums of the output layer
 };
 
 // acc[o][s]: two units o0, o0 + 1 by four samples s0.. of sum_k Wt[k][o] A[k][s]
@@ -61,35 +64,31 @@ __device__ __forceinline__ void layer(const float (*Wt)[WS], const float (*A)[SS
   }
 }
 
-// g[i][j] = sum_s D[o + 16 i][s] A[k + 16 j][s]: the tile's share of a weight gradient
-template <int NJ>
-__device__ __forceinline__ void outer(const float (*D)[SS], const float (*A)[SS], int o, int k, float (&g)[4][NJ]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) g[i][j] = 0.f;
-#pragma unroll 2
-  for (int s = 0; s < TB; s += 4) {
-    float4 d[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) d[i] = *reinterpret_cast<const float4*>(&D[o + 16 * i][s]);
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      const float4 a = *reinterpret_cast<const float4*>(&A[k + 16 * j][s]);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        g[i][j] = fmaf(d[i].w, a.w, fmaf(d[i].z, a.z, fmaf(d[i].y, a.y, fmaf(d[i].x, a.x, g[i][j]))));
-    }
+// Scratch of nb samples: rows of ld = nb rounded up to a multiple of 4
+struct Scratch {
+  float *h1, *h2, *d1, *d2, *d3;  // [64][ld] four times, [ld]
+  float* x;                       // [nin][ld]
+  float* prob;                    // [nb]
+  int ld;
+  __host__ __device__ Scratch(float* s, int nb, int nin) : ld((nb + 3) / 4 * 4) {
+    h1 = s;
+    h2 = h1 + (size_t)HID * ld;
+    d1 = h2 + (size_t)HID * ld;
+    d2 = d1 + (size_t)HID * ld;
+    d3 = d2 + (size_t)HID * ld;
+    x = d3 + ld;
+    prob = x + (size_t)nin * ld;
   }
-}
+  static size_t floats(int nb, int nin) { return (size_t)((nb + 3) / 4 * 4) * (4 * HID + 2 + nin); }
+};
 
 // One block per tile of 32 samples (grid-stride): thread t owns units 2 (t % 32)
-// and + 1 of samples 4 (t / 32).. in the layers, a 4 x NJ patch of the weight
-// gradients. prob: the samples' probabilities (for the loss), or NULL.
-__global__ void __launch_bounds__(NTT) k_train_tile(const float* __restrict__ X, int ldx, const uint8_t* __restrict__ y,
+// and + 1 of samples 4 (t / 32).. in the layers. want_prob: also the samples'
+// probabilities (for the loss).
+__global__ void __launch_bounds__(NTT) k_train_pass(const float* __restrict__ X, int ldx, const uint8_t* __restrict__ y,
                                                     const int64_t* __restrict__ perm, int64_t off, int nb, int nin,
                                                     const float* __restrict__ theta, float pos_weight, float inv_n,
-                                                    float* __restrict__ part, float* __restrict__ prob) {
+                                                    Scratch out, bool want_prob) {
   extern __shared__ __align__(16) unsigned char smraw[];
   TrainSmem& sm = *reinterpret_cast<TrainSmem*>(smraw);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -98,12 +97,6 @@ __global__ void __launch_bounds__(NTT) k_train_tile(const float* __restrict__ X,
   const float* W2 = b1 + HID;
   const float* b2 = W2 + HID * HID;
   const float* w3 = b2 + HID;
-  const int np = HID * nin + HID + HID * HID + HID + HID + 1;
-  float* gW1 = part + (size_t)blockIdx.x * np;
-  float* gb1 = gW1 + HID * nin;
-  float* gW2 = gb1 + HID;
-  float* gb2 = gW2 + HID * HID;
-  float* gw3 = gb2 + HID;
   for (int i = t; i < HID * HID; i += NTT) {
     const float x = W2[i];
     sm.w2[i / HID][i % HID] = x;
@@ -134,6 +127,14 @@ __global__ void __launch_bounds__(NTT) k_train_tile(const float* __restrict__ X,
       for (int o = warp; o < HID; o += 8)
         for (int k = lane; k < KC; k += 32) sm.w1t[k][o] = kb + k < nin ? W1[(size_t)o * nin + kb + k] : 0.f;
     };
+    // a warp's lanes write the tile's samples of one unit
+    auto put = [&](float* dst, const float (*src)[SS], int n, bool relu) {
+      if (lane < cnt)
+        for (int k = warp; k < n; k += 8) {
+          const float x = src[k][lane];
+          dst[(size_t)k * out.ld + base + lane] = relu ? fmaxf(x, 0.f) : x;
+        }
+    };
     __syncthreads();  // the weights are staged; the previous tile's reads are done
     // layer 1
     float acc[2][4];
@@ -147,7 +148,9 @@ __global__ void __launch_bounds__(NTT) k_train_tile(const float* __restrict__ X,
       stage_x(c * KC);
       if (first || nchunk > 1) stage_w1(c * KC);
       __syncthreads();
-      layer(sm.w1t, sm.xt, min(KC, nin - c * KC), o0, s0, acc);
+      const int kl = min(KC, nin - c * KC);
+      layer(sm.w1t, sm.xt, kl, o0, s0, acc);
+      put(out.x + (size_t)c * KC * out.ld, sm.xt, kl, false);
     }
 #pragma unroll
     for (int e = 0; e < 2; ++e)
@@ -165,57 +168,33 @@ __global__ void __launch_bounds__(NTT) k_train_tile(const float* __restrict__ X,
     for (int e = 0; e < 2; ++e)
       *reinterpret_cast<float4*>(&sm.d2[o0 + e][s0]) = make_float4(acc[e][0], acc[e][1], acc[e][2], acc[e][3]);
     __syncthreads();
-    // output layer: warp w sums units 8 w .. 8 w + 7 of sample `lane`
-    {
-      float z = 0.f;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) z = fmaf(fmaxf(sm.d2[8 * warp + k][lane], 0.f), sm.w3[8 * warp + k], z);
-      sm.part[warp][lane] = z;
-    }
-    __syncthreads();
+    // output layer: one chain per sample
     if (t < TB) {
       float z = b3;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) z += sm.part[k][t];
+#pragma unroll 16
+      for (int k = 0; k < HID; ++k) z = fmaf(fmaxf(sm.d2[k][t], 0.f), sm.w3[k], z);
       const float p = 1.f / (1.f + expf(-z));
       float d = 0.f;
       if (t < cnt) {
         const float yy = y[row(t)] ? 1.f : 0.f;
         // weighted BCE: -(pw y log p + (1-y) log(1-p)); dL/dz = pw y (p - 1) + (1 - y) p
         d = (pos_weight * yy * (p - 1.f) + (1.f - yy) * p) * inv_n;
-        if (prob) prob[base + t] = p;
+        if (want_prob) out.prob[base + t] = p;
+        out.d3[base + t] = d;
       }
       sm.d3[t] = d;
     }
     __syncthreads();
-    // delta2 = d3 w3 (Z2 > 0) over Z2; the output layer's gradient and b2's on the way:
-    // thread t: unit t / 4, samples 8 (t % 4)..
-    {
-      const int k = t >> 2, q = 8 * (t & 3);
-      const float wk = sm.w3[k];
-      float g3 = 0.f, g2 = 0.f, s3 = 0.f;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const float z = sm.d2[k][q + e], d = sm.d3[q + e];
-        const float dd = z > 0.f ? d * wk : 0.f;
-        g3 = fmaf(d, fmaxf(z, 0.f), g3);
-        g2 += dd;
-        s3 += d;
-        sm.d2[k][q + e] = dd;
-      }
-#pragma unroll
-      for (int o = 1; o < 4; o <<= 1) {
-        g3 += __shfl_xor_sync(0xffffffffu, g3, o);
-        g2 += __shfl_xor_sync(0xffffffffu, g2, o);
-        s3 += __shfl_xor_sync(0xffffffffu, s3, o);
-      }
-      if ((t & 3) == 0) {
-        gw3[k] = first ? g3 : gw3[k] + g3;
-        gb2[k] = first ? g2 : gb2[k] + g2;
-        if (k == 0) gw3[HID] = first ? s3 : gw3[HID] + s3;
-      }
+    put(out.h1, sm.h1, HID, false);
+    put(out.h2, sm.d2, HID, true);
+    __syncthreads();
+    // delta2 = d3 w3 (Z2 > 0) over Z2
+    for (int i = t; i < HID * TB; i += NTT) {
+      const int k = i / TB, q = i % TB;
+      sm.d2[k][q] = sm.d2[k][q] > 0.f ? sm.d3[q] * sm.w3[k] : 0.f;
     }
     __syncthreads();
+    put(out.d2, sm.d2, HID, false);
     // delta1 = W2^T delta2 (Z1 > 0)
 #pragma unroll
     for (int e = 0; e < 4; ++e) acc[0][e] = acc[1][e] = 0.f;
@@ -228,86 +207,100 @@ __global__ void __launch_bounds__(NTT) k_train_tile(const float* __restrict__ X,
       *reinterpret_cast<float4*>(&sm.d1[o0 + e][s0]) = d;
     }
     __syncthreads();
-    // weight gradients: thread t: rows (t / 16) + 16 i, columns (t % 16) + 16 j
-    const int go = t >> 4, gk = t & 15;
-    {
-      float g[4][4];
-      outer<4>(sm.d2, sm.h1, go, gk, g);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float* q = gW2 + (go + 16 * i) * HID + gk + 16 * j;
-          *q = first ? g[i][j] : *q + g[i][j];
-        }
-    }
-    for (int c = nchunk - 1; c >= 0; --c) {  // the last inputs are still staged
-      if (c < nchunk - 1) {
-        __syncthreads();
-        stage_x(c * KC);
-        __syncthreads();
-      }
-      float g[4][KC / 16];
-      outer<KC / 16>(sm.d1, sm.xt, go, gk, g);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < KC / 16; ++j) {
-          const int k = c * KC + gk + 16 * j;
-          if (k < nin) {
-            float* q = gW1 + (size_t)(go + 16 * i) * nin + k;
-            *q = first ? g[i][j] : *q + g[i][j];
-          }
-        }
-    }
-    if (t < HID) {
-      float s = 0.f;
-#pragma unroll
-      for (int e = 0; e < TB; ++e) s += sm.d1[t][e];
-      gb1[t] = first ? s : gb1[t] + s;
-    }
+    put(out.d1, sm.d1, HID, false);
   }
 }
 
 struct Adam {
   float *th, *m, *v;  // NULL th: the gradient is written to `grad`
-  float lr, c1, c2;
+  float lr, b1, b2, eps, c1, c2;
 };
 
-// Sums the nblk rows of the scratch matrix in a fixed order (eight interleaved
-// partial sums per weight) into the gradient, or straight into an Adam step
-// (beta 0.9 / 0.999, eps 1e-8). Blocks past the weights sum the loss.
-__global__ void __launch_bounds__(256) k_train_reduce(const float* __restrict__ part, int nblk, int np, int nred,
-                                                      float* __restrict__ grad, Adam a,
-                                                      const float* __restrict__ prob, const uint8_t* __restrict__ y,
-                                                      const int64_t* __restrict__ perm, int64_t off, int nb,
-                                                      float pos_weight, float inv_n, double* __restrict__ loss) {
-  __shared__ float red[8][32];
-  __shared__ double redd[8];
-  const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
-  if ((int)blockIdx.x < nred) {
-    const int i = blockIdx.x * 32 + lane;
-    float s = 0.f;
-    if (i < np)
-      for (int b = q; b < nblk; b += 8) s += part[(size_t)b * np + i];
-    red[q][lane] = s;
-    __syncthreads();
-    if (q || i >= np) return;
-    float g = red[0][lane];
+// Gradients of one layer: weight (o, k) of the patch of GO x GK weights is a chain
+// over the samples of delta_o times input k (k == K: the bias, input 1). Both factors
+// come through shared memory in chunks of GS samples, the next chunk's loads in
+// flight during this one's sums.
+struct Layer {
+  const float* delta;  // [nout][ld]
+  const float* act;    // [K][ld]
+  int nout, K, w, b;   // outputs, inputs, and where the weights and the biases lie in theta
+};
+
+__device__ __forceinline__ void layer_grad(const Layer& L, int patch, int nb, int ld, float* __restrict__ grad,
+                                           const Adam& a) {
+  constexpr int NT = GO * GK, Q = GS / 4, N = (GO + GK) * Q / NT;  // 16-byte words per thread and chunk
+  static_assert((GO * Q) % NT == 0 && (GK * Q) % NT == 0, "whole words per thread");
+  __shared__ __align__(16) float T[GO + GK][GS + 4];
+  const int t = threadIdx.x, kk = t % GK, oo = t / GK;
+  const int nk = (L.K + GK) / GK;  // columns 0 .. K
+  const int o0 = patch / nk * GO, k0 = patch % nk * GK;
+  float4 r[N];
+  // every load is unconditional (clamped indices), so that all are in flight
+  auto fetch = [&](int b0) {
 #pragma unroll
-    for (int k = 1; k < 8; ++k) g += red[k][lane];
-    if (!a.th) {
-      grad[i] = g;
-      return;
+    for (int i = 0; i < N; ++i) {
+      const int e = t + i * NT, q = e % Q, row = e / Q, s = min(b0 + 4 * q, ld - 4);
+      const float* src = row < GO ? L.delta + (size_t)min(o0 + row, L.nout - 1) * ld
+                                  : L.act + (size_t)min(k0 + row - GO, L.K - 1) * ld;
+      r[i] = *reinterpret_cast<const float4*>(src + s);
     }
-    const float mi = 0.9f * a.m[i] + (1.f - 0.9f) * g;
-    const float vi = 0.999f * a.v[i] + (1.f - 0.999f) * g * g;
-    a.m[i] = mi;
-    a.v[i] = vi;
-    a.th[i] -= a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + 1e-8f);
+  };
+  float g = 0.f;
+  fetch(0);
+  for (int b0 = 0; b0 < nb; b0 += GS) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int e = t + i * NT, q = e % Q, row = e / Q, s = b0 + 4 * q;
+      float4 v = r[i];
+      if (row >= GO && k0 + row - GO >= L.K) v = make_float4(1.f, 1.f, 1.f, 1.f);
+      // samples past the end add zero
+      if (s >= nb) v.x = 0.f;
+      if (s + 1 >= nb) v.y = 0.f;
+      if (s + 2 >= nb) v.z = 0.f;
+      if (s + 3 >= nb) v.w = 0.f;
+      *reinterpret_cast<float4*>(&T[row][4 * q]) = v;
+    }
+    __syncthreads();
+    if (b0 + GS < nb) fetch(b0 + GS);
+    // products and sums rounded separately
+#pragma unroll 8
+    for (int s = 0; s < GS; s += 4) {
+      const float4 d = *reinterpret_cast<const float4*>(&T[oo][s]);
+      const float4 x = *reinterpret_cast<const float4*>(&T[GO + kk][s]);
+      g = __fadd_rn(g, __fmul_rn(d.x, x.x));
+      g = __fadd_rn(g, __fmul_rn(d.y, x.y));
+      g = __fadd_rn(g, __fmul_rn(d.z, x.z));
+      g = __fadd_rn(g, __fmul_rn(d.w, x.w));
+    }
+  }
+  const int o = o0 + oo, k = k0 + kk;
+  if (o >= L.nout || k > L.K) return;
+  const int i = k == L.K ? L.b + o : L.w + o * L.K + k;
+  if (!a.th) {
+    grad[i] = g;
     return;
   }
-  const int s = (blockIdx.x - nred) * 256 + threadIdx.x;
+  const float mi = a.b1 * a.m[i] + (1.f - a.b1) * g;
+  const float vi = a.b2 * a.v[i] + (1.f - a.b2) * g * g;
+  a.m[i] = mi;
+  a.v[i] = vi;
+  a.th[i] -= a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+}
+
+// Patches of the three layers, then (loss) blocks of 64 samples
+__global__ void __launch_bounds__(GO* GK) k_train_grad(Layer l1, Layer l2, Layer l3, int n1, int n2, int n3,
+                                                       const int64_t* __restrict__ perm, int64_t off, int nb, int ld,
+                                                       float* __restrict__ grad, Adam a,
+                                                       const float* __restrict__ prob, const uint8_t* __restrict__ y,
+                                                       float pos_weight, float inv_n, double* __restrict__ loss) {
+  const int b = blockIdx.x;
+  if (b < n1 + n2 + n3) {
+    const Layer L = b < n1 ? l1 : b < n1 + n2 ? l2 : l3;
+    layer_grad(L, b < n1 ? b : b < n1 + n2 ? b - n1 : b - n1 - n2, nb, ld, grad, a);
+    return;
+  }
+  const int s = (b - n1 - n2 - n3) * GO * GK + threadIdx.x;
   double l = 0.0;
   if (s < nb) {
     const bool yy = y[perm ? perm[off + s] : off + s] != 0;
@@ -316,12 +309,7 @@ __global__ void __launch_bounds__(256) k_train_reduce(const float* __restrict__ 
     l *= (double)inv_n;
   }
   for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-  if (lane == 0) redd[q] = l;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int k = 1; k < 8; ++k) l += redd[k];
-    atomicAdd(loss, l);
-  }
+  if ((threadIdx.x & 31) == 0) atomicAdd(loss, l);
 }
 
 // loss (nullable) += the mean weighted loss of the nb samples; the gradient
@@ -331,30 +319,28 @@ int gradient(const float* X, int ldx, const uint8_t* y, const int64_t* perm, int
              void* scratch, cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
-    if (cudaFuncSetAttribute(k_train_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)) !=
+    if (cudaFuncSetAttribute(k_train_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)) !=
         cudaSuccess)
       return -3;
     attr = true;
   }
-  const int np = mlp_n_params(nin);
-  const int nblk = std::min((nb + TB - 1) / TB, MAXBLK);
-  float* part = static_cast<float*>(scratch);
-  float* prob = loss ? part + (size_t)nblk * np : nullptr;
+  const Scratch sc(static_cast<float*>(scratch), nb, nin);
   const float inv_n = 1.f / norm_n;
-  k_train_tile<<<nblk, NTT, sizeof(TrainSmem), st>>>(X, ldx, y, perm, off, nb, nin, theta, pos_weight, inv_n, part,
-                                                     prob);
-  const int nred = (np + 31) / 32;
-  k_train_reduce<<<nred + (loss ? (nb + 255) / 256 : 0), 256, 0, st>>>(part, nblk, np, nred, grad, a, prob, y, perm,
-                                                                      off, nb, pos_weight, inv_n, loss);
+  k_train_pass<<<std::min((nb + TB - 1) / TB, MAXBLK), NTT, sizeof(TrainSmem), st>>>(
+      X, ldx, y, perm, off, nb, nin, theta, pos_weight, inv_n, sc, loss != nullptr);
+  const int w2 = HID * nin + HID, w3 = w2 + HID * HID + HID;
+  const Layer l1{sc.d1, sc.x, HID, nin, 0, HID * nin}, l2{sc.d2, sc.h1, HID, HID, w2, w2 + HID * HID},
+      l3{sc.d3, sc.h2, 1, HID, w3, w3 + HID};
+  auto patches = [](const Layer& L) { return (L.nout + GO - 1) / GO * ((L.K + GK) / GK); };
+  const int n1 = patches(l1), n2 = patches(l2), n3 = patches(l3), nl = loss ? (nb + GO * GK - 1) / (GO * GK) : 0;
+  k_train_grad<<<n1 + n2 + n3 + nl, GO * GK, 0, st>>>(l1, l2, l3, n1, n2, n3, perm, off, nb, sc.ld, grad, a, sc.prob,
+                                                      y, pos_weight, inv_n, loss);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace
 
-size_t mlp_scratch_bytes(int nb, int nin) {
-  const size_t nblk = (size_t)std::min((nb + TB - 1) / TB, MAXBLK);
-  return (nblk * mlp_n_params(nin) + nb) * sizeof(float);
-}
+size_t mlp_scratch_bytes(int nb, int nin) { return Scratch::floats(nb, nin) * sizeof(float); }
 
 int mlp_loss_grad_dev(const float* X, int ldx, const uint8_t* y, int nb, int nin, const float* theta, float* grad,
                       double* loss, float pos_weight, void* scratch, cudaStream_t st) {
@@ -364,16 +350,16 @@ int mlp_loss_grad_dev(const float* X, int ldx, const uint8_t* y, int nb, int nin
 int mlp_train_dev(const float* X, int ldx, const uint8_t* y, int64_t n, int nin, float* theta, int epochs,
                   int batch, float lr, float pos_weight, uint64_t seed, double* last_loss, cudaStream_t st) {
   const int np = mlp_n_params(nin);
-  // one allocation: shuffle (8-byte elements first), loss, Adam moments, scratch
+  // one allocation: scratch (16-byte rows first), shuffle, loss, Adam moments
   const size_t bytes = n * sizeof(int64_t) + sizeof(double) + 2 * (size_t)np * sizeof(float) +
-                       mlp_scratch_bytes(batch, nin);
+                       (mlp_scratch_bytes(batch, nin) + 7) / 8 * 8;
   unsigned char* mem = nullptr;
   if (cudaMalloc(&mem, bytes) != cudaSuccess) return -3;
-  int64_t* perm = reinterpret_cast<int64_t*>(mem);
+  void* scratch = mem;
+  int64_t* perm = reinterpret_cast<int64_t*>(mem + (mlp_scratch_bytes(batch, nin) + 7) / 8 * 8);
   double* dloss = reinterpret_cast<double*>(perm + n);
   float* m = reinterpret_cast<float*>(dloss + 1);
   float* v = m + np;
-  void* scratch = v + np;
   int e = 0;
   if (cudaMemsetAsync(m, 0, 2 * (size_t)np * sizeof(float), st) != cudaSuccess) e = -3;
   std::vector<int64_t> hp(n);
@@ -389,7 +375,7 @@ int mlp_train_dev(const float* X, int ldx, const uint8_t* y, int64_t n, int nin,
     for (int64_t off = 0; off + batch <= n && !e; off += batch) {
       ++t;
       const float c1 = 1.f - powf(0.9f, (float)t), c2 = 1.f - powf(0.999f, (float)t);
-      e = gradient(X, ldx, y, perm, off, batch, nin, theta, nullptr, Adam{theta, m, v, lr, c1, c2}, loss, pos_weight,
+      e = gradient(X, ldx, y, perm, off, batch, nin, theta, nullptr, Adam{theta, m, v, lr, 0.9f, 0.999f, 1e-8f, c1, c2}, loss, pos_weight,
                    (float)batch, scratch, st);
     }
   }
