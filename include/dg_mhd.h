@@ -253,8 +253,9 @@ int dg_mhd_counters(dg_mhd_ctx* ctx, int64_t* pos_cells, double* inj_mass, doubl
 /* Workload of the positivity limiter in the FP32 form (measurement support,
  * no counterpart in the paper): cells whose FP32 bound could not clear them and
  * that therefore went to the listed-cell kernel (point-wise screen, then the
- * full procedure of the cells still open), summed over limiter passes since the last reset (FP64 contexts run the procedure on every cell
- * and count 0). Synchronises the device; reset = 1 clears the count. */
+ * full procedure of the cells still open), summed over limiter passes since the
+ * last reset (FP64 contexts count 0). Synchronises the device; reset = 1 clears
+ * the count. */
 int dg_mhd_positivity_listed(dg_mhd_ctx* ctx, int64_t* listed, int reset);
 
 /* Divergence diagnostics of App. C on a uniform mesh (DG_E_UNSUPPORTED on

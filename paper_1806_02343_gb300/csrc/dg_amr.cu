@@ -846,13 +846,13 @@ int build_amr(Ctx& c, const dg_mesh_desc* mesh) {
 
 OctPow<float> oct_pow32(const Ctx& c) {
   const AmrHost& h = c.amr;
-  return OctPow<float>{h.fL, h.fR, h.cstart, h.centry, h.dxc, h.btype, (const float*)h.ftab, (const float*)h.ctab, (const float*)h.ntab, c.g.ncell, c.g.stride,
-                       h.nblk};
+  return OctPow<float>{h.fL, h.fR, h.cstart, h.centry, h.dxc, h.btype, (const float*)h.ftab, (const float*)h.ctab,
+                    (const float*)h.ntab, c.g.ncell, c.g.stride, h.nblk};
 }
 OctPow<double> oct_pow64(const Ctx& c) {
   const AmrHost& h = c.amr;
-  return OctPow<double>{h.fL, h.fR, h.cstart, h.centry, h.dxc, h.btype, (const double*)h.ftab, (const double*)h.ctab, (const double*)h.ntab, c.g.ncell,
-                        c.g.stride, h.nblk};
+  return OctPow<double>{h.fL, h.fR, h.cstart, h.centry, h.dxc, h.btype, (const double*)h.ftab, (const double*)h.ctab,
+                    (const double*)h.ntab, c.g.ncell, c.g.stride, h.nblk};
 }
 
 void free_amr(Ctx& c) {
