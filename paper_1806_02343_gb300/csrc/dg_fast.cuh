@@ -120,7 +120,7 @@ struct FastGeom {
 };
 
 // copies the tables to the constant bank where this (T, DEG) keeps them there
-// (synchronous; returns 0 or -3)
+// (the Powell ones where they are built; synchronous; returns 0 or -3)
 template <typename T, int DEG>
 int fast_to_constant(const FastAll<T, DEG>& tabs);
 template <typename T, int DEG>

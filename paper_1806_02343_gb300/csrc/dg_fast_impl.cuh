@@ -21,6 +21,7 @@
 //   k_cell_glm reads coalesced.
 #include <cuda_runtime.h>
 
+#include <cstddef>
 #include <type_traits>
 #include <utility>
 
@@ -39,10 +40,12 @@ namespace {
 constexpr int TC = 32;        // cells (or faces) per block
 
 // Reference-element tables in the constant bank. They depend only on the
-// scheme and the degree (not on the mesh), so one copy serves every context;
-// indexed with compile-time offsets, each table value is a constant operand of
-// its FMA. Each (precision, degree) is its own translation unit (they compile
-// in parallel) with its own copy.
+// degree (not on the mesh), so one copy serves every context; indexed with
+// compile-time offsets, each table value is a constant operand of its FMA. Each
+// (precision, degree) is its own translation unit (they compile in parallel)
+// with its own copy. GLM contexts have no Powell tables (building them takes an
+// LDF basis) and leave those of the copy, the last member, as they are: Powell
+// contexts of the same degree may be in use.
 template <typename T, int DEG>
 struct FastConst {
   static constexpr bool on = false;
@@ -54,7 +57,8 @@ struct FastConst<DG_FAST_T, DG_FAST_DEG> {
   static constexpr bool on = true;
   __device__ static const FastAll<DG_FAST_T, DG_FAST_DEG>& get() { return c_fast; }
   static cudaError_t upload(const FastAll<DG_FAST_T, DG_FAST_DEG>& t) {
-    return cudaMemcpyToSymbol(c_fast, &t, sizeof(t));
+    using All = FastAll<DG_FAST_T, DG_FAST_DEG>;
+    return cudaMemcpyToSymbol(c_fast, &t, t.pow.ok ? sizeof(All) : offsetof(All, pow));
   }
 };
 #endif
