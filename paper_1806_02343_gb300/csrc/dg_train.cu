@@ -362,14 +362,24 @@ int mlp_train_dev(const float* X, int ldx, const uint8_t* y, int64_t n, int nin,
   float* v = m + np;
   int e = 0;
   if (cudaMemsetAsync(m, 0, 2 * (size_t)np * sizeof(float), st) != cudaSuccess) e = -3;
+  cudaEvent_t copied = nullptr;  // behind the last copy of the shuffle
+  if (cudaEventCreateWithFlags(&copied, cudaEventDisableTiming) != cudaSuccess) e = -3;
   std::vector<int64_t> hp(n);
   for (int64_t i = 0; i < n; ++i) hp[i] = i;
   std::mt19937_64 rng(seed);
   int t = 0;
   for (int ep = 0; ep < epochs && !e; ++ep) {
-    // (the previous epoch's kernels may still run: the copy below follows them on the stream)
+    // The copy below follows the previous epoch's kernels on the stream, and may read
+    // hp as late as that (staging pageable memory first is allowed, not promised): the
+    // next shuffle waits for it, while this epoch's kernels run.
+    if (ep > 0 && cudaEventSynchronize(copied) != cudaSuccess) {
+      e = -3;
+      break;
+    }
     std::shuffle(hp.begin(), hp.end(), rng);
-    if (cudaMemcpyAsync(perm, hp.data(), n * sizeof(int64_t), cudaMemcpyHostToDevice, st)) e = -3;
+    if (cudaMemcpyAsync(perm, hp.data(), n * sizeof(int64_t), cudaMemcpyHostToDevice, st) ||
+        cudaEventRecord(copied, st) != cudaSuccess)
+      e = -3;
     double* loss = ep == epochs - 1 ? dloss : nullptr;
     if (loss) cudaMemsetAsync(dloss, 0, sizeof(double), st);
     for (int64_t off = 0; off + batch <= n && !e; off += batch) {
@@ -380,6 +390,7 @@ int mlp_train_dev(const float* X, int ldx, const uint8_t* y, int64_t n, int nin,
     }
   }
   if (cudaStreamSynchronize(st) != cudaSuccess) e = -3;
+  if (copied) cudaEventDestroy(copied);
   if (!e && last_loss) {
     double l = 0.0;
     cudaMemcpy(&l, dloss, sizeof(double), cudaMemcpyDeviceToHost);

@@ -1,0 +1,52 @@
+"""Host side of the launch code, on a stand-in for the CUDA runtime
+(fake_cudart.cpp): kernels do nothing, copies and launch limits behave as the
+runtime documents them. No GPU."""
+import os
+import shutil
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    from paper_1806_02343_gb300 import build
+    build.build()
+    so = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    subprocess.run([shutil.which("g++") or "c++", "-O1", "-shared", "-fPIC", "-o", so,
+                    os.path.join(ROOT, "tests", "fake_cudart.cpp")], check=True)
+    return so
+
+
+def _run(fake, code, **env):
+    pre = "import ctypes, os, sys\nimport numpy as np\nfrom paper_1806_02343_gb300 import binding as Bd\n" \
+          "lib, vp = Bd.lib(), ctypes.c_void_p\n"
+    r = subprocess.run([sys.executable, "-c", pre + code], cwd=ROOT, capture_output=True, text=True, timeout=300,
+                       env=dict(os.environ, PYTHONPATH=ROOT, LD_PRELOAD=fake, **env))
+    assert r.returncode == 0, r.stdout + r.stderr
+    return r.stdout
+
+
+TRAIN = """
+def train(n=96, nin=6, epochs=6, batch=32):
+    X, y, th = (np.zeros(s, t) for s, t in (((n, nin), np.float32), (n, np.uint8), (64 * nin + 64 * 64 + 193, np.float32)))
+    p = lambda a: vp(a.ctypes.data)
+    return lib.dg_mhd_mlp_train(p(X), nin, p(y), n, nin, p(th), epochs, batch, 1e-3, 1.0, 5, None, None)
+"""
+
+
+def test_training_reads_every_epochs_own_shuffle(fake, tmp_path):
+    """The copy of a shuffle from pageable memory may run as late as its place in the stream: the permutations the
+    epochs train on do not depend on when."""
+    seen = []
+    for defer in "01":
+        log = str(tmp_path / f"copies{defer}")
+        _run(fake, TRAIN + "assert train() == 0\n", FAKE_DEFER=defer, FAKE_LOG=log)
+        seen.append(np.fromfile(log, np.int64).reshape(6, 96))
+    assert all(np.array_equal(np.sort(p), np.arange(96)) for p in seen[0])
+    assert len({p.tobytes() for p in seen[0]}) == 6
+    assert np.array_equal(*seen)
