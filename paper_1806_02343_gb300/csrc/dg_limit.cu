@@ -610,7 +610,7 @@ __device__ __forceinline__ bool pos_point_open(const T* uu, const double* m, con
   const T mag = T(0.5) * (uu[5] * uu[5] + uu[6] * uu[6] + uu[7] * uu[7]);
   const T pq = gm1 * (uu[4] - kin - mag);
   if (screen_t == T(0)) return pq < eps_p;
-  if (uu[0] < T(1e-2) * sc[0]) return true;
+  if (uu[0] < T(1e-2) * sc[0] || !pos_range((float)sc[0], (float)sc[4])) return true;
   const T kin_s = T(0.5) * (sc[1] * sc[1] + sc[2] * sc[2] + sc[3] * sc[3]) / uu[0];
   const T mag_s = T(0.5) * (sc[5] * sc[5] + sc[6] * sc[6] + sc[7] * sc[7]);
   return pq < eps_p + screen_t * gm1 * (sc[4] + kin_s + mag_s);
@@ -627,7 +627,7 @@ __device__ __forceinline__ bool pos_point_open_f(const float* uu, const float* m
   const float kin = 0.5f * (uu[1] * uu[1] + uu[2] * uu[2] + uu[3] * uu[3]) / uu[0];
   const float mag = 0.5f * (uu[5] * uu[5] + uu[6] * uu[6] + uu[7] * uu[7]);
   const float pq = gm1 * (uu[4] - kin - mag);
-  if (uu[0] < 1e-2f * sc[0]) return true;
+  if (uu[0] < 1e-2f * sc[0] || !pos_range(sc[0], sc[4])) return true;
   const float kin_s = 0.5f * (sc[1] * sc[1] + sc[2] * sc[2] + sc[3] * sc[3]) / uu[0];
   const float mag_s = 0.5f * (sc[5] * sc[5] + sc[6] * sc[6] + sc[7] * sc[7]);
   return pq < eps_p + screen_t * gm1 * (sc[4] + kin_s + mag_s);

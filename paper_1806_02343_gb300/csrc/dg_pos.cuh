@@ -16,13 +16,25 @@ __host__ __device__ __forceinline__ int screen_mean_row(const Geom& g, int k) {
   return k < 7 ? g.ldf0 + (k - 5) : g.bz2d;
 }
 
+// Whether the FP32 tests below can be trusted with a cell of this density and
+// energy: their products of two conserved variables (rho E, m^2, B^2) lose up to
+// 1.2e-38 where they leave FP32's normal numbers, and with both above 1e-30, and
+// their product, that stays below a hundredth of the tests' margins (1e-4 of the
+// energy, times at least a hundredth of the density). Below it -- FP64 states in
+// small units, or rows near the end of FP32's range -- every product may be zero
+// whatever the pressure: such cells take the FP64 procedure.
+__device__ __forceinline__ bool pos_range(float rho, float E) {
+  constexpr float tiny = 1e-30f;
+  return rho > tiny && E > tiny && rho * E > tiny;
+}
+
 // The end of pos_screen_rows: means mt and deviation bounds dv of the 8 variables
 __device__ __forceinline__ bool pos_screen_bound(const PosScreen& ps, const float* mt, float* dv) {
   const float mg = 1e-4f;
 #pragma unroll
   for (int v = 0; v < 8; ++v) dv[v] = dv[v] * (1.f + mg) + mg * fabsf(mt[v]);
   const float rlo = mt[0] - dv[0];
-  if (rlo > ps.eps_rho * 2.f) {
+  if (rlo > ps.eps_rho * 2.f && pos_range(rlo, mt[4])) {
     float kin = 0.f, mag = 0.f;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -85,7 +97,8 @@ __device__ __forceinline__ bool pos_screen_rows(const Geom& g, const PosScreen& 
 // |coefficients| x basis bound) every value carries at most about 30 roundings,
 // 2e-6 S_v; a point is cleared with rho >= 0.1 S_rho and
 //   rho (E - B^2/2 - eps_p/(g-1) - t (S_E + S_B^2/2)) >= m^2/2 + t S_m^2/2,
-// t = 1e-4: at least four times what those roundings can move either side.
+// t = 1e-4: at least four times what those roundings can move either side
+// (pos_range: and what products near the end of FP32's range lose).
 // A non-finite value clears nothing. coef(v, l): Legendre coefficient l of
 // variable v (v < 8).
 template <int DEG, typename Coef>
@@ -99,7 +112,7 @@ __device__ __forceinline__ bool pos_points_clear(Coef coef, const float (&mt)[8]
   const float c1 = eps_p / gm1 + t * (S[4] + 0.5f * (S[5] * S[5] + S[6] * S[6] + S[7] * S[7]));
   const float c2 = 0.5f * t * (S[1] * S[1] + S[2] * S[2] + S[3] * S[3]);
   const float r0 = fmaxf(eps_rho + t * S[0], 0.1f * S[0]);
-  bool ok = true;
+  bool ok = pos_range(S[0], S[4]);
   auto test = [&](const float (&u)[8]) {
     const float b2 = u[5] * u[5] + u[6] * u[6] + u[7] * u[7], m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
     const float e = u[4] - 0.5f * b2 - c1;
