@@ -233,10 +233,14 @@ __device__ __forceinline__ void face_coefs(const V* c, bool plus, V* g) {
 //   (a^2 - b^2)^2 + 4 a^2 b_t^2, a sum of squares;
 // * the upwind side of the contact is selected before the flux is assembled;
 //   the two jump terms carry the wave speeds clipped at zero. In a supersonic
-//   state the star terms are dropped by selection (they may be anything).
+//   state the star terms are dropped by selection (they may be anything), and
+//   the outer wave speeds alone select the side: without pressure and field
+//   S_L = S_R, and S_M is 0 / 0 or noise.
 // Writes the rotated flux (F[5] = 0) and returns B^n_F.
 __device__ __forceinline__ V vmin(V a, V b) { return a < b ? a : b; }
 __device__ __forceinline__ V vmax(V a, V b) { return a > b ? a : b; }
+// x > 0 (and not NaN) from the upper word, off the FP64 pipe; false for subnormal x
+__device__ __forceinline__ bool positive(V x) { return (unsigned)(__double2hiint(x) - 1) < 0x7ff00000u; }
 
 __device__ __forceinline__ V hlld(const V* uL, const V* uR, V gamma, V eps, V* F) {
   const V rL = uL[0], rR = uR[0];
@@ -300,7 +304,8 @@ __device__ __forceinline__ V hlld(const V* uL, const V* uR, V gamma, V eps, V* F
   const V wss = __fma_rn(sqL, wL, __fma_rn(sqR, wR, (zR - zL) * sgn)) * inv;
   const V yss = __fma_rn(sqL, yR, __fma_rn(sqR, yL, (vR - vL) * qs)) * inv;
   const V zss = __fma_rn(sqL, zR, __fma_rn(sqR, zL, (wR - wL) * qs)) * inv;
-  const bool left = SM >= 0.0;
+  const bool superL = positive(SL), superR = positive(-SR);
+  const bool left = superL | (!superR & (SM >= 0.0));  // (short-circuit operators: 3% slower passes)
   auto pick = [&](V a, V b) { return left ? a : b; };
   const V xr = pick(rL, rR), xu = pick(l.u, r.u), xv = pick(l.v, r.v), xw = pick(l.w, r.w);
   const V xy = pick(uL[6], uR[6]), xz = pick(uL[7], uR[7]), xE = pick(l.E, r.E), xp = pick(l.pT, r.pT);
@@ -308,9 +313,10 @@ __device__ __forceinline__ V hlld(const V* uL, const V* uR, V gamma, V eps, V* F
   const V xd = pick(dL, dR), xi = pick(ieL, ieR), xrs = pick(rsL, rsR);
   const V xvs = pick(vL, vR), xws = pick(wL, wR), xys = pick(yL, yR), xzs = pick(zL, zR);
   const V xq = pick(sqL, -sqR);
-  const bool super = pick(SL, -SR) > 0.0;
-  const V S1 = pick(vmin(SL, 0.0), vmax(SR, 0.0));
-  const V S2 = pick(vmin(SsL, 0.0), vmax(SsR, 0.0));
+  const bool super = left ? superL : superR;
+  // clipped at zero: the outer speed of a side that is not supersonic has its sign already
+  const V S1 = pick(SL, SR), Ss = pick(SsL, SsR);
+  const V S2 = (__double2hiint(Ss) < 0) == left ? Ss : 0.0;
   const V vb = __fma_rn(xu, bn, __fma_rn(xv, xy, xw * xz));
   const V vbs = __fma_rn(SM, bn, __fma_rn(xvs, xys, xws * xzs));
   const V vbss = __fma_rn(SM, bn, __fma_rn(vss, yss, wss * zss));
