@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(128) k_tvb_detect(Geom gin, LdfLeg ll, const T
       sf::each<0, 3>([&](auto AX) {
         constexpr int A = decltype(AX)::value;
         if (!clear) return;
-        clear = tvb_axis_clear<A, GLMF>(m, sls[A], gamma, ch, thr, beta, [&](float (&dp)[9], float (&dm)[9]) {
+        clear = tvb_axis_clear<A, GLMF>(m, sls[A], gamma, ch, thr, beta, kTvbWide<T>, [&](float (&dp)[9], float (&dm)[9]) {
 #pragma unroll
           for (int sd = 0; sd < 2; ++sd) {
             float mn[9], f = 0.5f;

@@ -19,7 +19,15 @@ namespace dgmhd {
 // primitive increments, kTvbRound (some 100 roundings) times the absolute values
 // of the terms they are the differences of. Nearer to a degeneracy (c_f ~ c_s,
 // or a transverse field near zero) only the direction-free bounds b are used.
-constexpr float kTvbWeight = 2e-2f, kTvbRound = 1e-5f;
+// Where c_f ~ c_s (gap c_f^2 - c_s^2 below kTvbGap c_f^2), b allows for weights
+// above 1 as well: the procedure takes any gap above rel c_f^2, and near a = c_A
+// without a transverse field the gap is what the rounding of its radicand leaves,
+// so that alpha^2 = (1 +- (a^2 - b^2) / gap) / 2 reaches (1 + 4 sqrt(eps) / rel) / 2:
+// weights up to 22 in FP32 (eps = 6e-8, rel = 1e-6; 11 seen), 150 in FP64 (1.1e-16,
+// 1e-12). At kTvbGap they are 1 to 0.2%.
+constexpr float kTvbWeight = 2e-2f, kTvbRound = 1e-5f, kTvbGap = 2e-2f;
+template <typename T>
+constexpr float kTvbWide = sizeof(T) == 4 ? 32.f : 256.f;
 
 template <int GLMF>
 struct TvbAmp {
@@ -38,11 +46,12 @@ template <int GLMF>
 struct TvbEig {
   float rho, ir, isr, a2i, v[3], B[3], gm1, ich;
   float cf, cs, af, as, by, bz, sgn, isra;
+  float wmax;       // bound of the weights
   bool sane, fine;  // the pressure keeps its leading digits; away from the degeneracies
 };
 
 template <int A, int GLMF>
-__device__ __forceinline__ void tvb_eig(const float (&m)[9], float gamma, float ch, TvbEig<GLMF>& e) {
+__device__ __forceinline__ void tvb_eig(const float (&m)[9], float gamma, float ch, float wide, TvbEig<GLMF>& e) {
   constexpr int T1 = (A + 1) % 3, T2 = (A + 2) % 3;
   e.rho = m[0];
   e.ir = tvb_rcp(m[0]);
@@ -64,6 +73,7 @@ __device__ __forceinline__ void tvb_eig(const float (&m)[9], float gamma, float 
   e.cf = tvb_sqrt(cf2);
   e.cs = tvb_sqrt(cs2);
   const float bt = tvb_sqrt(bt2), id = tvb_rcp(cf2 - cs2), ibt = tvb_rcp(bt);
+  e.wmax = cf2 - cs2 > kTvbGap * cf2 ? 1.f : wide;
   e.sane = p > 1e-4f * m[4];
   e.fine = cf2 - cs2 > 0.05f * cf2 && bt > 1e-3f * tvb_sqrt(m[0] * cf2) && p > 0.03f * m[4];
   e.af = tvb_sqrt(fmaxf(a2 - cs2, 0.f) * id);
@@ -109,7 +119,7 @@ __device__ __forceinline__ void tvb_amp(const TvbEig<GLMF>& e, const float (&d)[
   const float ef = kTvbWeight * wf + kTvbRound * rf;
 #pragma unroll
   for (int k = 0; k < 7; k += 2) {
-    o.b[k] = wf + ef;
+    o.b[k] = e.wmax * wf + ef;
     o.e[k] = ef;
   }
   const float wa = 0.5f * (nv + nb * e.isr), ea = kTvbWeight * wa + kTvbRound * 0.5f * st;
@@ -133,11 +143,12 @@ __device__ __forceinline__ void tvb_amp(const TvbEig<GLMF>& e, const float (&d)[
 
 // Axis A cannot trigger: every amplitude of the slopes `sl` stays below thr, or
 // both neighbour differences (dp, dm: loaded by `diffs` where needed) clear it.
+// wide: kTvbWide of the procedure's precision.
 template <int A, int GLMF, typename Diffs>
 __device__ __forceinline__ bool tvb_axis_clear(const float (&m)[9], const float (&sl)[9], float gamma, float ch,
-                                               float thr, float beta, Diffs diffs) {
+                                               float thr, float beta, float wide, Diffs diffs) {
   TvbEig<GLMF> e;
-  tvb_eig<A>(m, gamma, ch, e);
+  tvb_eig<A>(m, gamma, ch, wide, e);
   if (!e.sane) return false;
   TvbAmp<GLMF> x;
   tvb_amp<A>(e, sl, x);
