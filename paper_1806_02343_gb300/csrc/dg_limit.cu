@@ -422,23 +422,23 @@ __global__ void __launch_bounds__(128) k_tvb_detect(Geom gin, LdfLeg ll, const T
   const int64_t S = g.stride;
   const float gamma = (float)g.gamma;
   const float ch = GLMF ? sc->ch32 : 0.f;
-  // Legendre coefficient l of B component cc from the LDF rows of cell c
+  // Legendre coefficient l of B component cc from the LDF rows of cell c (constant
+  // and linear ones: the entries are multiples of 1/2, exact in FP32), and the means,
+  // in the state's precision: sums and differences that cancel are rounded after it
   auto ldf = [&](int64_t c, auto CC, auto L) {
-    float x = 0.f;
+    T x = T(0);
     sf::each<0, LdfPattern<DEG>::NDIV>([&](auto J) {
       constexpr int j = decltype(J)::value, cc = decltype(CC)::value, l = decltype(L)::value;
-      if constexpr (ldf_has<DEG>(j, cc, l))
-        x = fmaf((float)w[(int64_t)(5 * N + j) * S + c], ll.A[(j * 3 + cc) * N + l], x);
+      if constexpr (ldf_has<DEG>(j, cc, l)) x = fma(w[(int64_t)(5 * N + j) * S + c], (T)ll.A[(j * 3 + cc) * N + l], x);
     });
     return x;
   };
-  auto means = [&](int64_t c, float (&m)[9]) {
+  auto means = [&](int64_t c, T (&m)[9]) {
 #pragma unroll
     for (int k = 0; k < NM; ++k)
-      if (GLMF || k < 5) m[k] = (float)w[(int64_t)(k * N) * S + c];
+      if (GLMF || k < 5) m[k] = w[(int64_t)(k * N) * S + c];
     if constexpr (!GLMF) {
       sf::each<0, 3>([&](auto CC) { m[5 + decltype(CC)::value] = ldf(c, CC, std::integral_constant<int, 0>{}); });
-      m[8] = 0.f;
     }
   };
   // warp-uniform trip count (the appends below are warp ballots)
@@ -449,16 +449,20 @@ __global__ void __launch_bounds__(128) k_tvb_detect(Geom gin, LdfLeg ll, const T
     if (i < total) {
       c = list ? (int64_t)list[i] : i;
       const float thr = an.on ? (float)(mtilde * an.dxc[c]) : thr0;
+      T mt[9];
       float m[9], sls[3][9];  // every load of the cell's own rows is issued before the first use
-      means(c, m);
+      means(c, mt);
+#pragma unroll
+      for (int k = 0; k < 9; ++k) m[k] = k < NM ? (float)mt[k] : 0.f;
       sf::each<0, 3>([&](auto AX) {
         constexpr int A = decltype(AX)::value;
 #pragma unroll
         for (int v = 0; v < NM; ++v)
           if (GLMF || v < 5) sls[A][v] = (float)w[(int64_t)(v * N + 1 + A) * S + c];
         if constexpr (!GLMF) {
-          sf::each<0, 3>(
-              [&](auto CC) { sls[A][5 + decltype(CC)::value] = ldf(c, CC, std::integral_constant<int, 1 + A>{}); });
+          sf::each<0, 3>([&](auto CC) {
+            sls[A][5 + decltype(CC)::value] = (float)ldf(c, CC, std::integral_constant<int, 1 + A>{});
+          });
           sls[A][8] = 0.f;
         }
       });
@@ -469,28 +473,29 @@ __global__ void __launch_bounds__(128) k_tvb_detect(Geom gin, LdfLeg ll, const T
         clear = tvb_axis_clear<A, GLMF>(m, sls[A], gamma, ch, thr, beta, kTvbWide<T>, [&](float (&dp)[9], float (&dm)[9]) {
 #pragma unroll
           for (int sd = 0; sd < 2; ++sd) {
-            float mn[9], f = 0.5f;
+            T mn[9];
+            float f = 0.5f;
             if (!an.on) {
               means(nb(g, c, A, sd ? 1 : -1), mn);
             } else {  // the average of the leaves across the side, the centre distance 2, 1.5 or 3
               const int sidx = 2 * A + sd, inf = an.side_info[c * 6 + sidx];
               const int cnt = inf & 15, rel = inf >> 4;
 #pragma unroll
-              for (int k = 0; k < 9; ++k) mn[k] = 0.f;
+              for (int k = 0; k < 9; ++k) mn[k] = T(0);
               for (int q = 0; q < cnt; ++q) {
-                float t[9];
+                T t[9];
                 means((int64_t)an.side_nb[c * 24 + sidx * 4 + q], t);
 #pragma unroll
                 for (int k = 0; k < NM; ++k) mn[k] += t[k];
               }
-              const float ic = 1.f / (float)(cnt > 0 ? cnt : 1);
+              const T ic = T(1) / (T)(cnt > 0 ? cnt : 1);
 #pragma unroll
               for (int k = 0; k < NM; ++k) mn[k] *= ic;
               if (cnt > 0) f = rel == 0 ? 0.5f : (rel == 1 ? 1.f / 1.5f : 1.f / 3.f);
             }
 #pragma unroll
             for (int k = 0; k < 9; ++k) {
-              const float d = k < NM ? (sd ? mn[k] - m[k] : m[k] - mn[k]) * f : 0.f;
+              const float d = k < NM ? (float)(sd ? mn[k] - mt[k] : mt[k] - mn[k]) * f : 0.f;
               (sd ? dp[k] : dm[k]) = d;
             }
           }

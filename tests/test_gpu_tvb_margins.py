@@ -72,3 +72,50 @@ def test_fp32_near_the_double_degeneracy(d, axis):
     (h0, w_all), (h1, w_list) = outs
     assert 10 < h0.sum() < C // 2
     assert np.array_equal(h0, h1) and np.array_equal(w_all, w_list)
+
+
+@pytest.mark.parametrize("divb", ["glm", "powell"])
+@pytest.mark.parametrize("d", [1, 2])
+@pytest.mark.parametrize("size", [1e-2, 1e-3, 1e-4, 1e-6])
+def test_fp64_small_increments_on_a_background(divb, d, size):
+    """Entropy waves of a part `size` of the mean, slopes within 4e-8 / size of the limit that the smaller neighbour
+    difference sets: the differences of the means lose their digits if the means are rounded to FP32 first."""
+    import torch
+    from paper_1806_02343_gb300.binding import DG_LIMIT_TVB, Solver
+    n = (12, 9, 8)
+    S = Scheme(3, d, divb, G, n)
+    S.P.Mtilde = 1e-9 / S.dx
+    S.P.tvb_eps = 0.0
+    r = np.random.default_rng(3)
+    C = S.C
+    i = np.arange(C) % n[0]
+    x = size * np.cumsum(r.uniform(0.5, 1.5, n[0]))       # rising along x, one step back at the period
+    rho = 1.0 + x[i]
+    v = np.array([0.7, -0.4, 0.3])
+    B = np.array([0.5, 0.3, -0.6])
+    u = mhd.conserved(rho, np.tile(v, (C, 1)), np.full(C, 0.8), np.tile(B, (C, 1)), G)
+    if S.V == 9:
+        u = np.concatenate([u, np.zeros((C, 1))], 1)
+    dp, dm = 0.5 * (rho[S.nbr_plus[0]] - rho), 0.5 * (rho - rho[S.nbr_minus[0]])
+    s = S.P.beta * np.minimum(dp, dm) * (1.0 + np.minimum(4e-8 / size, 0.3) * r.uniform(-1.0, 1.0, C))
+    sl = np.zeros((C, 3, S.V))
+    s = np.where((dp > 0) & (dm > 0), s, 0.0)
+    sl[:, 0, 0] = s
+    sl[:, 0, 1:4] = s[:, None] * v
+    sl[:, 0, 4] = s * 0.5 * (v @ v)
+    w0, lim = _fill(S, u, sl)
+    if d == 2:
+        w0[:, S.modes.index((2, 0, 0))] = 1e-3 * size     # what a changed cell loses beyond its slopes
+    ch = 2.0
+    ref = np.any(lim(w0, ch if divb == "glm" else None) != w0, 1)
+    assert ref.sum() > C // 5
+    sol = Solver(3, n, d, divb, gamma=G, box_len=S.L, Mtilde=S.P.Mtilde, tvb_eps=0.0, limiter=DG_LIMIT_TVB)
+    if divb == "glm":
+        sol.set_glm(ch, 1.0)
+    w = to_device(w0, sol)
+    flags = torch.zeros(sol.stride, dtype=torch.uint8, device="cuda")
+    sol.limit(w, None, flags)
+    got = flags[:C].cpu().numpy().astype(bool)
+    # a slope within some roundings of its limit is decided by them: leave those out
+    close = np.abs(s - S.P.beta * np.minimum(dp, dm)) < 1e-12
+    assert np.array_equal(got[~close], ref[~close])
