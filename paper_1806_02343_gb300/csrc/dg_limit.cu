@@ -466,7 +466,8 @@ __global__ void __launch_bounds__(128) k_tvb_detect(Geom gin, LdfLeg ll, const T
           sls[A][8] = 0.f;
         }
       });
-      bool clear = !GLMF || ch > 0.f;  // no c_h yet: the procedure takes B_n and psi as separate fields
+      // (no c_h yet: the procedure takes B_n and psi as separate fields)
+      bool clear = (!GLMF || ch > 0.f) && tvb_range<T>(m);
       sf::each<0, 3>([&](auto AX) {
         constexpr int A = decltype(AX)::value;
         if (!clear) return;

@@ -35,6 +35,15 @@ struct TvbAmp {
   float b[9], e[9];        // upper bounds for any direction of the transverse field, errors
 };
 
+// The error terms hold while increments down to the FP64 rounding of the means
+// (1e-16 of them) are normal FP32 numbers: FP64 states whose density or energy is
+// outside 1e-15 .. 1e15 leave every cell to the procedure.
+template <typename T>
+__device__ __forceinline__ bool tvb_range(const float (&m)[9]) {
+  constexpr float lo = 1e-15f, hi = 1e15f;
+  return sizeof(T) == 4 || (m[0] > lo && m[0] < hi && m[4] > lo && m[4] < hi);
+}
+
 __device__ __forceinline__ float tvb_sqrt(float x) {
   float r;
   asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
