@@ -893,7 +893,7 @@ void launch_amr_operator(const Ctx& c, const Tables<T>& tb, const T* w, T* fbuf,
   const size_t sm = (size_t)cell_list_warp_elems(g, std::min(am.maxent, kEntryChunk), vec) * WPB * sizeof(T);
   auto run = [&](auto face_k, auto cell_k) {
     face_k<<<(unsigned)((np + 127) / 128), 128, 0, st>>>(g, tb, am, w, fbuf, sc, (T)eps, qbuf);
-    cudaFuncSetAttribute(cell_k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    raise_smem(cell_k, 200 * 1024);
     cell_k<<<(unsigned)((g.ncell + WPB - 1) / WPB), 32 * WPB, sm, st>>>(g, tb, am, w, fbuf, out, w0, ca, cb, combine,
                                                                        sc, wmean, w0mean, outmean, qbuf);
   };

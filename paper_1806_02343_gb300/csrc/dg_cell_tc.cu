@@ -431,12 +431,7 @@ void build_tc_tables(const std::vector<double>& Pv, const std::vector<double>& d
 int launch_cell_tc(const float* tabs, const FastAll<float, 2>& ft, const FastGeom& g, const float* w, const float* F,
                    float* out, const float* w0, double ca, double cb, int combine, const DevScalars* sc,
                    const double* wmean, const double* w0mean, double* outmean, int nsm, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(k_cell_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess)
-      return -3;
-    attr = true;
-  }
+  raise_smem(k_cell_tc, SMEM_BYTES);
   TcScal ts;
   for (int l = 0; l < NM; ++l) ts.minv[l] = ft.cell.minv[l];
   for (int p = 0; p < QF; ++p) ts.wf[p] = ft.cell.Pfw[0][p][0];

@@ -167,6 +167,14 @@ struct LdfLeg {
   int ok;
 };
 
+// Dynamic shared memory that a launch of kernel fn takes beyond the 48 KB default.
+// The limit belongs to the current device, so it is set at each launch; where that
+// fails, so does the launch.
+template <typename K>
+inline void raise_smem(K* fn, size_t bytes) {
+  cudaFuncSetAttribute(reinterpret_cast<const void*>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 // Launch accounting: counts every kernel launch; with `on`, records a CUDA
 // event pair on the launch stream around each launch of a given kind.
 struct Prof {

@@ -1421,11 +1421,6 @@ __global__ void __launch_bounds__(NTD) k_divb_list_pow(const OctPow<T> o, const 
   }
 }
 
-template <typename T>
-void set_smem_attr(const void* fn, size_t bytes) {
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 }  // namespace
 
 template <typename T, int DEG>
@@ -1444,11 +1439,7 @@ void launch_face_glm(const FastAll<T, DEG>& tabs, const FastGeom& g, const T* w,
                      double eps, cudaStream_t st) {
   const unsigned nb = (unsigned)((g.ncell + TC - 1) / TC);
   const size_t sm = fast_face_smem<T, DEG>();
-  static bool attr = false;
-  if (!attr) {
-    set_smem_attr<T>((const void*)k_face_glm3<T, DEG>, sm);
-    attr = true;
-  }
+  raise_smem(k_face_glm3<T, DEG>, sm);
   k_face_glm3<T, DEG><<<nb, NT, sm, st>>>(tabs.face[0], tabs.face[1], tabs.face[2], g, w, F, sc, (T)eps);
 }
 
@@ -1458,11 +1449,7 @@ void launch_cell_glm(const FastAll<T, DEG>& tabs, const FastGeom& g, const T* w,
                      const double* w0mean, double* outmean, cudaStream_t st) {
   const unsigned nb = (unsigned)((g.ncell + TC - 1) / TC);
   const size_t sm = fast_cell_smem<T, DEG>();
-  static bool attr = false;
-  if (!attr) {
-    set_smem_attr<T>((const void*)k_cell_glm<T, DEG>, sm);
-    attr = true;
-  }
+  raise_smem(k_cell_glm<T, DEG>, sm);
   // cmode: 0 plain rhs, 1 SSP combination with ca == 0, 2 with ca != 0
   const int cmode = combine ? (ca != 0.0 ? 2 : 1) : 0;
   k_cell_glm<T, DEG><<<nb, NT, sm, st>>>(tabs.cell, g, w, F, out, w0, ca, cb, (float)ca, (float)cb, cmode, sc,
@@ -1484,11 +1471,7 @@ template <typename T, int DEG>
 void launch_face_pow(const FastAll<T, DEG>&, const FastGeom& g, const T* w, T* F, double eps, cudaStream_t st) {
   const unsigned nb = (unsigned)((g.ncell + TC - 1) / TC);
   const size_t sm = pow_face_smem<T, DEG>();
-  static bool attr = false;
-  if (!attr) {
-    set_smem_attr<T>((const void*)k_face_pow3<T, DEG>, sm);
-    attr = true;
-  }
+  raise_smem(k_face_pow3<T, DEG>, sm);
   k_face_pow3<T, DEG><<<nb, NT, sm, st>>>(g, w, F, (T)eps);
 }
 
@@ -1498,11 +1481,7 @@ void launch_cell_pow(const FastAll<T, DEG>&, const FastGeom& g, const T* w, cons
                      const double* w0mean, double* outmean, cudaStream_t st) {
   const unsigned nb = (unsigned)((g.ncell + TC - 1) / TC);
   const size_t sm = pow_cell_smem<T, DEG>();
-  static bool attr = false;
-  if (!attr) {
-    set_smem_attr<T>((const void*)k_cell_pow<T, DEG>, sm);
-    attr = true;
-  }
+  raise_smem(k_cell_pow<T, DEG>, sm);
   const int cmode = combine ? (ca != 0.0 ? 2 : 1) : 0;
   k_cell_pow<T, DEG><<<nb, NTP, sm, st>>>(g, w, F, out, w0, ca, cb, (float)ca, (float)cb, cmode, sc, wmean, w0mean,
                                           outmean);
@@ -1520,11 +1499,7 @@ void launch_face_list_pow(const OctPow<T>& o, double gamma, const T* w, T* F, do
   constexpr int N = FastDims<DEG>::N, QF = FastDims<DEG>::QF;
   constexpr int NDIV = PowDims<DEG>::NDIV, NRP = 5 * N + NDIV;
   const size_t smf = (size_t)(2 * N * list_pts<T, DEG>() + 2 * NRP * TC + 2 * QF * 8 * TC) * sizeof(T);
-  static bool attr = false;
-  if (!attr) {
-    set_smem_attr<T>((const void*)k_face_list_pow<T, DEG>, smf);
-    attr = true;
-  }
+  raise_smem(k_face_list_pow<T, DEG>, smf);
   if (o.nblk > 0) k_face_list_pow<T, DEG><<<(unsigned)o.nblk, NT, smf, st>>>(o, (T)gamma, (T)eps, w, F);
 }
 
@@ -1535,11 +1510,7 @@ void launch_cell_list_pow(const OctPow<T>& o, double gamma, const T* w, const T*
   constexpr int N = FastDims<DEG>::N, QF = FastDims<DEG>::QF, QC = FastDims<DEG>::QC;
   constexpr int NDIV = PowDims<DEG>::NDIV;
   const size_t smc = (size_t)(QC * NSL * TC + NDIV * TC + 8 * TC + 30 * QF * list_row<T, DEG>()) * sizeof(T);
-  static bool attr = false;
-  if (!attr) {
-    set_smem_attr<T>((const void*)k_cell_list_pow<T, DEG>, smc);
-    attr = true;
-  }
+  raise_smem(k_cell_list_pow<T, DEG>, smc);
   const int cmode = combine ? (ca != 0.0 ? 2 : 1) : 0;
   const unsigned nb = (unsigned)((o.ncell + TC - 1) / TC);
   k_cell_list_pow<T, DEG><<<nb, NTP, smc, st>>>(o, (T)gamma, w, F, out, w0, ca, cb, (float)ca, (float)cb, cmode, sc,

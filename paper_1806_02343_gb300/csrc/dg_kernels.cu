@@ -842,7 +842,7 @@ void launch_cell(const Geom& g, const Tables<T>& tb, const T* w, const T* fbuf, 
   const bool vec = sizeof(T) == 4 && pinned_sizes_ok(g) && tb.dPv4 && tb.dLv4 && tb.Pf4 && tb.Lf4;
   const size_t sm = cell_smem<T>(g, vec);
   auto run = [&](auto k) {
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    raise_smem(k, 200 * 1024);
     k<<<nblocks(g.ncell, WARPS_PER_BLOCK), 32 * WARPS_PER_BLOCK, sm, st>>>(g, tb, w, fbuf, out, w0, ca, cb, combine,
                                                                         sc, wmean, w0mean, outmean, qbuf);
   };

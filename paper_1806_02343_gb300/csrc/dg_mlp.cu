@@ -888,7 +888,7 @@ static void tile_launch(Ctx& c, const void* w, uint8_t* flag, float* prob, cudaS
                         int32_t* plist) {
   constexpr size_t sm = tile_smem<KP, GLM>();
   const auto k = k_mlp_tile<KP, GLM, DEG>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  raise_smem(k, sm);
   // persistent: the weights are staged once per block. At most four blocks per
   // SM: each holds 128 of the SM's 512 tensor-memory columns
   const int per_sm = DEG <= 2 ? 4 : 2;
@@ -918,11 +918,7 @@ static void infer_launch(Ctx& c, const void* w, const double* wmean, uint8_t* fl
   const Geom& g = c.g;
   const size_t sm = (size_t)HID * (KP + 8) * 2 + (size_t)HID * (HID + 8) * 2 + (size_t)4 * 32 * (KP + 8) * 2 +
                     (3 * HID + 1) * sizeof(float) + 128;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_mlp_infer<T, KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr = true;
-  }
+  raise_smem(k_mlp_infer<T, KP>, sm);
   // persistent grid: a few blocks per SM (the weights are staged once per block)
   const int64_t tiles = (g.ncell + 127) / 128;
   const unsigned nb = (unsigned)std::min<int64_t>(tiles, (int64_t)c.nsm * 4);

@@ -524,7 +524,7 @@ extern "C" int dg_mhd_amr_marks(dg_mhd_ctx* ctx, const void* w, const double* wm
     const size_t sm = (size_t)L.no * std::max(L.n, L.nd) * 32 * sizeof(double);  // 53 KB at degree 2, 102 KB at 3
     auto run = [&](auto k, auto* x) {
       // (one value for every context: the largest, 8 octants of 50 rows)
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * RG_MAXD * 32 * (int)sizeof(double));
+      raise_smem(k, 8 * RG_MAXD * 32 * sizeof(double));
       k<<<nbg, 32, sm, st>>>(c.g, L, x, wmean, field_mask, c.amr.groups, c.amr.ngroups, c.amr.lev_dev, s_tilde,
                              min_level, marks);
     };

@@ -484,18 +484,10 @@ __global__ void __launch_bounds__(NTS, 2) k_sf_cell(const FastGeom g, const V* _
 
 }  // namespace
 
-static void sf_attr(const void* fn, size_t bytes) {
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <int DEG, bool GLM>
 void launch_sf_face(const FastGeom& g, const double* w, double* F, const DevScalars* sc, double eps, cudaStream_t st) {
   using D = SfDims<DEG>;
-  static bool attr = false;
-  if (!attr) {
-    sf_attr((const void*)k_sf_face<DEG, GLM>, D::face_smem);
-    attr = true;
-  }
+  raise_smem(k_sf_face<DEG, GLM>, D::face_smem);
   k_sf_face<DEG, GLM><<<(unsigned)((g.ncell + 31) / 32), NTS, D::face_smem, st>>>(g, w, F, sc, eps);
 }
 
@@ -503,11 +495,7 @@ template <int DEG, bool GLM>
 void launch_sf_cell(const FastGeom& g, const double* w, const double* F, double* out, const double* w0, double ca,
                     double cb, int combine, const DevScalars* sc, cudaStream_t st) {
   using D = SfDims<DEG>;
-  static bool attr = false;
-  if (!attr) {
-    sf_attr((const void*)k_sf_cell<DEG, GLM>, D::cell_smem);
-    attr = true;
-  }
+  raise_smem(k_sf_cell<DEG, GLM>, D::cell_smem);
   const int cmode = combine ? (ca != 0.0 ? 2 : 1) : 0;
   k_sf_cell<DEG, GLM><<<(unsigned)((g.ncell + 31) / 32), NTS, D::cell_smem, st>>>(g, w, F, out, w0, ca, cb, cmode, sc);
 }

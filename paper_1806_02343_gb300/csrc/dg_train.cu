@@ -317,13 +317,7 @@ __global__ void __launch_bounds__(GO* GK) k_train_grad(Layer l1, Layer l2, Layer
 int gradient(const float* X, int ldx, const uint8_t* y, const int64_t* perm, int64_t off, int nb, int nin,
              const float* theta, float* grad, const Adam& a, double* loss, float pos_weight, float norm_n,
              void* scratch, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(k_train_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)) !=
-        cudaSuccess)
-      return -3;
-    attr = true;
-  }
+  raise_smem(k_train_pass, sizeof(TrainSmem));
   const Scratch sc(static_cast<float*>(scratch), nb, nin);
   const float inv_n = 1.f / norm_n;
   k_train_pass<<<std::min((nb + TB - 1) / TB, MAXBLK), NTT, sizeof(TrainSmem), st>>>(

@@ -50,3 +50,39 @@ def test_training_reads_every_epochs_own_shuffle(fake, tmp_path):
     assert all(np.array_equal(np.sort(p), np.arange(96)) for p in seen[0])
     assert len({p.tobytes() for p in seen[0]}) == 6
     assert np.array_equal(*seen)
+
+
+CONTEXTS = """
+fake = ctypes.CDLL(os.environ["LD_PRELOAD"])
+def rhs(divb, degree, **prm):
+    m, p, h = Bd.mesh_desc(3, (6, 5, 4)), Bd.default_params(c_h_fixed=1.0, **prm), vp()
+    assert lib.dg_mhd_init(ctypes.byref(m), degree, Bd.DG_DIVB_GLM if divb == "glm" else Bd.DG_DIVB_POWELL, 5 / 3,
+                           ctypes.byref(p), ctypes.byref(h)) == 0
+    r, k, c, s = (ctypes.c_int64() for _ in range(4))
+    lib.dg_mhd_state_layout(h, *(ctypes.byref(x) for x in (r, k, c, s)))
+    buf = [np.zeros(r.value * s.value) for _ in range(4)]
+    w, out, wm, om = (vp(b.ctypes.data) for b in buf)
+    e = lib.dg_mhd_rhs(h, w, wm, out, om, None)
+    if not e and prm.get("precision"):
+        nin = 8 * [1, 4, 10, 20][degree] + 30
+        th = np.zeros(64 * nin + 64 * 64 + 193, np.float32)
+        e = lib.dg_mhd_mlp_set_weights(h, vp(th.ctypes.data), nin, 0.5) or lib.dg_mhd_mlp_infer(h, w, wm, out, None, None)
+    lib.dg_mhd_destroy(h)
+    return e
+bad = []
+for device in (0, 1):
+    fake.fake_device(device)
+    if train():
+        bad.append((device, "train"))
+    for prec in (Bd.DG_PREC_FP64, Bd.DG_PREC_FP32MIX):
+        for divb, degree, gen in [("glm", d, 0) for d in (1, 2, 3)] + [("powell", d, 0) for d in (1, 2)] + [("glm", 2, 2)]:
+            if rhs(divb, degree, precision=prec, generic_kernels=gen):
+                bad.append((device, divb, degree, prec, gen))
+print(bad)
+assert not bad, bad
+"""
+
+
+def test_launches_work_on_every_device(fake):
+    """A kernel's shared-memory limit is set on the device that a call runs on, not once per process."""
+    _run(fake, TRAIN + CONTEXTS)
