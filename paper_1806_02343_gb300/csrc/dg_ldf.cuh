@@ -52,6 +52,13 @@ template <int DEG>
 constexpr bool ldf_has(int j, int c, int l) {
   return (LdfPattern<DEG>::m(j) >> (c * LdfPattern<DEG>::N + l)) & 1u;
 }
+// functions with the coefficient (c, l)
+template <int DEG>
+constexpr int ldf_terms(int c, int l) {
+  int n = 0;
+  for (int j = 0; j < LdfPattern<DEG>::NDIV; ++j) n += ldf_has<DEG>(j, c, l) ? 1 : 0;
+  return n;
+}
 // component c of function j is not identically zero
 template <int DEG>
 constexpr bool ldf_has(int j, int c) {

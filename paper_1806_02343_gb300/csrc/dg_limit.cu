@@ -422,24 +422,33 @@ __global__ void __launch_bounds__(128) k_tvb_detect(Geom gin, LdfLeg ll, const T
   const int64_t S = g.stride;
   const float gamma = (float)g.gamma;
   const float ch = GLMF ? sc->ch32 : 0.f;
-  // Legendre coefficient l of B component cc from the LDF rows of cell c (constant
-  // and linear ones: the entries are multiples of 1/2, exact in FP32), and the means,
-  // in the state's precision: sums and differences that cancel are rounded after it
-  auto ldf = [&](int64_t c, auto CC, auto L) {
-    T x = T(0);
-    sf::each<0, LdfPattern<DEG>::NDIV>([&](auto J) {
-      constexpr int j = decltype(J)::value, cc = decltype(CC)::value, l = decltype(L)::value;
-      if constexpr (ldf_has<DEG>(j, cc, l)) x = fma(w[(int64_t)(5 * N + j) * S + c], (T)ll.A[(j * 3 + cc) * N + l], x);
-    });
-    return x;
-  };
-  auto means = [&](int64_t c, T (&m)[9]) {
+  // Row k of the cell means: the variable's (Legendre), or (k >= 5) constant LDF row
+  // k - 5, whose function lies along one axis, with coefficient +-1
+  constexpr int NRAW = GLMF ? 9 : 8;
+  auto raw_row = [&](int k) { return GLMF || k < 5 ? k * N : 5 * N + k - 5; };
+  // the means' values (or differences) from those of the raw rows
+  auto physical = [&](const float (&raw)[9], float (&m)[9]) {
 #pragma unroll
-    for (int k = 0; k < NM; ++k)
-      if (GLMF || k < 5) m[k] = w[(int64_t)(k * N) * S + c];
-    if constexpr (!GLMF) {
-      sf::each<0, 3>([&](auto CC) { m[5 + decltype(CC)::value] = ldf(c, CC, std::integral_constant<int, 0>{}); });
-    }
+    for (int k = 0; k < 9; ++k) m[k] = k < (GLMF ? 9 : 5) ? raw[k] : 0.f;
+    if constexpr (!GLMF)
+      sf::each<0, 9>([&](auto I) {
+        constexpr int j = decltype(I)::value / 3, cc = decltype(I)::value % 3;
+        if constexpr (ldf_has<DEG>(j, cc, 0)) m[5 + cc] = raw[5 + j] * ll.A[(j * 3 + cc) * N];
+      });
+  };
+  // Legendre coefficient l of B component cc from the LDF rows of cell c. The entries
+  // are multiples of 1/2; a sum of rows, which may cancel, is formed in the state's
+  // precision and rounded after it.
+  auto ldf = [&](int64_t c, auto CC, auto L) -> float {
+    constexpr int cc = decltype(CC)::value, l = decltype(L)::value;
+    constexpr int terms = ldf_terms<DEG>(cc, l);
+    using R = std::conditional_t<terms == 1, float, T>;
+    R x = R(0);
+    sf::each<0, LdfPattern<DEG>::NDIV>([&](auto J) {
+      constexpr int j = decltype(J)::value;
+      if constexpr (ldf_has<DEG>(j, cc, l)) x = fma((R)w[(int64_t)(5 * N + j) * S + c], (R)ll.A[(j * 3 + cc) * N + l], x);
+    });
+    return (float)x;
   };
   // warp-uniform trip count (the appends below are warp ballots)
   for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < total; i0 += step) {
@@ -449,11 +458,10 @@ __global__ void __launch_bounds__(128) k_tvb_detect(Geom gin, LdfLeg ll, const T
     if (i < total) {
       c = list ? (int64_t)list[i] : i;
       const float thr = an.on ? (float)(mtilde * an.dxc[c]) : thr0;
-      T mt[9];
-      float m[9], sls[3][9];  // every load of the cell's own rows is issued before the first use
-      means(c, mt);
+      float own[9], m[9], sls[3][9];  // every load of the cell's own rows is issued before the first use
 #pragma unroll
-      for (int k = 0; k < 9; ++k) m[k] = k < NM ? (float)mt[k] : 0.f;
+      for (int k = 0; k < NRAW; ++k) own[k] = (float)w[(int64_t)raw_row(k) * S + c];
+      physical(own, m);
       sf::each<0, 3>([&](auto AX) {
         constexpr int A = decltype(AX)::value;
 #pragma unroll
@@ -461,7 +469,7 @@ __global__ void __launch_bounds__(128) k_tvb_detect(Geom gin, LdfLeg ll, const T
           if (GLMF || v < 5) sls[A][v] = (float)w[(int64_t)(v * N + 1 + A) * S + c];
         if constexpr (!GLMF) {
           sf::each<0, 3>([&](auto CC) {
-            sls[A][5 + decltype(CC)::value] = (float)ldf(c, CC, std::integral_constant<int, 1 + A>{});
+            sls[A][5 + decltype(CC)::value] = ldf(c, CC, std::integral_constant<int, 1 + A>{});
           });
           sls[A][8] = 0.f;
         }
@@ -471,34 +479,33 @@ __global__ void __launch_bounds__(128) k_tvb_detect(Geom gin, LdfLeg ll, const T
       sf::each<0, 3>([&](auto AX) {
         constexpr int A = decltype(AX)::value;
         if (!clear) return;
-        clear = tvb_axis_clear<A, GLMF>(m, sls[A], gamma, ch, thr, beta, kTvbWide<T>, [&](float (&dp)[9], float (&dm)[9]) {
+        clear = tvb_axis_clear<T, A, GLMF>(m, sls[A], gamma, ch, thr, beta, [&](float (&dp)[9], float (&dm)[9]) {
 #pragma unroll
           for (int sd = 0; sd < 2; ++sd) {
-            T mn[9];
-            float f = 0.5f;
+            float r[9], f = 0.5f;
             if (!an.on) {
-              means(nb(g, c, A, sd ? 1 : -1), mn);
+              const int64_t n = nb(g, c, A, sd ? 1 : -1);
+#pragma unroll
+              for (int k = 0; k < NRAW; ++k) r[k] = (float)w[(int64_t)raw_row(k) * S + n];
             } else {  // the average of the leaves across the side, the centre distance 2, 1.5 or 3
               const int sidx = 2 * A + sd, inf = an.side_info[c * 6 + sidx];
               const int cnt = inf & 15, rel = inf >> 4;
+              T x[9];
 #pragma unroll
-              for (int k = 0; k < 9; ++k) mn[k] = T(0);
+              for (int k = 0; k < NRAW; ++k) x[k] = T(0);
               for (int q = 0; q < cnt; ++q) {
-                T t[9];
-                means((int64_t)an.side_nb[c * 24 + sidx * 4 + q], t);
+                const int64_t n = an.side_nb[c * 24 + sidx * 4 + q];
 #pragma unroll
-                for (int k = 0; k < NM; ++k) mn[k] += t[k];
+                for (int k = 0; k < NRAW; ++k) x[k] += w[(int64_t)raw_row(k) * S + n];
               }
               const T ic = T(1) / (T)(cnt > 0 ? cnt : 1);
 #pragma unroll
-              for (int k = 0; k < NM; ++k) mn[k] *= ic;
+              for (int k = 0; k < NRAW; ++k) r[k] = (float)(x[k] * ic);
               if (cnt > 0) f = rel == 0 ? 0.5f : (rel == 1 ? 1.f / 1.5f : 1.f / 3.f);
             }
 #pragma unroll
-            for (int k = 0; k < 9; ++k) {
-              const float d = k < NM ? (float)(sd ? mn[k] - mt[k] : mt[k] - mn[k]) * f : 0.f;
-              (sd ? dp[k] : dm[k]) = d;
-            }
+            for (int k = 0; k < NRAW; ++k) r[k] = (sd ? r[k] - own[k] : own[k] - r[k]) * f;
+            physical(r, sd ? dp : dm);
           }
         });
       });

@@ -92,20 +92,27 @@ __device__ __forceinline__ void tvb_eig(const float (&m)[9], float gamma, float 
   e.sgn = e.B[A] >= 0.f ? 1.f : -1.f;
 }
 
-// amplitudes of a conserved increment with their bounds and errors
-template <int A, int GLMF>
-__device__ __forceinline__ void tvb_amp(const TvbEig<GLMF>& e, const float (&d)[9], TvbAmp<GLMF>& o) {
+// amplitudes of a conserved increment with their bounds and errors. CAST: the
+// increment is a difference of means m rounded to FP32 beforehand (FP64 states),
+// off by up to 1.2e-7 |m| more. (FP64 differences rounded afterwards need no such
+// term, but their FP64 operations made a pass 13.6 -> 19.0 us on 21^3 cells; with
+// the term 16.0 us.)
+template <int A, bool CAST, int GLMF>
+__device__ __forceinline__ void tvb_amp(const TvbEig<GLMF>& e, const float (&d)[9], const float (&m)[9],
+                                        TvbAmp<GLMF>& o) {
   constexpr int T1 = (A + 1) % 3, T2 = (A + 2) % 3;
+  // the magnitudes that kTvbRound applies to
+  auto s = [&](int k) { return CAST ? fmaf(1.5e-7f / kTvbRound, fabsf(m[k]), fabsf(d[k])) : fabsf(d[k]); };
   const float dr = d[0], du = (d[1 + A] - e.v[A] * dr) * e.ir, dv = (d[1 + T1] - e.v[T1] * dr) * e.ir,
               dw = (d[1 + T2] - e.v[T2] * dr) * e.ir;
   const float ke = 0.5f * (e.v[0] * e.v[0] + e.v[1] * e.v[1] + e.v[2] * e.v[2]);
-  float dp = ke * dr + d[4], sp = ke * fabsf(dr) + fabsf(d[4]);
-  float su = (fabsf(d[1 + A]) + fabsf(e.v[A] * dr)) * e.ir, st = 0.f;
+  float dp = ke * dr + d[4], sp = ke * s(0) + s(4);
+  float su = (s(1 + A) + fabsf(e.v[A]) * s(0)) * e.ir, st = 0.f;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     dp -= e.v[i] * d[1 + i] + e.B[i] * d[5 + i];
-    sp += fabsf(e.v[i] * d[1 + i]) + fabsf(e.B[i] * d[5 + i]);
-    if (i != A) st += (fabsf(d[1 + i]) + fabsf(e.v[i] * dr)) * e.ir;
+    sp += fabsf(e.v[i]) * s(1 + i) + fabsf(e.B[i]) * s(5 + i);
+    if (i != A) st += (s(1 + i) + fabsf(e.v[i]) * s(0)) * e.ir;
   }
   dp *= e.gm1;
   sp *= e.gm1;
@@ -122,45 +129,45 @@ __device__ __forceinline__ void tvb_amp(const TvbEig<GLMF>& e, const float (&d)[
   o.c[1] = 0.5f * (vperp + e.sgn * bperp * e.isr);
   o.c[5] = 0.5f * (vperp - e.sgn * bperp * e.isr);
   o.c[3] = dr - dp * e.a2i;
-  const float nv = fabsf(dv) + fabsf(dw), nb = fabsf(dby) + fabsf(dbz);
+  const float nv = fabsf(dv) + fabsf(dw), nb = fabsf(dby) + fabsf(dbz), sb = s(5 + T1) + s(5 + T2);
   const float wf = h * e.cf * (fabsf(du) + nv) + 0.5f * (fabsf(dp) * e.ir * e.a2i + nb * e.isra);
-  const float rf = h * e.cf * (su + st) + 0.5f * (sp * e.ir * e.a2i + nb * e.isra);
+  const float rf = h * e.cf * (su + st) + 0.5f * (sp * e.ir * e.a2i + sb * e.isra);
   const float ef = kTvbWeight * wf + kTvbRound * rf;
 #pragma unroll
   for (int k = 0; k < 7; k += 2) {
     o.b[k] = e.wmax * wf + ef;
     o.e[k] = ef;
   }
-  const float wa = 0.5f * (nv + nb * e.isr), ea = kTvbWeight * wa + kTvbRound * 0.5f * st;
+  const float wa = 0.5f * (nv + nb * e.isr), ea = kTvbWeight * wa + kTvbRound * 0.5f * (CAST ? st + sb * e.isr : st);
   o.b[1] = o.b[5] = wa + ea;
   o.e[1] = o.e[5] = ea;
   // the entropy wave has no weights: rounding, and a^2's own error (3e-3 at the limit of `sane`)
-  o.e[3] = kTvbRound * (fabsf(dr) + sp * e.a2i) + 5e-3f * fabsf(dp) * e.a2i;
+  o.e[3] = kTvbRound * (s(0) + sp * e.a2i) + 5e-3f * fabsf(dp) * e.a2i;
   o.b[3] = fabsf(o.c[3]) + o.e[3];
   if constexpr (GLMF) {
     o.c[7] = 0.5f * (d[5 + A] - d[8] * e.ich);
     o.c[8] = 0.5f * (d[5 + A] + d[8] * e.ich);
-    o.e[7] = o.e[8] = kTvbRound * (fabsf(d[5 + A]) + fabsf(d[8] * e.ich));
+    o.e[7] = o.e[8] = kTvbRound * (s(5 + A) + s(8) * fabsf(e.ich));
     o.b[7] = fabsf(o.c[7]) + o.e[7];
     o.b[8] = fabsf(o.c[8]) + o.e[8];
   } else {
     o.c[7] = d[5 + A];
-    o.e[7] = kTvbRound * fabsf(d[5 + A]);
+    o.e[7] = kTvbRound * s(5 + A);
     o.b[7] = fabsf(o.c[7]) + o.e[7];
   }
 }
 
 // Axis A cannot trigger: every amplitude of the slopes `sl` stays below thr, or
 // both neighbour differences (dp, dm: loaded by `diffs` where needed) clear it.
-// wide: kTvbWide of the procedure's precision.
-template <int A, int GLMF, typename Diffs>
+// T: the procedure's precision.
+template <typename T, int A, int GLMF, typename Diffs>
 __device__ __forceinline__ bool tvb_axis_clear(const float (&m)[9], const float (&sl)[9], float gamma, float ch,
-                                               float thr, float beta, float wide, Diffs diffs) {
+                                               float thr, float beta, Diffs diffs) {
   TvbEig<GLMF> e;
-  tvb_eig<A>(m, gamma, ch, wide, e);
+  tvb_eig<A>(m, gamma, ch, kTvbWide<T>, e);
   if (!e.sane) return false;
   TvbAmp<GLMF> x;
-  tvb_amp<A>(e, sl, x);
+  tvb_amp<A, false>(e, sl, m, x);
   constexpr int V = GLMF ? 9 : 8;
   bool below = true;
 #pragma unroll
@@ -174,8 +181,8 @@ __device__ __forceinline__ bool tvb_axis_clear(const float (&m)[9], const float 
   float dpl[9], dmi[9];
   diffs(dpl, dmi);
   TvbAmp<GLMF> p, q;
-  tvb_amp<A>(e, dpl, p);
-  tvb_amp<A>(e, dmi, q);
+  tvb_amp<A, sizeof(T) == 8>(e, dpl, m, p);
+  tvb_amp<A, sizeof(T) == 8>(e, dmi, m, q);
   bool ok = true;
 #pragma unroll
   for (int k = 0; k < V; ++k) {
