@@ -33,6 +33,10 @@ constexpr int KC = 128;       // inputs per pass over W1 and X
 constexpr int WS = HID + 2;   // row stride of the transposed weights
 constexpr int MAXBLK = 304;   // blocks of the passes at most: two per SM
 constexpr int GO = 4, GK = 16, GS = 256;  // a gradient block: GO x GK weights, chunks of GS samples
+// samples per pair of launches: more than a mini-batch has, so that one pair is the
+// rule; a gradient of more samples keeps scratch for this many (0.4 GB at 110 inputs)
+// and its sums go on from pair to pair
+constexpr int PART = 1 << 18;
 
 struct TrainSmem {
   float w1t[KC][WS];    // W1 transposed, the current inputs
@@ -226,8 +230,8 @@ struct Layer {
   int nout, K, w, b;   // outputs, inputs, and where the weights and the biases lie in theta
 };
 
-__device__ __forceinline__ void layer_grad(const Layer& L, int patch, int nb, int ld, float* __restrict__ grad,
-                                           const Adam& a) {
+__device__ __forceinline__ void layer_grad(const Layer& L, int patch, int nb, int ld, bool go_on,
+                                           float* __restrict__ grad, const Adam& a) {
   constexpr int NT = GO * GK, Q = GS / 4, N = (GO + GK) * Q / NT;  // 16-byte words per thread and chunk
   static_assert((GO * Q) % NT == 0 && (GK * Q) % NT == 0, "whole words per thread");
   __shared__ __align__(16) float T[GO + GK][GS + 4];
@@ -246,6 +250,8 @@ __device__ __forceinline__ void layer_grad(const Layer& L, int patch, int nb, in
     }
   };
   float g = 0.f;
+  const int o = o0 + oo, k = k0 + kk;
+  if (go_on && o < L.nout && k <= L.K) g = grad[k == L.K ? L.b + o : L.w + o * L.K + k];
   fetch(0);
   for (int b0 = 0; b0 < nb; b0 += GS) {
     __syncthreads();
@@ -274,7 +280,6 @@ __device__ __forceinline__ void layer_grad(const Layer& L, int patch, int nb, in
       g = __fadd_rn(g, __fmul_rn(d.w, x.w));
     }
   }
-  const int o = o0 + oo, k = k0 + kk;
   if (o >= L.nout || k > L.K) return;
   const int i = k == L.K ? L.b + o : L.w + o * L.K + k;
   if (!a.th) {
@@ -288,16 +293,17 @@ __device__ __forceinline__ void layer_grad(const Layer& L, int patch, int nb, in
   a.th[i] -= a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
 }
 
-// Patches of the three layers, then (loss) blocks of 64 samples
+// Patches of the three layers, then (loss) blocks of 64 samples. go_on: the sums of
+// the samples before these are in `grad`.
 __global__ void __launch_bounds__(GO* GK) k_train_grad(Layer l1, Layer l2, Layer l3, int n1, int n2, int n3,
                                                        const int64_t* __restrict__ perm, int64_t off, int nb, int ld,
-                                                       float* __restrict__ grad, Adam a,
+                                                       bool go_on, float* __restrict__ grad, Adam a,
                                                        const float* __restrict__ prob, const uint8_t* __restrict__ y,
                                                        float pos_weight, float inv_n, double* __restrict__ loss) {
   const int b = blockIdx.x;
   if (b < n1 + n2 + n3) {
     const Layer L = b < n1 ? l1 : b < n1 + n2 ? l2 : l3;
-    layer_grad(L, b < n1 ? b : b < n1 + n2 ? b - n1 : b - n1 - n2, nb, ld, grad, a);
+    layer_grad(L, b < n1 ? b : b < n1 + n2 ? b - n1 : b - n1 - n2, nb, ld, go_on, grad, a);
     return;
   }
   const int s = (b - n1 - n2 - n3) * GO * GK + threadIdx.x;
@@ -312,29 +318,32 @@ __global__ void __launch_bounds__(GO* GK) k_train_grad(Layer l1, Layer l2, Layer
   if ((threadIdx.x & 31) == 0) atomicAdd(loss, l);
 }
 
-// loss (nullable) += the mean weighted loss of the nb samples; the gradient
-// into grad, or an Adam step
+// loss (nullable) += the mean weighted loss of the nb samples; the gradient into
+// grad, or an Adam step (grad: the sums, where nb > PART)
 int gradient(const float* X, int ldx, const uint8_t* y, const int64_t* perm, int64_t off, int nb, int nin,
              const float* theta, float* grad, const Adam& a, double* loss, float pos_weight, float norm_n,
              void* scratch, cudaStream_t st) {
   raise_smem(k_train_pass, sizeof(TrainSmem));
-  const Scratch sc(static_cast<float*>(scratch), nb, nin);
+  const Scratch sc(static_cast<float*>(scratch), std::min(nb, PART), nin);
   const float inv_n = 1.f / norm_n;
-  k_train_pass<<<std::min((nb + TB - 1) / TB, MAXBLK), NTT, sizeof(TrainSmem), st>>>(
-      X, ldx, y, perm, off, nb, nin, theta, pos_weight, inv_n, sc, loss != nullptr);
   const int w2 = HID * nin + HID, w3 = w2 + HID * HID + HID;
   const Layer l1{sc.d1, sc.x, HID, nin, 0, HID * nin}, l2{sc.d2, sc.h1, HID, HID, w2, w2 + HID * HID},
       l3{sc.d3, sc.h2, 1, HID, w3, w3 + HID};
   auto patches = [](const Layer& L) { return (L.nout + GO - 1) / GO * ((L.K + GK) / GK); };
-  const int n1 = patches(l1), n2 = patches(l2), n3 = patches(l3), nl = loss ? (nb + GO * GK - 1) / (GO * GK) : 0;
-  k_train_grad<<<n1 + n2 + n3 + nl, GO * GK, 0, st>>>(l1, l2, l3, n1, n2, n3, perm, off, nb, sc.ld, grad, a, sc.prob,
-                                                      y, pos_weight, inv_n, loss);
+  const int n1 = patches(l1), n2 = patches(l2), n3 = patches(l3);
+  for (int b = 0; b < nb; b += PART) {
+    const int n = std::min(PART, nb - b), nl = loss ? (n + GO * GK - 1) / (GO * GK) : 0;
+    k_train_pass<<<std::min((n + TB - 1) / TB, MAXBLK), NTT, sizeof(TrainSmem), st>>>(
+        X, ldx, y, perm, off + b, n, nin, theta, pos_weight, inv_n, sc, loss != nullptr);
+    k_train_grad<<<n1 + n2 + n3 + nl, GO * GK, 0, st>>>(l1, l2, l3, n1, n2, n3, perm, off + b, n, sc.ld, b > 0, grad,
+                                                        n == nb - b ? a : Adam{}, sc.prob, y, pos_weight, inv_n, loss);
+  }
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace
 
-size_t mlp_scratch_bytes(int nb, int nin) { return Scratch::floats(nb, nin) * sizeof(float); }
+size_t mlp_scratch_bytes(int nb, int nin) { return Scratch::floats(std::min(nb, PART), nin) * sizeof(float); }
 
 int mlp_loss_grad_dev(const float* X, int ldx, const uint8_t* y, int nb, int nin, const float* theta, float* grad,
                       double* loss, float pos_weight, void* scratch, cudaStream_t st) {
@@ -344,8 +353,8 @@ int mlp_loss_grad_dev(const float* X, int ldx, const uint8_t* y, int nb, int nin
 int mlp_train_dev(const float* X, int ldx, const uint8_t* y, int64_t n, int nin, float* theta, int epochs,
                   int batch, float lr, float pos_weight, uint64_t seed, double* last_loss, cudaStream_t st) {
   const int np = mlp_n_params(nin);
-  // one allocation: scratch (16-byte rows first), shuffle, loss, Adam moments
-  const size_t bytes = n * sizeof(int64_t) + sizeof(double) + 2 * (size_t)np * sizeof(float) +
+  // one allocation: scratch (16-byte rows first), shuffle, loss, Adam moments, gradient sums
+  const size_t bytes = n * sizeof(int64_t) + sizeof(double) + 3 * (size_t)np * sizeof(float) +
                        (mlp_scratch_bytes(batch, nin) + 7) / 8 * 8;
   unsigned char* mem = nullptr;
   if (cudaMalloc(&mem, bytes) != cudaSuccess) return -3;
@@ -353,7 +362,7 @@ int mlp_train_dev(const float* X, int ldx, const uint8_t* y, int64_t n, int nin,
   int64_t* perm = reinterpret_cast<int64_t*>(mem + (mlp_scratch_bytes(batch, nin) + 7) / 8 * 8);
   double* dloss = reinterpret_cast<double*>(perm + n);
   float* m = reinterpret_cast<float*>(dloss + 1);
-  float* v = m + np;
+  float *v = m + np, *sums = v + np;
   int e = 0;
   if (cudaMemsetAsync(m, 0, 2 * (size_t)np * sizeof(float), st) != cudaSuccess) e = -3;
   cudaEvent_t copied = nullptr;  // behind the last copy of the shuffle
@@ -379,8 +388,8 @@ int mlp_train_dev(const float* X, int ldx, const uint8_t* y, int64_t n, int nin,
     for (int64_t off = 0; off + batch <= n && !e; off += batch) {
       ++t;
       const float c1 = 1.f - powf(0.9f, (float)t), c2 = 1.f - powf(0.999f, (float)t);
-      e = gradient(X, ldx, y, perm, off, batch, nin, theta, nullptr, Adam{theta, m, v, lr, 0.9f, 0.999f, 1e-8f, c1, c2}, loss, pos_weight,
-                   (float)batch, scratch, st);
+      e = gradient(X, ldx, y, perm, off, batch, nin, theta, sums, Adam{theta, m, v, lr, 0.9f, 0.999f, 1e-8f, c1, c2},
+                   loss, pos_weight, (float)batch, scratch, st);
     }
   }
   if (cudaStreamSynchronize(st) != cudaSuccess) e = -3;

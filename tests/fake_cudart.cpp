@@ -5,7 +5,8 @@
 //   the work queued before them, when something waits for them (FAKE_DEFER=1), or
 //   at the call, as from a staging buffer. Their bytes go to the file FAKE_LOG;
 // * the shared-memory limit of a kernel is 48 KB until it is raised, on the
-//   device that is current (fake_device); a launch above it is an error.
+//   device that is current (fake_device); a launch above it is an error;
+// * with FAKE_MEMORY the device holds that many bytes.
 #include <cstdint>
 #include <cstdio>
 #include <cstdlib>
@@ -25,6 +26,8 @@ std::deque<Op> queue;
 uint64_t queued = 0, done = 0;
 int device = 0, last_error = 0;
 std::map<std::pair<int, const void*>, size_t> limit;
+std::map<void*, size_t> sizes;
+size_t held = 0;
 struct Dim3 {
   unsigned x, y, z;
 };
@@ -61,9 +64,16 @@ void fake_device(int d) { device = d; }
 int cudaGetDevice(int* d) { return *d = device, 0; }
 int cudaDeviceGetAttribute(int* v, int, int) { return *v = 152, 0; }
 int cudaGetLastError() { return std::exchange(last_error, 0); }
-int cudaMalloc(void** p, size_t n) { return (*p = std::calloc(n ? n : 1, 1)) ? 0 : 2; }
+int cudaMalloc(void** p, size_t n) {
+  static const size_t all = std::getenv("FAKE_MEMORY") ? std::strtoull(std::getenv("FAKE_MEMORY"), nullptr, 10) : ~0ull;
+  if (n > all - held || !(*p = std::calloc(n ? n : 1, 1))) return 2;
+  held += sizes[*p] = n;
+  return 0;
+}
 int cudaFree(void* p) {
   run_to(queued);
+  held -= sizes[p];
+  sizes.erase(p);
   std::free(p);
   return 0;
 }

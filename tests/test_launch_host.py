@@ -86,3 +86,17 @@ assert not bad, bad
 def test_launches_work_on_every_device(fake):
     """A kernel's shared-memory limit is set on the device that a call runs on, not once per process."""
     _run(fake, TRAIN + CONTEXTS)
+
+
+GRADIENT = """
+n, nin = 1 << 21, 110
+X, y, th = np.zeros((n, nin), np.float32), np.zeros(n, np.uint8), np.zeros(64 * nin + 64 * 64 + 193, np.float32)
+grad, p = np.zeros_like(th), lambda a: vp(a.ctypes.data)
+assert lib.dg_mhd_mlp_loss_grad(p(X), nin, p(y), n, nin, p(th), 1.0, p(grad), None, None) == 0
+assert train(n=n, nin=nin, epochs=1, batch=n) == 0
+"""
+
+
+def test_gradients_of_many_samples_fit_beside_them(fake):
+    """Two million samples (0.9 GB of inputs) with 2.2 GB left on the device: four activation rows of each fit."""
+    _run(fake, TRAIN + GRADIENT, FAKE_MEMORY=str(2200 << 20))
