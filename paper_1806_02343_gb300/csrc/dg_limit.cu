@@ -407,8 +407,8 @@ __device__ bool tvb_cell(const Geom& g, const LimTabs& lt, T* w, const double* w
 // slopes; the neighbours' means are read for the rest. The procedure on every
 // cell, one thread each with its arrays in local memory, was latency-bound. Per
 // pass, before and now with the procedure on the list: 1,387,520-leaf octree 0.83
-// and 0.06 ms; 48^3 FP64 blast 0.67 and 0.18 ms; 256^3 turbulence, the indicator's
-// list, 0.69 and 0.59 ms.
+// and 0.06 ms; 48^3 FP64 blast 0.67 and 0.19 ms; 256^3 turbulence, the indicator's
+// list, 0.69 and 0.57 ms.
 template <typename T, bool SCREEN, int DEG, int GLMF>
 __global__ void __launch_bounds__(128) k_tvb_detect(Geom gin, LdfLeg ll, const T* __restrict__ w, float thr0,
                                                     double mtilde, float beta, DevScalars* sc, AmrNb an,
@@ -1028,9 +1028,10 @@ __global__ void k_pos(Geom g, Tables<T> tb, LimTabs lt, T* w, double* wmean, dg_
 // What bounded it: every open cell cost its warp about 45 FP64 instructions
 // (conversions and warp minima, 16 cycles of the SM each) although hardly any
 // needs its FP64 pressures -- 86% of the cells of a Mach-1.5 flow are listed and
-// none limited -- and the lists of a blast filled only 131 warps. Measured per
-// pass: flow, 436,000 of 504,000 cells listed, 1.69 ms; 256^3 turbulence,
-// 415,000 listed, 1.60 ms; 128^3 Powell blast, 4,000 listed, 0.69 ms.
+// none limited -- and the lists of a blast filled only 131 warps. Per pass, before
+// and now: flow, 436,000 of 504,000 cells listed, 1.69 and 0.095 ms; 256^3
+// turbulence, 415,000 listed, 1.60 and 0.13 ms; 128^3 Powell blast, 4,000 listed,
+// 0.69 and 0.14 ms.
 template <int DEG, int GLMF>
 __global__ void __launch_bounds__(128) k_pos_list(Geom gin, Tables<float> tb, PosScreen ps, LdfLeg ll, float* w,
                                                   double* wmean, dg_mhd_params p, DevScalars* sc,

@@ -223,7 +223,7 @@ __device__ __forceinline__ void face_coefs(const V* c, bool plus, V* g) {
 // ------------------------------------------------------------------ face flux
 // HLLD flux of the rotated conserved traces u = (rho, m_n, m_t1, m_t2, E, B_n,
 // B_t1, B_t2) (Miyoshi & Kusano 2005; the solver of Sec. 4.1.2), the scheme of
-// dg_phys.cuh's `face_flux` with fewer FP64 operations (about 345 per point
+// dg_phys.cuh's `face_flux` with fewer FP64 operations (about 340 per point
 // against 490; every division and square root costs about nine):
 // * one division for 1 / rho of both sides and one for the four star-state
 //   denominators (products of the operands: they stay in range for densities

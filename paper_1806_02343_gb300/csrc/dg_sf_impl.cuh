@@ -7,8 +7,8 @@
 // sparse map of dg_ldf.cuh; the ninth warp works on points only.
 // Both kernels are bound by the FP64 pipe (2 operations per clock and SM).
 // Measured on GB300, smooth GLM state, 45 x 40 x 36 cells, degree 2, per
-// evaluation: face + cell 2.22 + 1.66 ms with dense contractions, 1.25 + 0.56
-// now; Powell blast, 48^3 cells: 3.88 + 3.27 ms, 2.02 + 0.93 now.
+// evaluation: face + cell 2.22 + 1.66 ms with dense contractions, 1.23 + 0.56
+// now; Powell blast, 48^3 cells: 3.88 + 3.27 ms, 1.98 + 0.93 now.
 #include <type_traits>
 
 #include "dg_fast.cuh"
